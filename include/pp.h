@@ -267,9 +267,13 @@ PP_API pp_status pp_relax_scan(const float* ff, const pp_grid* grid, const pp_sc
  *          runs the scan again on the complete grid).
  *   plan   DEVICE pixel-to-warp plan from pp_relax_plan for a scan of the same
  *          nx and ny, built with plan_k and plan_lanes, or NULL: the plan's
- *          pixels run in warps of plan_lanes lanes ahead of the 8x4 pixel
+ *          pixels run in warps of plan_lanes lanes ahead of the pixel
  *          tiles, which skip them.  A stale plan (another image's) costs time,
- *          never correctness. */
+ *          never correctness.
+ *   plan_lanes without a plan: at most that many pixels to a warp, 1..32 (the
+ *          next power of two below; anything else: the library chooses, narrow
+ *          warps for scans too small to fill the GPU).  32 suits scans that
+ *          share the GPU with others in flight. */
 typedef struct {
     int* zspan;
     const int* plan;

@@ -39,7 +39,7 @@ class Simulator:
         0.025 on a force grid and 0 on a tricubic energy grid, whose scan is bound by issue slots rather
         than by its slowest tile (flake60 at 0.2 A: 1.42 ms on its own plan against 1.31 without).
         auto_plan: every scan builds the plan for the next from its own iteration counts.
-        plan_min_tiles: scans of fewer 8x4 pixel tiles get no plan (None: the GPU's SM count)."""
+        plan_min_tiles: scans of fewer 8x4 pixel tiles get no plan (None: eight per SM)."""
         self.case = case
         self.device = torch.device(device)
         if tuning is not None:
@@ -89,6 +89,7 @@ class Simulator:
         self._plan_k = 0       # k and lanes the held plan was built with
         self._plan_lanes = 0
         self._plan_ready = False
+        self.scan_lanes = 0    # pixels per warp of scans without a plan (0: the library's choice)
 
     def make_ff(self, atoms_dev, stream=None):
         if self.zpt is not None:
@@ -104,7 +105,7 @@ class Simulator:
         plan = (self._plan, self._plan_k, self._plan_lanes) if self._plan_ready else None
         pp.pp_relax_scan(self.ff, self.grid, self.scan, self.tip, self.fire, self.pos, self.fz, self.iters,
                          self.dfp if self.fused_df else None, out if self.fused_df else None, stream,
-                         zspan=zspan, plan=plan)
+                         zspan=zspan, plan=plan, lanes=self.scan_lanes)
         if not self.fused_df:
             pp.pp_fz_to_df(self.fz, self.scan.nz, self.scan.nx * self.scan.ny, self.scan.dz, self.dfp, out, stream)
         if self.auto_plan and self.iters is not None:
@@ -120,10 +121,11 @@ class Simulator:
         tiles = ((self.scan.nx + 7) // 8) * ((self.scan.ny + 3) // 4)
         least = self.plan_min_tiles
         if least is None:
-            least = torch.cuda.get_device_properties(self.device).multi_processor_count
+            least = 8 * torch.cuda.get_device_properties(self.device).multi_processor_count
         if tiles < least:
-            # fewer 8x4 tiles than SMs: no tile shares an SM, and building the plan costs more than it
-            # saves (benzene, 50 tiles: 0.163 against 0.149 ms per forward pass)
+            # smaller scans run narrow warps throughout or leave issue slots free; building the plan then
+            # costs more than it saves (181x181 px, 1058 tiles: 0.236 ms with its own plan and its build
+            # against 0.215 without; 128x128: 0.201 against 0.199; 256x256, 2048 tiles: 0.549 against 0.609)
             return
         npix = self.scan.nx * self.scan.ny
         k = max(1, min(npix, int(round(self.plan_frac * npix))))
@@ -394,6 +396,11 @@ class Pipeline:
         sim_kwargs.setdefault("plan_frac", 0.0)
         self.sims = [Simulator(case, **sim_kwargs) for _ in range(slots)]
         self.streams = [torch.cuda.Stream() for _ in range(slots)]
+        if slots > 1:
+            # full warps: the narrow ones a small scan takes by itself spend the issue slots that the
+            # other items' scans need (96x96 px, 4 slots: 0.101 ms per item at 32 pixels to a warp, 0.129 at 8)
+            for sim in self.sims:
+                sim.scan_lanes = 32
         self._host = None
 
     @property

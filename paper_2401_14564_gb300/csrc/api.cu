@@ -370,6 +370,7 @@ static pp_status relax_scan_impl(const char* name, const float* ff, const pp_gri
         df_stencil(fused_df->A_pp, scan->dz, fused_df->k, fused_df->f0, m, L.coef);
     }
     L.zspan = zspan;
+    if (opts && !opts->plan && opts->plan_lanes >= 1 && opts->plan_lanes <= 32) L.tile_lanes = opts->plan_lanes;
     if (opts && opts->plan) {
         const int npix = scan->nx * scan->ny;
         const int* plan = static_cast<const int*>(opts->plan);

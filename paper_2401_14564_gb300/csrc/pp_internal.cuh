@@ -164,6 +164,8 @@ struct RelaxLaunch {
     const int* plan_list;
     const unsigned* plan_mask;
     int plan_hblocks, plan_lanes;
+    int tile_lanes;          // pixels per tile warp asked for (1..32), 0: the launcher's choice
+    int tile_wsh, tile_hsh;  // log2 of the pixel tile of a warp along x and y (set by the launcher)
     float coef[2 * kMaxDfHalfWidth + 1];
 };
 cudaError_t launch_relax_scan(const RelaxLaunch& L, cudaStream_t s);

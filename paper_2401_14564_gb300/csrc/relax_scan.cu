@@ -13,7 +13,8 @@
 // relative precision however stiff the spring (with d itself the extension
 // would be quantised at ulp(R0) ~ 5e-7 A, i.e. 3e-4 eV/A at 1e4 N/m).
 //
-// Lanes of a warp cover an 8x4 pixel tile, so the 32 PPs sit in neighbouring
+// Lanes of a warp cover an 8x4 pixel tile (a smaller one in scans too small to
+// fill the GPU, see tile_shape), so the 32 PPs sit in neighbouring
 // grid cells and their corner loads share L1 lines.  Each lane advances to its
 // next height as soon as it has converged; the warp only waits for its
 // slowest lane once, at the end of the columns, not at every height.
@@ -25,9 +26,7 @@
 namespace pp {
 namespace {
 
-constexpr int kThreads = 32;  // one warp per CTA: an 8x4 pixel tile (evens out warps per SM)
-constexpr int kTileX = 8;
-constexpr int kTileY = 4;
+constexpr int kThreads = 32;  // one warp per CTA: one pixel tile (evens out warps per SM)
 
 // Node range [lo, hi] (clamped to the grid) covering coordinates a..b along one axis.
 __device__ __forceinline__ int2 node_range(float a, float b, float inv_d, float g0s, int n) {
@@ -37,7 +36,7 @@ __device__ __forceinline__ int2 node_range(float a, float b, float inv_d, float 
     return make_int2(lo, hi);
 }
 
-// Linear layout: ask L2 for the grid rows under this warp's 8x4 tile over the
+// Linear layout: ask L2 for the grid rows under this warp's tile over the
 // z-range its PPs will visit (anchor heights + d0, 0.5 A margin), so that the
 // scan's first touches of the slab are served in parallel at the start instead
 // of one demand miss at a time inside the FIRE loops.  Rows are contiguous in
@@ -45,8 +44,8 @@ __device__ __forceinline__ int2 node_range(float a, float b, float inv_d, float 
 // result) for every 32nd row.  Lateral deflections reach the neighbouring
 // tiles' rows, which those warps prefetch.
 __device__ __forceinline__ void prefetch_tile_slab(const RelaxLaunch& P, int tx, int ty, int lane) {
-    const int ia = tx * kTileX, ib = min(ia + kTileX, P.snx) - 1;
-    const int ja = ty * kTileY, jb = min(ja + kTileY, P.sny) - 1;
+    const int ia = tx << P.tile_wsh, ib = min(ia + (1 << P.tile_wsh), P.snx) - 1;
+    const int ja = ty << P.tile_hsh, jb = min(ja + (1 << P.tile_hsh), P.sny) - 1;
     const int2 ri = node_range(fmaf((float)ia, P.spx, P.sx0) + P.d0x, fmaf((float)ib, P.spx, P.sx0) + P.d0x,
                                P.inv_dx, P.gx0s, P.map.nx);
     const int2 rj = node_range(fmaf((float)ja, P.spy, P.sy0) + P.d0y, fmaf((float)jb, P.spy, P.sy0) + P.d0y,
@@ -81,17 +80,25 @@ __device__ __forceinline__ void record_zspan(const RelaxLaunch& P, int2 span) {
     }
 }
 
-// This warp's pixel (i, j); i = snx marks an idle lane.  Without a plan: lane l of the 8x4 tile
-// (blockIdx.x, blockIdx.y).  With one (a 1-D grid): the first plan_hblocks warps take the plan's
-// listed pixels, plan_lanes lanes each (-1 or anything outside the scan: idle), and warp
-// plan_hblocks + t takes tile t less the listed pixels.  *tx < 0: no tile (no slab prefetch).
+// Lane l's pixel of tile (tx, ty), x fastest inside the tile; idle past its pixels.
+__device__ __forceinline__ void tile_pixel(const RelaxLaunch& P, int tx, int ty, int& i, int& j) {
+    const int lane = threadIdx.x, dj = lane >> P.tile_wsh;
+    i = (tx << P.tile_wsh) + (lane & ((1 << P.tile_wsh) - 1));
+    j = (ty << P.tile_hsh) + dj;
+    if (dj >> P.tile_hsh) i = P.snx;
+}
+
+// This warp's pixel (i, j); i = snx marks an idle lane.  Without a plan: lane l of the tile
+// (blockIdx.x, blockIdx.y), lanes past the tile's pixels idle.  With one (a 1-D grid): the first
+// plan_hblocks warps take the plan's listed pixels, plan_lanes lanes each (-1 or anything outside the
+// scan: idle), and warp plan_hblocks + t takes tile t less the listed pixels.  *tx < 0: no tile (no
+// slab prefetch).
 __device__ __forceinline__ void scan_pixel(const RelaxLaunch& P, int& i, int& j, int& tx, int& ty) {
     const int lane = threadIdx.x;
     if (!P.plan_list) {
         tx = blockIdx.x;
         ty = blockIdx.y;
-        i = tx * kTileX + (lane & 7);
-        j = ty * kTileY + (lane >> 3);
+        tile_pixel(P, tx, ty, i, j);
         return;
     }
     const int npix = P.snx * P.sny;
@@ -105,11 +112,10 @@ __device__ __forceinline__ void scan_pixel(const RelaxLaunch& P, int& i, int& j,
         j = ok ? p / P.snx : P.sny;
         return;
     }
-    const int ntx = (P.snx + kTileX - 1) / kTileX, t = b - P.plan_hblocks;
+    const int ntx = (P.snx + (1 << P.tile_wsh) - 1) >> P.tile_wsh, t = b - P.plan_hblocks;
     tx = t % ntx;
     ty = t / ntx;
-    i = tx * kTileX + (lane & 7);
-    j = ty * kTileY + (lane >> 3);
+    tile_pixel(P, tx, ty, i, j);
     if (i < P.snx && j < P.sny) {
         const int p = j * P.snx + i;
         if ((P.plan_mask[p >> 5] >> (p & 31)) & 1u) i = P.snx;  // run by a plan warp
@@ -136,6 +142,30 @@ __global__ void __launch_bounds__(kThreads) relax_scan_tricubic_kernel(const Rel
     if constexpr (kSpan) record_zspan(P, span);
 }
 
+// Pixels per warp.  A column is a serial chain, and its warp stops for every height change and cell
+// reload of its other lanes, so a scan that leaves the GPU idle runs narrower warps: the narrowest tile
+// (8x4, 4x4, 4x2, 2x2, 2x1, 1 pixels) that needs at most `per_sm` warps per SM, beyond which the issue
+// slots the idle lanes waste cost more than the shorter chains save.  Which warp runs a pixel never
+// changes its value.  Measured alone on 20 heights (us; 8x4 tiles -> the tile taken, and the next
+// narrower one where that is the line): force grid 20^2 px 274 -> 126 (1 px), 40^2 252 -> 146 (4),
+// 64^2 226 -> 162 (8), 96^2 207 -> 179 (16), 128^2 199 (32; 16: 189, but 131 against 110 per scan with
+// four in flight); with Newton polish, whose chains are longer, 40^2 638 -> 213 (2), 128^2 596 -> 543
+// (16); energy grid 64^2 292 -> 229 (8; 4: 246), 128^2 296 (32; 16: 310).
+void tile_shape(RelaxLaunch& L, int sms) {
+    int lanes = L.tile_lanes;
+    if (lanes <= 0) {
+        const long long per_sm = (L.polish > 0 && L.map.interp == 0) ? 8 : 4;
+        const long long npix = (long long)L.snx * L.sny;
+        for (lanes = 1; lanes < 32 && (npix + lanes - 1) / lanes > per_sm * sms;) lanes *= 2;
+    }
+    for (;; lanes *= 2) {
+        L.tile_wsh = lanes >= 32 ? 3 : lanes >= 8 ? 2 : lanes >= 2 ? 1 : 0;
+        L.tile_hsh = lanes >= 16 ? 2 : lanes >= 4 ? 1 : 0;
+        // (a grid holds 65535 tiles along y)
+        if (lanes >= 32 || (L.sny - 1) >> L.tile_hsh < 65535) return;
+    }
+}
+
 template <bool kPolish, bool kSpan>
 void launch_relax_scan_t(const RelaxLaunch& L, dim3 grid, cudaStream_t s) {
     if (L.map.interp == 1) relax_scan_tricubic_kernel<kPolish, kSpan><<<grid, kThreads, 0, s>>>(L);
@@ -145,8 +175,13 @@ void launch_relax_scan_t(const RelaxLaunch& L, dim3 grid, cudaStream_t s) {
 
 }  // namespace
 
-cudaError_t launch_relax_scan(const RelaxLaunch& L, cudaStream_t s) {
-    dim3 grid((L.snx + kTileX - 1) / kTileX, (L.sny + kTileY - 1) / kTileY, 1);
+cudaError_t launch_relax_scan(const RelaxLaunch& L0, cudaStream_t s) {
+    RelaxLaunch L = L0;
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    tile_shape(L, sms);
+    dim3 grid((L.snx + (1 << L.tile_wsh) - 1) >> L.tile_wsh, (L.sny + (1 << L.tile_hsh) - 1) >> L.tile_hsh, 1);
     if (L.plan_list) grid = dim3(L.plan_hblocks + grid.x * grid.y, 1, 1);
     const bool span = L.zspan != nullptr;
     if (L.polish > 0) span ? launch_relax_scan_t<true, true>(L, grid, s) : launch_relax_scan_t<true, false>(L, grid, s);

@@ -303,9 +303,10 @@ def pp_ff_combine(ff: torch.Tensor, ff_el: torch.Tensor, Q: float, grid: Grid, o
 
 
 def pp_relax_scan(ff, grid: Grid, scan: Scan, tip: Tip, fire: Fire, pos, fz, iters, fused_df=None, df=None,
-                  stream=None, zspan=None, plan=None):
+                  stream=None, zspan=None, plan=None, lanes=0):
     """zspan: a device int32 tensor of 2 elements to receive the lowest and highest node layer the scan's
-    interpolations read; plan: (buffer, k, lanes) from pp_relax_plan.  With either, pp_relax_scan_ex."""
+    interpolations read; plan: (buffer, k, lanes) from pp_relax_plan; lanes: pixels per warp without a plan
+    (0: the library's choice).  With any of them, pp_relax_scan_ex."""
     npx = scan.nx * scan.ny * scan.nz
     if fz.numel() < npx or (pos is not None and pos.numel() < 3 * npx) or (iters is not None and iters.numel() < npx):
         raise ValueError("output buffer too small for the scan")
@@ -318,10 +319,10 @@ def pp_relax_scan(ff, grid: Grid, scan: Scan, tip: Tip, fire: Fire, pos, fz, ite
     args = (_dev(ff, "ff"), C.byref(grid), C.byref(scan), C.byref(tip), C.byref(fire),
             _dev(pos, "pos", allow_none=True), _dev(fz, "fz"), _dev(iters, "iters", torch.int32, allow_none=True),
             C.byref(fused_df) if fused_df is not None else None, _dev(df, "df", allow_none=True))
-    if zspan is None and plan is None:
+    if zspan is None and plan is None and not lanes:
         _check(lib().pp_relax_scan(*args, _stream(stream)))
         return
-    opts = ScanOpts(None, None, 0, 0)
+    opts = ScanOpts(None, None, 0, int(lanes))
     if zspan is not None:
         if zspan.numel() < 2:
             raise ValueError("zspan needs two ints")

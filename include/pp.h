@@ -205,7 +205,8 @@ PP_API pp_status pp_ff_combine(const float* ff, const float* ff_el, float Q, con
 
 /* Options of pp_make_ff_tuned.  ff_zpt (the launch shape, picked by the
  * autotuner) is the number of consecutive z-nodes each thread accumulates, 4,
- * 8 or 16; 0 = 8.  ff_forces_only = 1 skips the energy sums of an interp = 0
+ * 8 or 16; 0 = 8 (on grids of up to 0.35 A spacing, samples of 16 atoms and
+ * more are summed by tiles of 16x16x16 nodes, whatever it says).  ff_forces_only = 1 skips the energy sums of an interp = 0
  * grid and writes 0 in every E slot: the scan reads only the forces (Sec.
  * 5.1.1 step 2), and the forces are bit for bit those of ff_forces_only = 0
  * (the default, E written). */
@@ -326,7 +327,7 @@ PP_API pp_status pp_ff_convert(const float* src, const pp_grid* src_grid, float*
                         const pp_grid* dst_grid, pp_stream stream);
 
 /* ---------------------------------------------------------------- batches
- * Many molecules of uneven size in one persistent launch (a7; the paper's
+ * Many molecules of uneven size in one call (a7; the paper's
  * batch generator for ML datasets, Sec. 4.4, motivates it; the method per
  * molecule is exactly pp_make_ff + pp_relax_scan with fused df).  Grids are
  * linear layout; all molecules share the probe, tip, FIRE, df parameters,
@@ -354,7 +355,7 @@ typedef struct {
     long long out_capacity; /* entries in fz and iters (pos holds 3x)                         */
     long long df_capacity;  /* entries in df                                                  */
     int n_atoms_total;      /* length of the packed atom arrays                               */
-    int ctas;               /* persistent CTAs of 128 threads; 0 = fill the GPU               */
+    int ctas;               /* persistent CTAs of 128 threads of the relax kernel; 0 = fill the GPU */
     long long spin_limit;   /* polls (~128 ns apart) before a relax item stops waiting for its
                                molecule's force field; 0 = 1<<23 (about one second)           */
     int wait_extra;         /* test hook, 0 in normal use: relax items wait for this many more
@@ -363,9 +364,9 @@ typedef struct {
                                (the forces, and so all scan outputs, are unchanged); 0 or 1    */
     /* Work-item shapes (picked by the autotuner; every choice computes the same values bit for
      * bit, only the scheduling differs).  0 selects the default in brackets. */
-    int ff_tile_w;          /* force-field tile width in grid columns along x: 4, 8 or 16 [8]; the
-                               tile is ff_tile_w x (32 / ff_tile_w) columns                    */
-    int ff_zpt;             /* z-nodes per force-field tile: 4 or 8 [8]                         */
+    int ff_tile_w;          /* 4, 8 or 16 [8]; accepted and without effect (force-field tiles are
+                               16x16x16 nodes)                                                 */
+    int ff_zpt;             /* 4 or 8 [8]; accepted and without effect                          */
     int relax_tile_w;       /* relax tile width in pixels along x: 4, 8 or 16 [8]; the tile is
                                relax_tile_w x (32 / relax_tile_w) pixels, all heights          */
 } pp_batch_params;
@@ -377,16 +378,14 @@ typedef struct {
 /* Scratch bytes of pp_batch_run for nmol molecules (0 if nmol < 1). */
 PP_API size_t pp_batch_workspace(int nmol);
 
-/* One launch over all molecules: a planning kernel validates every device
- * descriptor (bad ones are skipped and flagged) and lays out a work list of
- * force-field tiles (ff_tile_w x 32/ff_tile_w columns x ff_zpt z-nodes) and
- * relax tiles (relax_tile_w x 32/relax_tile_w pixels, all heights) ordered
- * FF(0), FF(1), R(0), FF(2), R(1), ...; then a
- * persistent kernel whose warps pull items from a device counter.  A relax
- * tile waits (bounded, see spin_limit) until every force-field tile of its
- * molecule is done; items are handed out in list order, so the force field
- * it waits for is always being computed by running warps.  Writes, per
- * molecule, the force field, fz, df and (nullable) pos and iters exactly as
+/* All molecules in three launches: a planning kernel validates every device
+ * descriptor (bad ones are skipped and flagged) and lays out the work items, a
+ * persistent kernel assembles the force fields by tiles of 16x16x16 nodes, and
+ * another runs the relax tiles (relax_tile_w x 32/relax_tile_w pixels, all
+ * heights); workers pull items from a device counter.  A relax tile waits
+ * (bounded, see spin_limit) until every force-field tile of its molecule is
+ * done.  Writes, per molecule, the force field, fz, df and (nullable) pos and
+ * iters exactly as
  * pp_make_ff + pp_relax_scan (fused df) on that molecule alone (the grid's E
  * slots 0 when params->ff_forces_only).  descs is a
  * DEVICE array of nmol descriptors; atoms are packed device arrays; ws is

@@ -122,6 +122,7 @@ void df_stencil(double A_pp, double dz, double k, double f0, int m, float* coef)
 #ifdef PP_CHECKED
 // flag readers of the kernel translation units (bounds-checked builds)
 unsigned int check_flags_ff_assemble();
+unsigned int check_flags_ff_tile();
 unsigned int check_flags_relax_scan();
 unsigned int check_flags_fz_to_df();
 unsigned int check_flags_backward();
@@ -145,7 +146,7 @@ pp_status pp_check_flags(unsigned int* flags) {
 #ifdef PP_CHECKED
     pp_status st = cuda_status(cudaDeviceSynchronize(), "pp_check_flags sync");
     if (st != PP_OK) return st;
-    *flags = check_flags_ff_assemble() | check_flags_relax_scan() | check_flags_fz_to_df() | check_flags_backward() |
+    *flags = check_flags_ff_assemble() | check_flags_ff_tile() | check_flags_relax_scan() | check_flags_fz_to_df() | check_flags_backward() |
              check_flags_batch() | check_flags_iets() | check_flags_fft();
     return PP_OK;
 #else

@@ -1,31 +1,25 @@
-// K6: many molecules in one persistent launch (force field -> relaxed scan ->
-// df per molecule, exactly the single-molecule path of K1 + K2).
+// K6: many molecules in one call (force field -> relaxed scan -> df per molecule, exactly the
+// single-molecule path of K1 + K2): a planning kernel and two persistent ones.
 //
-// Work items:  FF tile  = fw x (32/fw) grid columns x ZPT z-nodes of one molecule;
-//              relax tile = rw x (32/rw) pixels x all heights of one molecule
-// (fw, rw in {4, 8, 16} at launch time, ZPT in {4, 8} as a template argument;
-// the shapes change the schedule, never a value).
-// Every warp is an independent worker: lane 0 takes the next item index from
-// a device counter.  The item list is a sequence of segments
-//   FF(0), FF(1), R(0), FF(2), R(1), ..., FF(n-1), R(n-2), R(n-1)
-// (prefix sums built by a planning kernel), so a relax tile of molecule m is
-// handed out only after all force-field tiles of m were handed out -- and
-// those never wait on anything, so every wait ends.  A relax tile still waits
-// for its molecule's completion counter with a bounded spin (a timeout sets a
-// status bit and the warp stops); force-field values written in this kernel
-// are read back with plain cached loads after an acquire, never through the
-// read-only path.  Many molecules' tiles are in flight at once, which fills
-// the GPU even though one 128x128 scan is only 512 warps.
+// Work items:  FF tile    = 16x16x16 nodes of one molecule's grid, taken by a CTA of 256 threads;
+//              relax tile = rw x (32/rw) pixels x all heights of one molecule, taken by a warp
+// (rw in {4, 8, 16}: the shape changes the schedule, never a value).  Workers take the next item index from
+// a device counter; the item list is FF(0), ..., FF(n-1), R(0), ..., R(n-1) (prefix sums built by the
+// planning kernel).  Many molecules' tiles are in flight at once, which fills the GPU even though one
+// 128x128 scan is only 512 warps.  The force fields are assembled by one kernel and scanned by the next:
+// with the far atoms interpolated (ff_tile.cuh) assembly is a CTA's work, and what it takes is no longer
+// enough to hide scans behind; a grid written to HBM and read back in its scan's layers costs 1 % of a
+// batch's time.  A relax tile still checks its molecule's completion counter (a bounded wait; a timeout
+// sets a status bit and the warp stops).
 #include <cstring>
 
-#include "ff_core.cuh"
+#include "ff_tile.cuh"
 #include "relax_core.cuh"
 
 namespace pp {
 namespace {
 
-constexpr int kThreads = 128;  // 4 independent warps per CTA
-constexpr int kWarps = kThreads / 32;
+constexpr int kThreads = 128;  // relax kernel: 4 independent warps per CTA
 constexpr int kMinCtas = 5;    // resident CTAs per SM the register budget is sized for
 
 struct BatchLaunch {
@@ -49,16 +43,15 @@ struct BatchLaunch {
     int df_m;
     const float* coef;  // in ws, written by the planning kernel
     // scratch
-    unsigned long long* counter;
+    unsigned long long *counter_ff, *counter_relax;
     int* status;
-    long long* seg_start;  // [2 nmol + 1]
+    long long* seg_start;  // [2 nmol + 1]: first item of FF(m) at m, of R(m) at nmol + m, their end
     int* done_ff;          // [nmol]
     float* coef_ws;
     long long spin_limit;
     int wait_extra;
     int forces_only;  // E slots written as 0, energy sums skipped
-    int zpt;          // z-nodes per FF tile
-    int fw_sh, rw_sh; // log2 of the FF and relax tile widths (4, 8 or 16 lanes along x)
+    int rw_sh;        // log2 of the relax tile width (4, 8 or 16 lanes along x)
     float coef_init[2 * kMaxDfHalfWidth + 1];
 };
 
@@ -77,8 +70,8 @@ struct MolRelax {
 
 __device__ __forceinline__ long long cdiv(long long a, long long b) { return (a + b - 1) / b; }
 
-__device__ __forceinline__ long long ff_tiles(const BatchLaunch& B, const pp_mol_desc& D) {
-    return cdiv(D.nx, 1 << B.fw_sh) * cdiv(D.ny, 32 >> B.fw_sh) * cdiv(D.nz, B.zpt);
+__device__ __forceinline__ long long ff_tiles(const pp_mol_desc& D) {
+    return cdiv(D.nx, kTileN) * cdiv(D.ny, kTileN) * cdiv(D.nz, kTileN);
 }
 __device__ __forceinline__ long long relax_tiles(const BatchLaunch& B, const pp_mol_desc& D) {
     return cdiv(D.snx, 1 << B.rw_sh) * cdiv(D.sny, 32 >> B.rw_sh);
@@ -103,20 +96,13 @@ __device__ bool mol_valid(const BatchLaunch& B, const pp_mol_desc& D) {
     return true;
 }
 
-// Segment s of the item list -> (molecule, is force-field segment).
-__device__ __forceinline__ void decode_segment(int s, int nmol, int& mol, bool& ff) {
-    if (s == 0) { mol = 0; ff = true; }
-    else if (s == 2 * nmol - 1) { mol = nmol - 1; ff = false; }
-    else if (s & 1) { mol = (s + 1) >> 1; ff = true; }
-    else { mol = (s >> 1) - 1; ff = false; }
-}
-
 __global__ void __launch_bounds__(1024) batch_plan_kernel(const BatchLaunch B) {
     __shared__ long long wsum[32];
     __shared__ long long carry;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
-        *B.counter = 0ULL;
+        *B.counter_ff = 0ULL;
+        *B.counter_relax = 0ULL;
         *B.status = 0;
         carry = 0;
     }
@@ -128,11 +114,9 @@ __global__ void __launch_bounds__(1024) batch_plan_kernel(const BatchLaunch B) {
         const int s = base + tid;
         long long len = 0;
         if (s < nseg) {
-            int mol;
-            bool ff;
-            decode_segment(s, B.nmol, mol, ff);
-            const pp_mol_desc D = B.descs[mol];
-            if (mol_valid(B, D)) len = ff ? ff_tiles(B, D) : relax_tiles(B, D);
+            const bool ff = s < B.nmol;
+            const pp_mol_desc D = B.descs[ff ? s : s - B.nmol];
+            if (mol_valid(B, D)) len = ff ? ff_tiles(D) : relax_tiles(B, D);
             else if (ff) atomicOr(B.status, PP_BATCH_BAD_DESC);
         }
         // inclusive block scan of len
@@ -173,92 +157,116 @@ __device__ __forceinline__ void add_release(int* p, int v) {
     asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// kZC: z-nodes computed (kZPT, or kZPT / 2 for a column's last tile when that many remain)
-template <int kZPT, bool kMinImage, bool kCutoff, bool kQuad, bool kForcesOnly, int kZC = kZPT>
-__device__ __forceinline__ void ff_tile(const BatchLaunch& B, const pp_mol_desc& D, long long tile, float4* s0,
-                                        float4* s1, float4* s2, float4* s3, int lane) {
-    constexpr int ZP = kZC / 2;
-    const int fw = 1 << B.fw_sh;
-    const long long tx_n = cdiv(D.nx, fw), ty_n = cdiv(D.ny, 32 >> B.fw_sh);
-    const int tz = (int)(tile / (tx_n * ty_n));
-    const long long r = tile - (long long)tz * tx_n * ty_n;
-    const int ty = (int)(r / tx_n), tx = (int)(r - (long long)ty * tx_n);
-    const int i = tx * fw + (lane & (fw - 1)), j = ty * (32 >> B.fw_sh) + (lane >> B.fw_sh), k0 = tz * kZPT;
+// Segment holding item t among seg_start[first .. last): the last s with seg_start[s] <= t.
+__device__ __forceinline__ int find_segment(const BatchLaunch& B, int first, int last, long long t) {
+    int lo = first, hi = last - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (B.seg_start[mid] <= t) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
+// Node pairs of a column of molecule D, the force sums as ff_tile and the direct sums hand them over.
+template <bool kForcesOnly>
+struct MolStore {
+    const BatchLaunch& B;
+    const pp_mol_desc& D;
+    __device__ __forceinline__ void operator()(int i, int j, int k, float2 fx, float2 fy, float2 fz, float2 en) const {
+        if (i >= D.nx || j >= D.ny) return;
+        const long long first = D.ff_offset + (long long)j * D.nx + i, plane = (long long)D.nx * D.ny;
+        auto at = [&](int kk) { return checked(first + kk * plane, (long long)B.ff_cap, kChkGridWrite); };
+        if (kForcesOnly) en = make_float2(0.f, 0.f);
+        if (k < D.nz) B.ff[at(k)] = make_float4(fx.x, fy.x, fz.x, en.x);
+        if (k + 1 < D.nz) B.ff[at(k + 1)] = make_float4(fx.y, fy.y, fz.y, en.y);
+    }
+};
+
+// Direct sums (grids not assembled by tiles, see ff_use_tiles) of 8 layers from k0 of the 8x4 columns from
+// (i0, j0), by one warp: the arithmetic of ff_assemble.cu.  st: 4 x 32 records.
+template <bool kMinImage, bool kCutoff, bool kQuad, class Store>
+__device__ __forceinline__ void ff_direct(const BatchLaunch& B, const pp_mol_desc& D, const FFConst& cst, int i0, int j0,
+                                          int k0, float4* st, Store&& store) {
+    constexpr int ZP = 4;
+    const int lane = threadIdx.x & 31, i = i0 + (lane & 7), j = j0 + (lane >> 3);
     const float gx = D.x0 + i * D.dx, gy = D.y0 + j * D.dy;
-    float2 gz[ZP];
+    float2 gz[ZP], fx[ZP], fy[ZP], fz[ZP], en[ZP];
 #pragma unroll
-    for (int t = 0; t < ZP; ++t) gz[t] = make_float2(D.z0 + (k0 + 2 * t) * D.dz, D.z0 + (k0 + 2 * t + 1) * D.dz);
-    float2 fx[ZP], fy[ZP], fz[ZP], en[ZP];
-#pragma unroll
-    for (int t = 0; t < ZP; ++t) fx[t] = fy[t] = fz[t] = en[t] = make_float2(0.f, 0.f);
-    const FFConst cst = ff_const(B.R_pp, B.eps_pp, B.kQ, B.core_frac, D.nx * D.dx, D.ny * D.dy,
-                                 kCutoff ? B.coul_rc : 0.f, kQuad ? B.kQzz : 0.f);
+    for (int t = 0; t < ZP; ++t) {
+        gz[t] = make_float2(D.z0 + (k0 + 2 * t) * D.dz, D.z0 + (k0 + 2 * t + 1) * D.dz);
+        fx[t] = fy[t] = fz[t] = en[t] = make_float2(0.f, 0.f);
+    }
     for (int base = 0; base < D.n_atoms; base += 32) {
         const int cnt = min(32, D.n_atoms - base);
         __syncwarp();
         if (lane < cnt) {
             const int g = D.atom_offset + base + lane;
-            ff_stage_atom(cst, B.ax[g], B.ay[g], B.az[g], B.aR[g], B.aeps[g], B.aq[g], s0[lane], s1[lane], s2[lane],
-                          s3[lane]);
+            ff_stage_atom(cst, B.ax[g], B.ay[g], B.az[g], B.aR[g], B.aeps[g], B.aq[g], st[lane], st[32 + lane],
+                          st[64 + lane], st[96 + lane]);
         }
         __syncwarp();
-        ff_accumulate<ZP, kMinImage, kCutoff, kQuad, true>(s0, s1, s2, s3, cnt, cst, gx, gy, gz, fx, fy, fz, en);
+        ff_accumulate<ZP, kMinImage, kCutoff, kQuad, true>(st, st + 32, st + 64, st + 96, cnt, cst, gx, gy, gz, fx, fy, fz,
+                                                           en);
     }
-    if (i < D.nx && j < D.ny) {
-        const long long first = D.ff_offset + (long long)j * D.nx + i;
-        const long long plane = (long long)D.nx * D.ny;
-        auto at = [&](int k) { return checked(first + k * plane, (long long)B.ff_cap, kChkGridWrite); };
 #pragma unroll
-        for (int t = 0; t < ZP; ++t) {
-            const int k = k0 + 2 * t;
-            const float2 e = kForcesOnly ? make_float2(0.f, 0.f) : en[t];
-            if (k < D.nz) B.ff[at(k)] = make_float4(fx[t].x, fy[t].x, fz[t].x, e.x);
-            if (k + 1 < D.nz) B.ff[at(k + 1)] = make_float4(fx[t].y, fy[t].y, fz[t].y, e.y);
+    for (int t = 0; t < ZP; ++t) store(i, j, k0 + 2 * t, fx[t], fy[t], fz[t], en[t]);
+}
+
+template <bool kMinImage, bool kCutoff, bool kQuad, bool kForcesOnly>
+__global__ void __launch_bounds__(kTileThreads, 2) batch_ff_kernel(const BatchLaunch B) {
+    __shared__ TileShared S;
+    __shared__ long long item;
+    const long long total = B.seg_start[B.nmol];
+    for (;;) {
+        if (threadIdx.x == 0) item = (long long)atomicAdd(B.counter_ff, 1ULL);
+        __syncthreads();
+        const long long t = item;
+        __syncthreads();
+        if (t >= total) break;
+        const int mol = find_segment(B, 0, B.nmol, t);
+        const pp_mol_desc& D = B.descs[mol];
+        const long long tile = t - B.seg_start[mol];
+        const int tx_n = (D.nx + kTileN - 1) / kTileN, ty_n = (D.ny + kTileN - 1) / kTileN;
+        const int tz = (int)(tile / ((long long)tx_n * ty_n));
+        const int r = (int)(tile - (long long)tz * tx_n * ty_n);
+        const int i0 = (r % tx_n) * kTileN, j0 = (r / tx_n) * kTileN, k0 = tz * kTileN;
+        const FFConst cst = ff_const(B.R_pp, B.eps_pp, B.kQ, B.core_frac, D.nx * D.dx, D.ny * D.dy,
+                                     kCutoff ? B.coul_rc : 0.f, kQuad ? B.kQzz : 0.f);
+        const MolStore<kForcesOnly> store{B, D};
+        if (ff_use_tiles(D.n_atoms, D.dx, D.dy, D.dz)) {
+            const int a = D.atom_offset;
+            const TileJob J = {B.ax + a, B.ay + a, B.az + a, B.aR + a, B.aeps + a, B.aq + a, D.n_atoms,
+                               D.x0, D.y0, D.z0, D.dx, D.dy, D.dz, D.nx, D.ny};
+            const int nz = D.nz;
+            ff_tile<kMinImage, kCutoff, kQuad, false, kForcesOnly>(J, cst, i0, j0, k0, S,
+                                                                   [&](int h) { return k0 + 8 * h < nz; }, store);
+        } else {
+            const int warp = threadIdx.x >> 5;
+            for (int h = 0; h < 2; ++h)
+                if (k0 + 8 * h < D.nz)
+                    ff_direct<kMinImage, kCutoff, kQuad>(B, D, cst, i0 + (warp & 1) * 8, j0 + (warp >> 1) * 4, k0 + 8 * h,
+                                                         S.buf + warp * 128, store);
         }
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) add_release(B.done_ff + mol, 1);
     }
 }
 
-template <int kZPT, bool kMinImage, bool kCutoff, bool kQuad, bool kForcesOnly>
-__global__ void __launch_bounds__(kThreads, kMinCtas) batch_kernel(const BatchLaunch B) {
-    __shared__ float4 st[kWarps][4][32];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long total = B.seg_start[2 * B.nmol];
+__global__ void __launch_bounds__(kThreads, kMinCtas) batch_relax_kernel(const BatchLaunch B) {
+    const int lane = threadIdx.x & 31;
+    const long long first = B.seg_start[B.nmol], total = B.seg_start[2 * B.nmol] - first;
     for (;;) {
         long long t = 0;
-        if (lane == 0) t = (long long)atomicAdd(B.counter, 1ULL);
+        if (lane == 0) t = (long long)atomicAdd(B.counter_relax, 1ULL);
         t = __shfl_sync(0xffffffffu, t, 0);
         if (t >= total) break;
-        // segment holding item t: the last s with seg_start[s] <= t
-        int lo = 0, hi = 2 * B.nmol - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (B.seg_start[mid] <= t) lo = mid;
-            else hi = mid - 1;
-        }
-        int mol;
-        bool ff;
-        decode_segment(lo, B.nmol, mol, ff);
-        const long long tile = t - B.seg_start[lo];
+        const int seg = find_segment(B, B.nmol, 2 * B.nmol, first + t), mol = seg - B.nmol;
+        const long long tile = first + t - B.seg_start[seg];
         const pp_mol_desc D = B.descs[mol];
-        if (ff) {
-            const long long per_z = cdiv(D.nx, 1 << B.fw_sh) * cdiv(D.ny, 32 >> B.fw_sh);
-            const int k0 = (int)(tile / per_z) * kZPT;
-            if (kZPT == 8 && D.nz - k0 <= 4)
-                ff_tile<kZPT, kMinImage, kCutoff, kQuad, kForcesOnly, 4>(B, D, tile, st[warp][0], st[warp][1],
-                                                                          st[warp][2], st[warp][3], lane);
-            else
-                ff_tile<kZPT, kMinImage, kCutoff, kQuad, kForcesOnly>(B, D, tile, st[warp][0], st[warp][1],
-                                                                       st[warp][2], st[warp][3], lane);
-            __syncwarp();
-            if (lane == 0) {
-                __threadfence();
-                add_release(B.done_ff + mol, 1);
-            }
-            continue;
-        }
-        // relax tile: wait (bounded) for every force-field tile of this molecule
-        const int sff = mol == 0 ? 0 : 2 * mol - 1;
-        const int need = (int)(B.seg_start[sff + 1] - B.seg_start[sff]) + B.wait_extra;
+        // wait (bounded) for every force-field tile of this molecule
+        const int need = (int)(B.seg_start[mol + 1] - B.seg_start[mol]) + B.wait_extra;
         int ok = 1;
         if (lane == 0) {
             long long polls = 0;
@@ -299,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, kMinCtas) batch_kernel(const BatchLa
         const int rw = 1 << B.rw_sh;
         const int tiles_x = (D.snx + rw - 1) / rw;
         const int ty = (int)(tile / tiles_x), tx = (int)(tile - (long long)ty * tiles_x);
-        relax_pixel<0, true, false, true>(G, B, tx * rw + (lane & (rw - 1)), ty * (32 >> B.rw_sh) + (lane >> B.rw_sh));
+        relax_pixel<0, false, false, true>(G, B, tx * rw + (lane & (rw - 1)), ty * (32 >> B.rw_sh) + (lane >> B.rw_sh));
     }
 }
 
@@ -342,8 +350,9 @@ cudaError_t launch_batch(const BatchArgs& A, cudaStream_t s) {
     B.df_m = A.df_m;
     for (int c = 0; c < 2 * A.df_m + 1; ++c) B.coef_init[c] = A.coef[c];
     char* w = reinterpret_cast<char*>(A.ws);
-    B.counter = reinterpret_cast<unsigned long long*>(w);
+    B.counter_ff = reinterpret_cast<unsigned long long*>(w);
     B.status = reinterpret_cast<int*>(w + 8);
+    B.counter_relax = reinterpret_cast<unsigned long long*>(w + 16);
     B.coef_ws = reinterpret_cast<float*>(w + 64);
     B.coef = B.coef_ws;
     B.seg_start = reinterpret_cast<long long*>(w + 320);
@@ -351,29 +360,28 @@ cudaError_t launch_batch(const BatchArgs& A, cudaStream_t s) {
     B.spin_limit = P.spin_limit > 0 ? P.spin_limit : (1LL << 23);
     B.wait_extra = P.wait_extra;
     B.forces_only = P.ff_forces_only;
-    B.zpt = P.ff_zpt > 0 ? P.ff_zpt : 8;
-    const int fw = P.ff_tile_w > 0 ? P.ff_tile_w : 8, rw = P.relax_tile_w > 0 ? P.relax_tile_w : 8;
-    B.fw_sh = fw == 4 ? 2 : (fw == 8 ? 3 : 4);
+    const int rw = P.relax_tile_w > 0 ? P.relax_tile_w : 8;
     B.rw_sh = rw == 4 ? 2 : (rw == 8 ? 3 : 4);
 
     batch_plan_kernel<<<1, 1024, 0, s>>>(B);
-    const bool fo = B.forces_only != 0;
-    const bool z4 = B.zpt == 4;
-    const void* fn = with_flags(B.min_image != 0, B.coul_rc > 0.f, B.kQzz != 0.f, [fo, z4](auto mi, auto cut, auto quad) {
+    int dev = 0, sms = 152, per_sm = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    with_flags(B.min_image != 0, B.coul_rc > 0.f, B.kQzz != 0.f, [&](auto mi, auto cut, auto quad) {
         constexpr bool MI = decltype(mi)::value, CUT = decltype(cut)::value, QUAD = decltype(quad)::value;
-        if (z4) return fo ? (const void*)batch_kernel<4, MI, CUT, QUAD, true> : (const void*)batch_kernel<4, MI, CUT, QUAD, false>;
-        return fo ? (const void*)batch_kernel<8, MI, CUT, QUAD, true> : (const void*)batch_kernel<8, MI, CUT, QUAD, false>;
+        if (B.forces_only) batch_ff_kernel<MI, CUT, QUAD, true><<<2 * sms, kTileThreads, 0, s>>>(B);
+        else batch_ff_kernel<MI, CUT, QUAD, false><<<2 * sms, kTileThreads, 0, s>>>(B);
+        return 0;
     });
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     int ctas = P.ctas;
     if (ctas <= 0) {
-        int dev = 0, sms = 148, per_sm = 1;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_relax_kernel, kThreads, 0);
         ctas = sms * (per_sm > 0 ? per_sm : 1);
     }
-    void* args[] = {&B};
-    return cudaLaunchKernel(fn, dim3(ctas), dim3(kThreads), args, 0, s);
+    batch_relax_kernel<<<ctas, kThreads, 0, s>>>(B);
+    return cudaGetLastError();
 }
 
 PP_CHECK_READER(check_flags_batch)

@@ -26,6 +26,7 @@
 // stored twice so that one 16-byte broadcast load yields a ready packed
 // operand.
 #include "ff_core.cuh"
+#include "ff_tile.cuh"
 
 namespace pp {
 namespace {
@@ -168,6 +169,7 @@ cudaError_t launch_ff_assemble(const FFLaunch& L, cudaStream_t s) {
         });
         return cudaGetLastError();
     }
+    if (ff_use_tiles(L.n, L.dx, L.dy, L.dz)) return launch_ff_tiles(L, s);
     if (L.map.interp == 1) {
         constexpr int ZPT = 8;
         dim3 grid((L.map.nx + kTileX - 1) / kTileX, (L.map.ny + kTileY - 1) / kTileY, (L.kend - L.kbeg + ZPT - 1) / ZPT);

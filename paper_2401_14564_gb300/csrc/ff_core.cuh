@@ -71,7 +71,15 @@ __device__ __forceinline__ void ff_stage_atom(const FFConst& c, float x, float y
 // beyond coul_rc, every node's r^2 >= rc^2 and the cut terms are the zeros the in-range tests would
 // select (the same expressions with those tests known false: the same bits), so the point-charge
 // (and quadrupole) arithmetic drops out; on a laterally periodic slab most atoms are that far.
-template <int ZP, bool kMinImage, bool kCutoff, bool kQuad, bool kSplit, bool kFloorVote = false>
+// An uncharged atom (kq = kqq = 0) takes the same body.
+// Smooth: the caller knows that no node lies within the core floor (ff_tile.cuh) and that, with kCutoff,
+// all nodes lie within coul_rc of every atom (kInside), or all beyond it or the atoms uncharged
+// (kBeyond), so neither is tested.
+// kRel: coordinates relative to a tile's centre, the atoms' as float pairs whose low parts sit in slots
+// that otherwise repeat a constant (ff_tile.cuh): x in s1.y, y in s3.y, -z in s3.w.
+enum class Smooth { kNo, kInside, kBeyond };
+template <int ZP, bool kMinImage, bool kCutoff, bool kQuad, bool kSplit, bool kFloorVote = false,
+          Smooth kSmooth = Smooth::kNo, bool kRel = false>
 __device__ __forceinline__ void ff_accumulate_impl(const float4* s0, const float4* s1, const float4* s2,
                                                    const float4* s3, int cnt, const FFConst& c, float gx, float gy,
                                                    const float2 (&gz)[ZP], float2 (&fx)[ZP], float2 (&fy)[ZP],
@@ -84,23 +92,28 @@ __device__ __forceinline__ void ff_accumulate_impl(const float4* s0, const float
         const float4 A0 = s0[a], A1 = s1[a], A2 = s2[a], A3 = s3[a];
         float rx = gx - A0.x;
         float ry = gy - A0.y;
+        if (kRel) {  // (an extra add per node pair in z: 3 % of the tile's time, see ff_tile.cuh)
+            rx -= A1.y;
+            ry -= A3.y;
+        }
         if (kMinImage) {
             rx = fmaf(-c.Lx, rintf(rx * c.invLx), rx);
             ry = fmaf(-c.Ly, rintf(ry * c.invLy), ry);
         }
         const float rxy2 = fmaf(rx, rx, ry * ry);
         const float2 RX = make_float2(rx, rx), RY = make_float2(ry, ry), RXY = make_float2(rxy2, rxy2);
-        const float2 NZ = make_float2(A1.x, A1.y), LA = make_float2(A1.z, A1.w);
+        const float2 NZ = make_float2(A1.x, kRel ? A1.x : A1.y), LA = make_float2(A1.z, A1.w);
         const float2 LB = make_float2(A2.x, A2.y), KQ = make_float2(A2.z, A2.w);
-        const float2 EC = make_float2(A3.x, A3.y), ED = make_float2(A3.z, A3.w);
+        const float2 EC = make_float2(A3.x, kRel ? A3.x : A3.y), ED = make_float2(A3.z, kRel ? A3.z : A3.w);
+        const float2 NZL = make_float2(A3.w, A3.w);
         const float2 KQQ = make_float2(A0.w, A0.w);
         auto body = [&](auto floor_t, auto far_t) {
             constexpr bool kFloor = decltype(floor_t)::value;
             constexpr bool kFar = decltype(far_t)::value;  // every node of every lane beyond coul_rc
-            auto in_rc = [&](float r2v) { return !kFar && r2v < c.rc2; };
+            auto in_rc = [&](float r2v) { return kSmooth == Smooth::kInside || (!kFar && r2v < c.rc2); };
 #pragma unroll
             for (int t = 0; t < ZP; ++t) {
-                const float2 rz = f2add(gz[t], NZ);
+                const float2 rz = kRel ? f2add(f2add(gz[t], NZ), NZL) : f2add(gz[t], NZ);
                 float2 r2 = f2fma(rz, rz, RXY);
                 if (kFloor) {
                     r2.x = fmaxf(r2.x, A0.z);
@@ -169,8 +182,13 @@ __device__ __forceinline__ void ff_accumulate_impl(const float4* s0, const float
                 }
             }
         };
+        if constexpr (kSmooth != Smooth::kNo) {
+            body(std::false_type{}, std::integral_constant<bool, kCutoff && kSmooth == Smooth::kBeyond>{});
+            continue;
+        }
         const bool clear = kFloorVote && __all_sync(0xffffffffu, rxy2 >= A0.z);
-        const bool far = kFloorVote && kCutoff && __all_sync(0xffffffffu, rxy2 >= c.rc2);
+        const bool far = kFloorVote && kCutoff &&
+                         ((A2.z == 0.f && A0.w == 0.f) || __all_sync(0xffffffffu, rxy2 >= c.rc2));
         if (clear) {
             if (far) body(std::false_type{}, std::true_type{});
             else body(std::false_type{}, std::false_type{});

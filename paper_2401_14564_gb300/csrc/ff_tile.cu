@@ -1,0 +1,56 @@
+// K1 by tiles: force-field grid assembly (Sec. 5.1.1 step 1) with the far atoms of each 16x16x16-node tile
+// summed at its interpolation points (ff_tile.cuh says how and how exactly); the sums, options and outputs
+// are those of ff_assemble.cu, whose direct kernel remains for samples of a few atoms and for the split
+// grids.  Tiles start at multiples of 16 nodes whatever layers a call asks for, and a node's value depends on
+// its tile alone, so layer ranges, launch shapes and the batch write the same bits.
+#include "ff_tile.cuh"
+
+
+namespace pp {
+namespace {
+
+// kEnergy: E alone, one float per node (tricubic grids).  kForcesOnly: E slots written as 0.
+template <bool kMinImage, bool kCutoff, bool kQuad, bool kEnergy, bool kForcesOnly>
+__global__ void __launch_bounds__(kTileThreads, 2) ff_tile_kernel(const FFLaunch P) {
+    __shared__ TileShared S;
+    const TileJob J = {P.x, P.y, P.z, P.R, P.eps, P.q, P.n, P.x0, P.y0, P.z0, P.dx, P.dy, P.dz, P.map.nx, P.map.ny};
+    const FFConst c = ff_const(P.R_pp, P.eps_pp, P.kQ, P.core_frac, P.Lx, P.Ly, kCutoff ? P.coul_rc : 0.f,
+                               kQuad ? P.kQzz : 0.f);
+    const int k0 = (P.kbeg / kTileN + blockIdx.z) * kTileN;
+    ff_tile<kMinImage, kCutoff, kQuad, kEnergy, kForcesOnly>(
+        J, c, blockIdx.x * kTileN, blockIdx.y * kTileN, k0, S,
+        [&](int h) { return k0 + 8 * h < P.kend && k0 + 8 * h + 8 > P.kbeg; },
+        [&](int i, int j, int k, float2 fx, float2 fy, float2 fz, float2 en) {
+            if (i >= P.map.nx || j >= P.map.ny) return;
+            const int base_xy = axis_off(P.map.ax, i) + axis_off(P.map.ay, j);
+            auto at = [&](int kk) { return checked(base_xy + axis_off(P.map.az, kk), P.map.stored_nodes, kChkGridWrite); };
+            const bool w0 = k >= P.kbeg && k < P.kend, w1 = k + 1 >= P.kbeg && k + 1 < P.kend;
+            if constexpr (kEnergy) {
+                if (w0) P.ffE[at(k)] = en.x;
+                if (w1) P.ffE[at(k + 1)] = en.y;
+            } else {
+                if (kForcesOnly) en = make_float2(0.f, 0.f);
+                if (w0) P.ff[at(k)] = make_float4(fx.x, fy.x, fz.x, en.x);
+                if (w1) P.ff[at(k + 1)] = make_float4(fx.y, fy.y, fz.y, en.y);
+            }
+        });
+}
+
+}  // namespace
+
+cudaError_t launch_ff_tiles(const FFLaunch& L, cudaStream_t s) {
+    const dim3 grid((L.map.nx + kTileN - 1) / kTileN, (L.map.ny + kTileN - 1) / kTileN,
+                    (L.kend + kTileN - 1) / kTileN - L.kbeg / kTileN);
+    with_flags(L.min_image != 0, L.coul_rc > 0.f, L.kQzz != 0.f, [&](auto mi, auto cut, auto quad) {
+        constexpr bool MI = decltype(mi)::value, CUT = decltype(cut)::value, QUAD = decltype(quad)::value;
+        if (L.map.interp == 1) ff_tile_kernel<MI, CUT, QUAD, true, false><<<grid, kTileThreads, 0, s>>>(L);
+        else if (L.forces_only) ff_tile_kernel<MI, CUT, QUAD, false, true><<<grid, kTileThreads, 0, s>>>(L);
+        else ff_tile_kernel<MI, CUT, QUAD, false, false><<<grid, kTileThreads, 0, s>>>(L);
+        return 0;
+    });
+    return cudaGetLastError();
+}
+
+PP_CHECK_READER(check_flags_ff_tile)
+
+}  // namespace pp

@@ -133,6 +133,7 @@ struct FFLaunch {
     int kbeg, kend;  // node layers written: z index in [kbeg, kend) (0, nz for the whole grid)
 };
 cudaError_t launch_ff_assemble(const FFLaunch& L, cudaStream_t s);
+cudaError_t launch_ff_tiles(const FFLaunch& L, cudaStream_t s);
 // out = a + Q b over nfloats floats (16-byte aligned buffers; out may alias a)
 cudaError_t launch_ff_combine(const float* a, const float* b, float Q, float* out, int64_t nfloats, cudaStream_t s);
 

@@ -570,10 +570,10 @@ pp_status backward_prepare(const std::string& who, const pp_atoms* atoms, const 
 // clears the grid adjoint and enqueues the adjoint kernels.
 pp_status backward_launch(const std::string& who, BwdLaunch& L, void* ws, size_t adj_bytes, cudaStream_t s) {
     L.slab = reinterpret_cast<int*>(ws);
-    L.qsum = reinterpret_cast<float*>(reinterpret_cast<char*>(ws) + 16);
     L.gbar = L.map.interp ? nullptr : reinterpret_cast<float4*>(reinterpret_cast<char*>(ws) + kBwdHeader);
     L.gbarE = L.map.interp ? reinterpret_cast<float*>(reinterpret_cast<char*>(ws) + kBwdHeader) : nullptr;
     L.qsumd = reinterpret_cast<double*>(reinterpret_cast<char*>(ws) + 32);
+    L.tipd = reinterpret_cast<double*>(reinterpret_cast<char*>(ws) + 64);
     pp_status st = cuda_status(cudaMemsetAsync(reinterpret_cast<char*>(ws) + kBwdHeader, 0, adj_bytes, s),
                                (who + " memset").c_str());
     if (st != PP_OK) return st;

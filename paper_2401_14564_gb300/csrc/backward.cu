@@ -21,16 +21,21 @@
 //         and Cq_i = sum_g Gbar_g . Phi (the quadrupole force per unit
 //         k_e q_i Qzz / 2); eps via e_iPP = sqrt(e_i e_PP).
 // No relaxation iterate is stored or replayed: only the saved p*.
-#include "interp.cuh"
+#include "ff_tile.cuh"
 
 namespace pp {
 namespace {
 
 constexpr int kAdjThreads = 128;
+// Resident CTAs per SM of K4, which waits on its gathers: 6 at 80 registers (flake60, whole adjoint: 5 at 93
+// registers 262 us, 6: 253, 7: 255, 8: 268; launched as one wave, where 8 CTAs per SM at 93 registers ran
+// as 1.6).
+constexpr int kAdjCtas = 6;
 constexpr int kFFBThreads = 64;
 constexpr int kFFBNodes = 512;  // grid nodes staged per K5 CTA
 
-__device__ __forceinline__ float warp_sum(float v) {
+template <class T>
+__device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
@@ -41,9 +46,10 @@ __global__ void init_kernel(const BwdLaunch P) {
     if (t == 0) {
         P.slab[0] = 0x7fffffff;
         P.slab[1] = -1;
+        P.slab[2] = 0;
         P.gtip[0] = P.gtip[1] = P.gtip[2] = P.gtip[3] = P.gtip[4] = 0.f;
-        P.qsum[0] = P.qsum[1] = 0.f;
         P.qsumd[0] = P.qsumd[1] = 0.0;
+        P.tipd[0] = P.tipd[1] = P.tipd[2] = 0.0;
     }
     for (int a = t; a < P.n; a += gridDim.x * blockDim.x) {
         P.gx[a] = 0.f; P.gy[a] = 0.f; P.gz[a] = 0.f;
@@ -86,8 +92,8 @@ __device__ __forceinline__ float df_transpose(const BwdLaunch& P, int k, int pix
 // adjoint is one scalar per node, Ebar_g = sum lambda . grad w_g(p*) over the 64 stencil nodes
 // (F_S = -sum_g E_g grad w_g).
 template <int LAYOUT, int M, bool kTri>
-__global__ void __launch_bounds__(kAdjThreads) relax_adjoint_kernel(const BwdLaunch P) {
-    __shared__ float sred[3][kAdjThreads / 32];
+__global__ void __launch_bounds__(kAdjThreads, kTri ? 1 : kAdjCtas) relax_adjoint_kernel(const BwdLaunch P) {
+    __shared__ double sred[3][kAdjThreads / 32];
     __shared__ int sk[2][kAdjThreads / 32];
     const int npix = P.snx * P.sny;
     const int64_t total = (int64_t)npix * P.snz;
@@ -206,30 +212,29 @@ __global__ void __launch_bounds__(kAdjThreads) relax_adjoint_kernel(const BwdLau
         }
     }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    gkx = warp_sum(gkx);
-    gky = warp_sum(gky);
-    gkR = warp_sum(gkR);
+    // (the tip sums cancel over the image: beyond a thread's own points they are summed in FP64)
+    double dkx = warp_sum((double)gkx), dky = warp_sum((double)gky), dkR = warp_sum((double)gkR);
     kmin = __reduce_min_sync(0xffffffffu, kmin);
     kmax = __reduce_max_sync(0xffffffffu, kmax);
     if (lane == 0) {
-        sred[0][warp] = gkx;
-        sred[1][warp] = gky;
-        sred[2][warp] = gkR;
+        sred[0][warp] = dkx;
+        sred[1][warp] = dky;
+        sred[2][warp] = dkR;
         sk[0][warp] = kmin;
         sk[1][warp] = kmax;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int w = 1; w < kAdjThreads / 32; ++w) {
-            gkx += sred[0][w];
-            gky += sred[1][w];
-            gkR += sred[2][w];
+            dkx += sred[0][w];
+            dky += sred[1][w];
+            dkR += sred[2][w];
             kmin = min(kmin, sk[0][w]);
             kmax = max(kmax, sk[1][w]);
         }
-        if (gkx != 0.f) atomicAdd(P.gtip + 0, gkx * P.nm);
-        if (gky != 0.f) atomicAdd(P.gtip + 1, gky * P.nm);
-        if (gkR != 0.f) atomicAdd(P.gtip + 2, gkR * P.nm);
+        if (dkx != 0.0) atomicAdd(P.tipd + 0, dkx);
+        if (dky != 0.0) atomicAdd(P.tipd + 1, dky);
+        if (dkR != 0.0) atomicAdd(P.tipd + 2, dkR);
         if (kmax >= 0) {
             atomicMin(P.slab + 0, kmin);
             atomicMax(P.slab + 1, kmax);
@@ -246,6 +251,124 @@ __global__ void __launch_bounds__(kAdjThreads) relax_adjoint_kernel(const BwdLau
 // test, the rsqrt and the minimum image stay per node).
 __device__ __forceinline__ float2 sel2(bool c0, bool c1, float2 a, float2 b) {
     return make_float2(c0 ? a.x : b.x, c1 ? a.y : b.y);
+}
+
+// One atom's constants and derivative sums (packed over the two nodes of a pair).
+struct BwdAtom {
+    float2 AX, AY, AZ, RR2, EIJ, QQ, E12, E12R;
+    float rmin2, kqq;
+    float2 GPX, GPY, GPZ, GR, GE, CC, CQ;
+
+    // position (x, y, z), R_i + R_PP, e_iPP, kQ q, k_e Qzz q / 2
+    __device__ __forceinline__ void set(float x, float y, float z, float Rij, float eij, float qq, float core_frac,
+                                        float kq2) {
+        rmin2 = (core_frac * Rij) * (core_frac * Rij);
+        kqq = kq2;
+        AX = make_float2(x, x); AY = make_float2(y, y); AZ = make_float2(z, z);
+        RR2 = make_float2(Rij * Rij, Rij * Rij); EIJ = make_float2(eij, eij); QQ = make_float2(qq, qq);
+        E12 = make_float2(12.f * eij, 12.f * eij); E12R = make_float2(12.f * eij / Rij, 12.f * eij / Rij);
+        GPX = GPY = GPZ = GR = GE = CC = CQ = make_float2(0.f, 0.f);
+    }
+};
+
+struct BwdConst {
+    float core_frac, Lx, Ly, invLx, invLy, rc2, irc2;
+};
+
+// Adds the derivatives of the pair terms of the node pair A = (x0, x1, y0, y1), B = (z0, z1, gx0, gx1),
+// G = (gy0, gy1, gz0, gz1) to the atom's sums.  kSmooth as in ff_core.cuh: no node inside the floor, and
+// with kCutoff all within coul_rc or all beyond.  `live`: the warp's lanes with an atom.
+template <bool kMinImage, bool kCutoff, bool kQuad, Smooth kSmooth>
+__device__ __forceinline__ void bwd_pair(BwdAtom& a, const BwdConst& c, float4 A, float4 B, float4 G, unsigned live) {
+    const float2 TWELVE = make_float2(12.f, 12.f), EIGHT = make_float2(8.f, 8.f), M14 = make_float2(-14.f, -14.f);
+    const float2 M6 = make_float2(-6.f, -6.f), M3 = make_float2(-3.f, -3.f), CF = make_float2(c.core_frac, c.core_frac);
+    float2 DX = f2sub(make_float2(A.x, A.y), a.AX), DY = f2sub(make_float2(A.z, A.w), a.AY);
+    const float2 DZ = f2sub(make_float2(B.x, B.y), a.AZ);
+    const float2 GX = make_float2(B.z, B.w), GY = make_float2(G.x, G.y), GZ = make_float2(G.z, G.w);
+    if (kMinImage) {
+        DX.x = fmaf(-c.Lx, rintf(DX.x * c.invLx), DX.x);
+        DX.y = fmaf(-c.Lx, rintf(DX.y * c.invLx), DX.y);
+        DY.x = fmaf(-c.Ly, rintf(DY.x * c.invLy), DY.x);
+        DY.y = fmaf(-c.Ly, rintf(DY.y * c.invLy), DY.y);
+    }
+    const float2 R2raw = f2fma(DX, DX, f2fma(DY, DY, f2mul(DZ, DZ)));
+    constexpr bool kAll = kSmooth != Smooth::kNo;
+    const bool c0 = !kAll && R2raw.x < a.rmin2, c1 = !kAll && R2raw.y < a.rmin2;  // core floor per node
+    const float2 R2v = make_float2(c0 ? a.rmin2 : R2raw.x, c1 ? a.rmin2 : R2raw.y);
+    // kFar: both nodes lie at or beyond coul_rc from every live lane's atom (a warp vote), so
+    // each in-range test below is false and is taken as such: the cut point-charge and
+    // quadrupole terms become the zeros they select, and their arithmetic drops out
+    auto pair = [&](auto far_t) {
+        constexpr bool kFar = decltype(far_t)::value;
+        auto in_rc = [&](float r2v) { return kSmooth == Smooth::kInside || (!kFar && r2v < c.rc2); };
+        const float2 RS = make_float2(rsqrtf(R2v.x), rsqrtf(R2v.y));
+        const float2 IR2 = f2mul(RS, RS);
+        const float2 U = f2mul(a.RR2, IR2);
+        const float2 S6 = f2mul(f2mul(U, U), U);
+        const float2 S12 = f2mul(S6, S6);
+        const float2 SLJ = f2mul(f2mul(TWELVE, f2sub(S12, S6)), IR2);                 // LJ S per unit e_iPP
+        const float2 DSLJDR = f2mul(f2mul(a.E12, f2fma(EIGHT, S6, f2mul(M14, S12))), f2mul(IR2, RS));
+        const float2 DSLJDRR = f2mul(f2mul(a.E12R, f2fma(TWELVE, S12, f2mul(M6, S6))), IR2);
+        float2 Cv, DC;
+        if (kCutoff) {
+            const bool i0 = in_rc(R2v.x), i1 = in_rc(R2v.y);
+            const float2 z = make_float2(0.f, 0.f);
+            Cv = sel2(i0, i1, f2mul(RS, f2sub(IR2, make_float2(c.irc2, c.irc2))), z);     // 1/r^3 - 1/(r rc^2)
+            DC = sel2(i0, i1, f2mul(IR2, f2fma(M3, IR2, make_float2(c.irc2, c.irc2))), z);  // -3/r^4 + 1/(r^2 rc^2)
+        } else {
+            Cv = f2mul(RS, IR2);
+            DC = f2mul(M3, f2mul(IR2, IR2));
+        }
+        const float2 S = f2fma(a.EIJ, SLJ, f2mul(a.QQ, Cv));
+        const float2 DSDR = f2fma(a.QQ, DC, DSLJDR);
+        const float2 AD = f2fma(GX, DX, f2fma(GY, DY, f2mul(GZ, DZ)));
+        const float2 RAD = sel2(c0, c1, make_float2(0.f, 0.f), f2mul(f2mul(DSDR, AD), RS));  // dS/dr (a.delta)/r
+        a.GPX = f2sub(a.GPX, f2fma(S, GX, f2mul(RAD, DX)));
+        a.GPY = f2sub(a.GPY, f2fma(S, GY, f2mul(RAD, DY)));
+        a.GPZ = f2sub(a.GPZ, f2fma(S, GZ, f2mul(RAD, DZ)));
+        a.GR = f2fma(AD, sel2(c0, c1, f2fma(DSDR, CF, DSLJDRR), DSLJDRR), a.GR);
+        a.GE = f2fma(AD, SLJ, a.GE);
+        a.CC = f2fma(AD, Cv, a.CC);
+        if (kQuad) {
+            // Phi = A delta - 6 dz r^-5 z_hat, A = 15 dz^2 r^-7 - 3 r^-5 (cut off at rc)
+            const bool q0 = !kCutoff || in_rc(R2v.x), q1 = !kCutoff || in_rc(R2v.y);
+            const float2 z = make_float2(0.f, 0.f);
+            const float2 IR5 = f2mul(f2mul(IR2, IR2), RS), IR7 = f2mul(IR5, IR2), DZ2 = f2mul(DZ, DZ);
+            const float2 Aq = sel2(q0, q1, f2fma(f2mul(make_float2(15.f, 15.f), DZ2), IR7, f2mul(M3, IR5)), z);
+            const float2 A6 = sel2(q0, q1, f2mul(make_float2(6.f, 6.f), f2mul(DZ, IR5)), z);
+            a.CQ = f2fma(Aq, AD, f2fma(f2mul(make_float2(-1.f, -1.f), A6), GZ, a.CQ));  // a . Phi
+            // a . dPhi/dr at fixed delta, and the z row of a^T dPhi/d delta at fixed r
+            const float2 W = sel2(q0, q1,
+                                  f2mul(RS, f2fma(f2fma(f2mul(make_float2(-105.f, -105.f), DZ2), IR7,
+                                                        f2mul(make_float2(15.f, 15.f), IR5)),
+                                                  AD, f2mul(f2mul(make_float2(30.f, 30.f), DZ), f2mul(IR5, GZ)))),
+                                  z);
+            const float2 ZROW = sel2(q0, q1,
+                                     f2fma(f2mul(make_float2(30.f, 30.f), f2mul(DZ, IR7)), AD,
+                                           f2mul(f2mul(M6, IR5), GZ)),
+                                     z);
+            const float2 WR = sel2(c0, c1, z, f2mul(W, RS));  // r follows delta unless floored
+            const float2 MK = make_float2(-a.kqq, -a.kqq);
+            a.GPX = f2fma(MK, f2fma(Aq, GX, f2mul(WR, DX)), a.GPX);
+            a.GPY = f2fma(MK, f2fma(Aq, GY, f2mul(WR, DY)), a.GPY);
+            a.GPZ = f2fma(MK, f2fma(Aq, GZ, f2fma(WR, DZ, ZROW)), a.GPZ);
+            a.GR = sel2(c0, c1, f2fma(make_float2(a.kqq * c.core_frac, a.kqq * c.core_frac), W, a.GR), a.GR);
+        }
+    };
+    if (kAll) pair(std::integral_constant<bool, kCutoff && kSmooth == Smooth::kBeyond>{});
+    else if (kCutoff && __all_sync(live, R2v.x >= c.rc2 && R2v.y >= c.rc2)) pair(std::true_type{});
+    else pair(std::false_type{});
+}
+
+template <bool kMinImage, bool kCutoff>
+__device__ __forceinline__ BwdConst bwd_const(const BwdLaunch& P) {
+    BwdConst c;
+    c.core_frac = P.core_frac;
+    c.Lx = P.Lx; c.Ly = P.Ly;
+    c.invLx = kMinImage ? 1.f / P.Lx : 0.f; c.invLy = kMinImage ? 1.f / P.Ly : 0.f;
+    c.rc2 = kCutoff ? P.coul_rc * P.coul_rc : 0.f;
+    c.irc2 = kCutoff ? 1.f / c.rc2 : 0.f;
+    return c;
 }
 
 template <bool kMinImage, bool kCutoff, bool kQuad>
@@ -310,11 +433,7 @@ __global__ void __launch_bounds__(kFFBThreads) ff_backward_kernel(const BwdLaunc
     }
     __syncthreads();
     const int npairs = (cnt + 1) >> 1;
-    const float rc2 = kCutoff ? P.coul_rc * P.coul_rc : 0.f;
-    const float irc2 = kCutoff ? 1.f / rc2 : 0.f;
-    const float invLx = kMinImage ? 1.f / P.Lx : 0.f, invLy = kMinImage ? 1.f / P.Ly : 0.f;
-    const float2 TWELVE = make_float2(12.f, 12.f), EIGHT = make_float2(8.f, 8.f), M14 = make_float2(-14.f, -14.f);
-    const float2 M6 = make_float2(-6.f, -6.f), M3 = make_float2(-3.f, -3.f), CF = make_float2(P.core_frac, P.core_frac);
+    const BwdConst cst = bwd_const<kMinImage, kCutoff>(P);
     float qC = 0.f, qCq = 0.f;  // this thread's q_i C_i and q_i Cq_i (tip quadrupole only)
     for (int a0 = 0; a0 < P.n; a0 += kFFBThreads) {
         const int ia = a0 + threadIdx.x;
@@ -324,91 +443,12 @@ __global__ void __launch_bounds__(kFFBThreads) ff_backward_kernel(const BwdLaunc
         const float Rij = P.aR[ia] + P.R_pp;
         const float eij = sqrtf(P.aeps[ia] * P.eps_pp);
         const float qq = P.kQ * P.aq[ia];
-        const float rmin2 = (P.core_frac * Rij) * (P.core_frac * Rij);
-        const float kqq = kQuad ? P.kQzz * P.aq[ia] : 0.f;
-        const float2 AX = make_float2(ax, ax), AY = make_float2(ay, ay), AZ = make_float2(azz, azz);
-        const float2 RR2 = make_float2(Rij * Rij, Rij * Rij), EIJ = make_float2(eij, eij), QQ = make_float2(qq, qq);
-        const float2 E12 = make_float2(12.f * eij, 12.f * eij), E12R = make_float2(12.f * eij / Rij, 12.f * eij / Rij);
-        float2 GPX = make_float2(0.f, 0.f), GPY = GPX, GPZ = GPX, GR = GPX, GE = GPX, CC = GPX, CQ = GPX;
-        for (int pr = 0; pr < npairs; ++pr) {
-            const float4 A = sxy[pr], B = szg[pr], G = sgg[pr];
-            float2 DX = f2sub(make_float2(A.x, A.y), AX), DY = f2sub(make_float2(A.z, A.w), AY);
-            const float2 DZ = f2sub(make_float2(B.x, B.y), AZ);
-            const float2 GX = make_float2(B.z, B.w), GY = make_float2(G.x, G.y), GZ = make_float2(G.z, G.w);
-            if (kMinImage) {
-                DX.x = fmaf(-P.Lx, rintf(DX.x * invLx), DX.x);
-                DX.y = fmaf(-P.Lx, rintf(DX.y * invLx), DX.y);
-                DY.x = fmaf(-P.Ly, rintf(DY.x * invLy), DY.x);
-                DY.y = fmaf(-P.Ly, rintf(DY.y * invLy), DY.y);
-            }
-            const float2 R2raw = f2fma(DX, DX, f2fma(DY, DY, f2mul(DZ, DZ)));
-            const bool c0 = R2raw.x < rmin2, c1 = R2raw.y < rmin2;  // core floor per node
-            const float2 R2v = make_float2(c0 ? rmin2 : R2raw.x, c1 ? rmin2 : R2raw.y);
-            // kFar: both nodes lie at or beyond coul_rc from every live lane's atom (a warp vote), so
-            // each in-range test below is false and is taken as such: the cut point-charge and
-            // quadrupole terms become the zeros they select, and their arithmetic drops out
-            auto pair = [&](auto far_t) {
-                constexpr bool kFar = decltype(far_t)::value;
-                auto in_rc = [&](float r2v) { return !kFar && r2v < rc2; };
-                const float2 RS = make_float2(rsqrtf(R2v.x), rsqrtf(R2v.y));
-                const float2 IR2 = f2mul(RS, RS);
-                const float2 U = f2mul(RR2, IR2);
-                const float2 S6 = f2mul(f2mul(U, U), U);
-                const float2 S12 = f2mul(S6, S6);
-                const float2 SLJ = f2mul(f2mul(TWELVE, f2sub(S12, S6)), IR2);                 // LJ S per unit e_iPP
-                const float2 DSLJDR = f2mul(f2mul(E12, f2fma(EIGHT, S6, f2mul(M14, S12))), f2mul(IR2, RS));
-                const float2 DSLJDRR = f2mul(f2mul(E12R, f2fma(TWELVE, S12, f2mul(M6, S6))), IR2);
-                float2 Cv, DC;
-                if (kCutoff) {
-                    const bool i0 = in_rc(R2v.x), i1 = in_rc(R2v.y);
-                    const float2 z = make_float2(0.f, 0.f);
-                    Cv = sel2(i0, i1, f2mul(RS, f2sub(IR2, make_float2(irc2, irc2))), z);     // 1/r^3 - 1/(r rc^2)
-                    DC = sel2(i0, i1, f2mul(IR2, f2fma(M3, IR2, make_float2(irc2, irc2))), z);  // -3/r^4 + 1/(r^2 rc^2)
-                } else {
-                    Cv = f2mul(RS, IR2);
-                    DC = f2mul(M3, f2mul(IR2, IR2));
-                }
-                const float2 S = f2fma(EIJ, SLJ, f2mul(QQ, Cv));
-                const float2 DSDR = f2fma(QQ, DC, DSLJDR);
-                const float2 AD = f2fma(GX, DX, f2fma(GY, DY, f2mul(GZ, DZ)));
-                const float2 RAD = sel2(c0, c1, make_float2(0.f, 0.f), f2mul(f2mul(DSDR, AD), RS));  // dS/dr (a.delta)/r
-                GPX = f2sub(GPX, f2fma(S, GX, f2mul(RAD, DX)));
-                GPY = f2sub(GPY, f2fma(S, GY, f2mul(RAD, DY)));
-                GPZ = f2sub(GPZ, f2fma(S, GZ, f2mul(RAD, DZ)));
-                GR = f2fma(AD, sel2(c0, c1, f2fma(DSDR, CF, DSLJDRR), DSLJDRR), GR);
-                GE = f2fma(AD, SLJ, GE);
-                CC = f2fma(AD, Cv, CC);
-                if (kQuad) {
-                    // Phi = A delta - 6 dz r^-5 z_hat, A = 15 dz^2 r^-7 - 3 r^-5 (cut off at rc)
-                    const bool q0 = !kCutoff || in_rc(R2v.x), q1 = !kCutoff || in_rc(R2v.y);
-                    const float2 z = make_float2(0.f, 0.f);
-                    const float2 IR5 = f2mul(f2mul(IR2, IR2), RS), IR7 = f2mul(IR5, IR2), DZ2 = f2mul(DZ, DZ);
-                    const float2 Aq = sel2(q0, q1, f2fma(f2mul(make_float2(15.f, 15.f), DZ2), IR7, f2mul(M3, IR5)), z);
-                    const float2 A6 = sel2(q0, q1, f2mul(make_float2(6.f, 6.f), f2mul(DZ, IR5)), z);
-                    CQ = f2fma(Aq, AD, f2fma(f2mul(make_float2(-1.f, -1.f), A6), GZ, CQ));  // a . Phi
-                    // a . dPhi/dr at fixed delta, and the z row of a^T dPhi/d delta at fixed r
-                    const float2 W = sel2(q0, q1,
-                                          f2mul(RS, f2fma(f2fma(f2mul(make_float2(-105.f, -105.f), DZ2), IR7,
-                                                                f2mul(make_float2(15.f, 15.f), IR5)),
-                                                          AD, f2mul(f2mul(make_float2(30.f, 30.f), DZ), f2mul(IR5, GZ)))),
-                                          z);
-                    const float2 ZROW = sel2(q0, q1,
-                                             f2fma(f2mul(make_float2(30.f, 30.f), f2mul(DZ, IR7)), AD,
-                                                   f2mul(f2mul(M6, IR5), GZ)),
-                                             z);
-                    const float2 WR = sel2(c0, c1, z, f2mul(W, RS));  // r follows delta unless floored
-                    const float2 MK = make_float2(-kqq, -kqq);
-                    GPX = f2fma(MK, f2fma(Aq, GX, f2mul(WR, DX)), GPX);
-                    GPY = f2fma(MK, f2fma(Aq, GY, f2mul(WR, DY)), GPY);
-                    GPZ = f2fma(MK, f2fma(Aq, GZ, f2fma(WR, DZ, ZROW)), GPZ);
-                    GR = sel2(c0, c1, f2fma(make_float2(kqq * P.core_frac, kqq * P.core_frac), W, GR), GR);
-                }
-            };
-            if (kCutoff && __all_sync(live, R2v.x >= rc2 && R2v.y >= rc2)) pair(std::true_type{});
-            else pair(std::false_type{});
-        }
-        const float gpx = GPX.x + GPX.y, gpy = GPY.x + GPY.y, gpz = GPZ.x + GPZ.y;
-        const float gRr = GR.x + GR.y, ge = GE.x + GE.y, C = CC.x + CC.y, Cq = CQ.x + CQ.y;
+        BwdAtom at;
+        at.set(ax, ay, azz, Rij, eij, qq, P.core_frac, kQuad ? P.kQzz * P.aq[ia] : 0.f);
+        for (int pr = 0; pr < npairs; ++pr)
+            bwd_pair<kMinImage, kCutoff, kQuad, Smooth::kNo>(at, cst, sxy[pr], szg[pr], sgg[pr], live);
+        const float gpx = at.GPX.x + at.GPX.y, gpy = at.GPY.x + at.GPY.y, gpz = at.GPZ.x + at.GPZ.y;
+        const float gRr = at.GR.x + at.GR.y, ge = at.GE.x + at.GE.y, C = at.CC.x + at.CC.y, Cq = at.CQ.x + at.CQ.y;
         atomicAdd(P.gx + ia, gpx);
         atomicAdd(P.gy + ia, gpy);
         atomicAdd(P.gz + ia, gpz);
@@ -426,10 +466,319 @@ __global__ void __launch_bounds__(kFFBThreads) ff_backward_kernel(const BwdLaunc
         qC = warp_sum(qC);
         qCq = warp_sum(qCq);
         if ((threadIdx.x & 31) == 0) {
-            atomicAdd(P.qsum + 0, qC);
-            atomicAdd(P.qsum + 1, qCq);
+            atomicAdd(P.qsumd + 0, (double)qC);
+            atomicAdd(P.qsumd + 1, (double)qCq);
         }
     }
+}
+
+// K5 by tiles (the grids K1 assembles by tiles): the transpose of ff_tile.cuh's interpolation.  The node
+// adjoints of a 16x16x16-node tile are carried to its 8x8x8 Chebyshev points (along z, y, x), where the far
+// atoms' pair derivatives are contracted with 512 points instead of up to 4096 nodes; near atoms are
+// contracted with the nodes that hold an adjoint.  The derivatives are one order steeper than the terms:
+// worst relative error of a far pair 4e-7 at 10 half extents, for atoms that are the smaller part of
+// every gradient.  Atoms and node pairs share a CTA's 256 threads: atom slot tid mod 2^s, 2^s >= the list's
+// length, and the 256 / 2^s threads of a slot take the node pairs in turn, so a list of 5 near atoms and one
+// of 200 far ones both fill the warps.  A tile over a molecule has every atom near and one beside it none,
+// so a tile's near work is four CTAs' (four layers each) and its far work a fifth's.
+// The gradients cancel over the image, so their sums over the CTAs go to up to 32 replicas (in the adjoint
+// grid's unused fourth components) that finalize_tile_kernel adds in FP64: thousands of FP32 additions to one word
+// had cost 1-3e-6 relative in R and eps.
+// Bound by the FP32 pipes like the direct contraction.  Measured (the whole adjoint): 60-atom flake,
+// 256x256x40 points, 417 -> 253 us; 40-atom molecule with the tip's quadrupole, 128x128x20 points, 146 -> 105 us (with
+// one CTA a tile 173: its busiest SM had 3.1 times the average's work); 300 atoms 906 -> 360 us.
+struct BwdTileShared {
+    float4 a[6 * 256];        // sums along z [component][z point][column]; then point pairs and node pairs
+    float b[192 * 17];        // sums along y [component][z point][y point][node along x], rows of 16 + 1 pad;
+                              // then atom records, two float4 each
+    int count[kTileThreads / 32];
+    int nodes;
+};
+static_assert(sizeof(float) * 192 * 17 >= 2 * sizeof(float4) * kTileChunk, "atom records fit");
+
+constexpr int kBwdLayers = 4;                          // layers of a near part
+constexpr int kBwdParts = kTileN / kBwdLayers + 1;     // near parts, then the far part
+
+template <bool kMinImage, bool kCutoff, bool kQuad>
+__global__ void __launch_bounds__(kTileThreads, 2) ff_backward_tile_kernel(const BwdLaunch P) {
+    __shared__ BwdTileShared S;
+    const int klo = P.slab[0], khi = P.slab[1];
+    const int i0 = blockIdx.x * kTileN, j0 = blockIdx.y * kTileN;
+    const int k0 = (blockIdx.z / kBwdParts) * kTileN, part = blockIdx.z % kBwdParts;
+    const bool far_part = part == kBwdParts - 1;
+    const int ka = far_part ? 0 : part * kBwdLayers, kb = far_part ? kTileN : ka + kBwdLayers;  // this CTA's layers
+    if (k0 + ka > khi || k0 + kb - 1 < klo) return;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const float half = 0.5f * (kTileN - 1);
+    // this thread's column of nodes: adjoints of the layers K4 touched (0 elsewhere)
+    const int ci = tid & (kTileN - 1), cj = tid >> 4;
+    const bool inside = i0 + ci < P.map.nx && j0 + cj < P.map.ny;
+    const int base_xy = inside ? axis_off(P.map.ax, i0 + ci) + axis_off(P.map.ay, j0 + cj) : 0;
+    auto adjoint = [&](int k) {
+        if (!inside || k0 + k < klo || k0 + k > khi) return make_float4(0.f, 0.f, 0.f, 0.f);
+        return P.gbar[checked(base_xy + axis_off(P.map.az, k0 + k), P.map.stored_nodes, kChkGridRead)];
+    };
+    // the far part's sums along z at the points; the near parts' own layers
+    float z[3][kTileP];
+    bool any = false;
+    if (far_part) {
+#pragma unroll
+        for (int m = 0; m < kTileP; ++m) z[0][m] = z[1][m] = z[2][m] = 0.f;
+#pragma unroll 4
+        for (int k = 0; k < kTileN; ++k) {
+            const float4 g = adjoint(k);
+            any |= g.x != 0.f || g.y != 0.f || g.z != 0.f;
+#pragma unroll
+            for (int m = 0; m < kTileP; ++m) {
+                const float w = c_tile.l[k][m];
+                z[0][m] = fmaf(w, g.x, z[0][m]);
+                z[1][m] = fmaf(w, g.y, z[1][m]);
+                z[2][m] = fmaf(w, g.z, z[2][m]);
+            }
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < kBwdLayers; ++k) {
+            const float4 g = adjoint(ka + k);
+            any |= g.x != 0.f || g.y != 0.f || g.z != 0.f;
+            z[0][k] = g.x;
+            z[1][k] = g.y;
+            z[2][k] = g.z;
+        }
+    }
+    if (!__syncthreads_or(any)) return;
+
+    const float2 cx = tile_centre(P.x0, i0, P.dx), cy = tile_centre(P.y0, j0, P.dy), cz = tile_centre(P.z0, k0, P.dz);
+    const float hx = __fmul_rn(half, P.dx), hy = __fmul_rn(half, P.dy), hz = __fmul_rn(half, P.dz);
+    const float hmax = fmaxf(hx, fmaxf(hy, hz));
+    const FFConst fc = ff_const(P.R_pp, P.eps_pp, P.kQ, P.core_frac, P.Lx, P.Ly, kCutoff ? P.coul_rc : 0.f, 0.f);
+    const BwdConst cst = bwd_const<kMinImage, kCutoff>(P);
+    float4* const pt = S.a;          // point pairs: xy, zg, gg (bwd_pair's A, B, G), 256 of each
+    float4* const nd = S.a + 768;    // node pairs, likewise
+    float4* const rec = reinterpret_cast<float4*>(S.b);
+
+    // the adjoints at the tile's points, as 256 pairs along x
+    auto to_points = [&]() {
+        float* const Z = reinterpret_cast<float*>(S.a);
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int m = 0; m < kTileP; ++m) Z[(c * kTileP + m) * 256 + tid] = z[c][m];
+        __syncthreads();
+        for (int row = tid >> 4; row < 3 * kTileP; row += 16) {
+            const int i = tid & 15;
+            float y[kTileP];
+#pragma unroll
+            for (int m = 0; m < kTileP; ++m) y[m] = 0.f;
+#pragma unroll
+            for (int j = 0; j < kTileN; ++j) {
+                const float v = Z[row * 256 + j * kTileN + i];
+#pragma unroll
+                for (int m = 0; m < kTileP; ++m) y[m] = fmaf(c_tile.l[j][m], v, y[m]);
+            }
+#pragma unroll
+            for (int m = 0; m < kTileP; ++m) S.b[(row * kTileP + m) * 17 + i] = y[m];
+        }
+        __syncthreads();
+        if (tid < 192) {
+            float x[kTileP];
+#pragma unroll
+            for (int m = 0; m < kTileP; ++m) x[m] = 0.f;
+#pragma unroll
+            for (int i = 0; i < kTileN; ++i) {
+                const float v = S.b[tid * 17 + i];
+#pragma unroll
+                for (int m = 0; m < kTileP; ++m) x[m] = fmaf(c_tile.l[i][m], v, x[m]);
+            }
+            const int c = tid >> 6, row = tid & 63;  // row = 8 z point + y point
+            float* const out = reinterpret_cast<float*>(c == 0 ? pt + 256 : pt + 512) + (c == 1 ? 0 : 2);
+#pragma unroll
+            for (int m = 0; m < kTileP; ++m) out[(row * 4 + (m >> 1)) * 4 + (m & 1)] = x[m];
+        }
+        const int px = 2 * (tid & 3), row = tid >> 2;
+        const float y = __fmul_rn(g_tile.at[row & 7], P.dy), zz = __fmul_rn(g_tile.at[row >> 3], P.dz);
+        pt[tid] = make_float4(__fmul_rn(g_tile.at[px], P.dx), __fmul_rn(g_tile.at[px + 1], P.dx), y, y);
+        float2* const zg = reinterpret_cast<float2*>(pt + 256 + tid);
+        zg[0] = make_float2(zz, zz);
+        __syncthreads();
+    };
+
+    const int first_sum = 7 * (int)((blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)) % P.replicas);
+    BwdAtom at;
+    int slots = 1, slot = 0, sub = 0, nsub = kTileThreads, ia = -1;
+    // takes the records first .. first + cnt - 1 as this CTA's atoms
+    auto take = [&](int first, int cnt) {
+        slots = 1;
+        while (slots < cnt) slots <<= 1;
+        slot = tid & (slots - 1);
+        sub = tid / slots;
+        nsub = kTileThreads / slots;
+        const int r = 2 * (first + (slot < cnt ? slot : 0));
+        const float4 u = rec[r], v = rec[r + 1];
+        at.set(u.x, u.y, u.z, u.w, v.x, P.kQ * v.y, P.core_frac, kQuad ? P.kQzz * v.y : 0.f);
+        ia = slot < cnt ? __float_as_int(v.z) : -1;
+    };
+    // adds this CTA's sums to its replica
+    auto flush = [&]() {
+        float v[7] = {at.GPX.x + at.GPX.y, at.GPY.x + at.GPY.y, at.GPZ.x + at.GPZ.y, at.GR.x + at.GR.y,
+                      at.GE.x + at.GE.y, at.CC.x + at.CC.y, at.CQ.x + at.CQ.y};
+        for (int o = slots; o < 32; o <<= 1) {
+#pragma unroll
+            for (int q = 0; q < (kQuad ? 7 : 6); ++q) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+        }
+        if (ia < 0 || (slots < 32 && lane >= slots)) return;
+#pragma unroll
+        for (int q = 0; q < (kQuad ? 7 : 6); ++q)
+            atomicAdd(&P.gbar[checked((first_sum + q) * P.n + ia, P.map.stored_nodes, kChkGridWrite)].w, v[q]);
+    };
+
+    bool have_points = false;
+    for (int base = 0; base < P.n; base += kTileChunk) {
+        const int a = base + tid;
+        const bool live = a < P.n;
+        float rx = 0.f, ry = 0.f, rz = 0.f, Rij = 1.f, eij = 0.f, q = 0.f;
+        bool far = false, charged = true;
+        if (live) {
+            rx = __fsub_rn(__fsub_rn(P.ax[a], cx.x), cx.y);
+            ry = __fsub_rn(__fsub_rn(P.ay[a], cy.x), cy.y);
+            rz = __fsub_rn(__fsub_rn(P.az[a], cz.x), cz.y);
+            if (kMinImage) {
+                rx = wrap_image(rx, fc.Lx, fc.invLx);
+                ry = wrap_image(ry, fc.Ly, fc.invLy);
+            }
+            const float R = P.aR[a], eps = P.aeps[a];
+            q = P.aq[a];
+            Rij = R + P.R_pp;
+            eij = sqrtf(eps * P.eps_pp);
+            // (the charge's derivative is wanted of neutral atoms too: every atom counts as charged)
+            far = tile_far<kMinImage, kCutoff>(fc, rx, ry, rz, hx, hy, hz, hmax, R, eps, q == 0.f ? 1.f : q, &charged);
+        }
+        auto stage = [&](int s) {
+            rec[2 * s] = make_float4(rx, ry, rz, Rij);
+            rec[2 * s + 1] = make_float4(eij, q, __int_as_float(a), 0.f);
+        };
+        int n_in = 0, n_out = 0;
+        int s_far = tile_slot(far && charged, S.count, &n_in);
+        if (kCutoff) {
+            const int s = tile_slot(far && !charged, S.count, &n_out);
+            if (!charged) s_far = n_in + s;
+        }
+        if (P.n <= kTileChunk && n_in + n_out < kFarMin) {
+            far = false;
+            n_in = n_out = 0;
+        }
+        if (far_part) {
+            if (n_in + n_out == 0) continue;
+            if (!have_points) to_points();
+            have_points = true;
+            if (far) stage(s_far);
+            __syncthreads();
+            if (n_in > 0) {
+                take(0, n_in);
+                for (int p = sub; p < 256; p += nsub)
+                    bwd_pair<false, kCutoff, kQuad, Smooth::kInside>(at, cst, pt[p], pt[256 + p], pt[512 + p], 0xffffffffu);
+                flush();
+            }
+            if (kCutoff && n_out > 0) {
+                take(n_in, n_out);
+                for (int p = sub; p < 256; p += nsub)
+                    bwd_pair<false, kCutoff, kQuad, Smooth::kBeyond>(at, cst, pt[p], pt[256 + p], pt[512 + p], 0xffffffffu);
+                flush();
+            }
+            continue;
+        }
+        int n_near = 0;
+        const int s_near = tile_slot(live && !far, S.count, &n_near);
+        if (n_near == 0) continue;
+        if (live && !far) stage(s_near);
+        __syncthreads();
+        take(0, n_near);
+        // the nodes with an adjoint, two layers (up to 512 nodes) at a time
+        float* const fxy = reinterpret_cast<float*>(nd);
+        float* const fzg = reinterpret_cast<float*>(nd + 256);
+        float* const fgg = reinterpret_cast<float*>(nd + 512);
+#pragma unroll
+        for (int kk = 0; kk < kBwdLayers; kk += 2) {
+            __syncthreads();
+            if (tid == 0) S.nodes = 0;
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const float gx = z[0][kk + u], gy = z[1][kk + u], gz = z[2][kk + u];
+                const bool keep = gx != 0.f || gy != 0.f || gz != 0.f;
+                const unsigned mask = __ballot_sync(0xffffffffu, keep);
+                int first = 0;
+                if (lane == 0 && mask) first = atomicAdd(&S.nodes, __popc(mask));
+                first = __shfl_sync(0xffffffffu, first, 0);
+                if (keep) {
+                    const int s = first + __popc(mask & ((1u << lane) - 1u)), w = (s >> 1) * 4, l = s & 1;
+                    fxy[w + l] = __fmul_rn((float)ci - half, P.dx);
+                    fxy[w + 2 + l] = __fmul_rn((float)cj - half, P.dy);
+                    fzg[w + l] = __fmul_rn((float)(ka + kk + u) - half, P.dz);
+                    fzg[w + 2 + l] = gx;
+                    fgg[w + l] = gy;
+                    fgg[w + 2 + l] = gz;
+                }
+            }
+            __syncthreads();
+            const int cnt = S.nodes;
+            if (cnt == 0) continue;
+            // whole rounds for every thread (the cutoff's warp votes): pad with the first node, adjoint zero
+            const int pairs = ((cnt + 1) / 2 + nsub - 1) / nsub * nsub;
+            for (int s = cnt + tid; s < 2 * pairs; s += kTileThreads) {
+                const int w = (s >> 1) * 4, l = s & 1;
+                fxy[w + l] = fxy[0];
+                fxy[w + 2 + l] = fxy[2];
+                fzg[w + l] = fzg[0];
+                fzg[w + 2 + l] = fgg[w + l] = fgg[w + 2 + l] = 0.f;
+            }
+            __syncthreads();
+            for (int p = sub; p < pairs; p += nsub)
+                bwd_pair<kMinImage, kCutoff, kQuad, Smooth::kNo>(at, cst, nd[p], nd[256 + p], nd[512 + p], 0xffffffffu);
+        }
+        flush();
+    }
+}
+
+// Gradients from the tile kernel's replicas, a warp per atom.  dL/dq = k_e (Q C + (Qzz/2) Cq),
+// dL/dQ = k_e sum_i q_i C_i and dL/dQzz = (k_e/2) sum_i q_i Cq_i, the sums over replicas and atoms in FP64; the
+// last block writes the tip's.
+__global__ void __launch_bounds__(256) finalize_tile_kernel(const BwdLaunch P) {
+    __shared__ double sum[2][8];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, a = blockIdx.x * 8 + warp;
+    double v[7];
+#pragma unroll
+    for (int q = 0; q < 7; ++q) {
+        v[q] = a < P.n && lane < P.replicas ? (double)P.gbar[(7 * lane + q) * P.n + a].w : 0.0;
+        v[q] = warp_sum(v[q]);
+    }
+    if (lane == 0) {
+        const double q = a < P.n ? (double)P.aq[a] : 0.0;
+        sum[0][warp] = a < P.n ? q * v[5] : 0.0;
+        sum[1][warp] = a < P.n ? q * v[6] : 0.0;
+        if (a < P.n) {
+            const float eij = sqrtf(P.aeps[a] * P.eps_pp);
+            P.gx[a] = (float)v[0];
+            P.gy[a] = (float)v[1];
+            P.gz[a] = (float)v[2];
+            P.gR[a] = (float)v[3];
+            P.geps[a] = eij > 0.f ? (float)(v[4] * (double)P.eps_pp / (2.0 * (double)eij)) : 0.f;
+            P.gq[a] = (float)((double)P.ke * ((double)P.Q * v[5] + 0.5 * (double)P.Qzz * v[6]));
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int t = 0; t < 2; ++t) {
+        double d = 0.0;
+        for (int w = 0; w < 8; ++w) d += sum[t][w];
+        atomicAdd(P.qsumd + t, d);
+    }
+    __threadfence();
+    if (atomicAdd(P.slab + 2, 1) != (int)gridDim.x - 1) return;
+    __threadfence();
+    for (int t = 0; t < 3; ++t) P.gtip[t] = (float)(P.tipd[t] * (double)P.nm);
+    P.gtip[3] = (float)((double)P.ke * atomicAdd(P.qsumd + 0, 0.0));
+    P.gtip[4] = P.Qzz != 0.f ? (float)(0.5 * (double)P.ke * atomicAdd(P.qsumd + 1, 0.0)) : 0.f;
 }
 
 // s + t with the rounding error carried in c (Kahan): the f32x2 instructions are not reassociated.
@@ -612,28 +961,16 @@ __global__ void __launch_bounds__(kFFBThreads) ff_backward_energy_kernel(const B
     }
 }
 
-// Charges and well depths from the accumulated sums; dL/dQ by a block reduction
-// (with a tip quadrupole, or on an energy grid, K5 has already combined the charge
-// terms and summed q_i C_i and q_i Cq_i).
+// Charges and well depths from the accumulated sums; dL/dQ by a block reduction (with a tip quadrupole, or
+// on an energy grid, K5 has already combined the charge terms and summed q_i C_i and q_i Cq_i).
 __global__ void finalize_kernel(const BwdLaunch P) {
-    __shared__ float red[32];
-    if (P.Qzz != 0.f || P.map.interp) {
-        for (int a = threadIdx.x; a < P.n; a += blockDim.x) {
-            P.gq[a] *= P.ke;
-            const float eij = sqrtf(P.aeps[a] * P.eps_pp);
-            P.geps[a] = eij > 0.f ? P.geps[a] * P.eps_pp / (2.f * eij) : 0.f;
-        }
-        if (threadIdx.x == 0) {
-            P.gtip[3] = P.map.interp ? (float)((double)P.ke * P.qsumd[0]) : P.ke * P.qsum[0];
-            P.gtip[4] = P.map.interp ? (float)(0.5 * (double)P.ke * P.qsumd[1]) : 0.5f * P.ke * P.qsum[1];
-        }
-        return;
-    }
-    float acc = 0.f;
+    __shared__ double red[32];
+    const bool combined = P.Qzz != 0.f || P.map.interp;
+    double acc = 0.0;
     for (int a = threadIdx.x; a < P.n; a += blockDim.x) {
         const float C = P.gq[a] * P.ke;  // sum (a.delta) k_e c
-        acc = fmaf(P.aq[a], C, acc);
-        P.gq[a] = P.Q * C;
+        acc += (double)P.aq[a] * (double)C;
+        P.gq[a] = combined ? C : P.Q * C;
         const float eij = sqrtf(P.aeps[a] * P.eps_pp);
         P.geps[a] = eij > 0.f ? P.geps[a] * P.eps_pp / (2.f * eij) : 0.f;
     }
@@ -641,9 +978,12 @@ __global__ void finalize_kernel(const BwdLaunch P) {
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
     if (threadIdx.x < 32) {
-        float v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.f;
-        v = warp_sum(v);
-        if (threadIdx.x == 0) P.gtip[3] = v;
+        const double v = warp_sum(threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0);
+        if (threadIdx.x == 0) {
+            for (int t = 0; t < 3; ++t) P.gtip[t] = (float)(P.tipd[t] * (double)P.nm);
+            P.gtip[3] = combined ? (float)((double)P.ke * P.qsumd[0]) : (float)v;
+            P.gtip[4] = combined ? (float)(0.5 * (double)P.ke * P.qsumd[1]) : 0.f;
+        }
     }
 }
 
@@ -681,18 +1021,34 @@ void launch_adjoint(const BwdLaunch& L, int blocks, cudaStream_t s) {
 
 }  // namespace
 
-cudaError_t launch_backward(const BwdLaunch& L, cudaStream_t s) {
+cudaError_t launch_backward(const BwdLaunch& L0, cudaStream_t s) {
+    BwdLaunch L = L0;
     init_kernel<<<(L.n + 255) / 256 + 1, 256, 0, s>>>(L);
     const int64_t total = (int64_t)L.snx * L.sny * L.snz;
-    // one wave of resident blocks (8 per SM at this register count), grid-stride inside
-    int dev = 0, sms = 148;
+    // one wave of resident blocks, grid-stride inside
+    int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t need = (total + kAdjThreads - 1) / kAdjThreads;
-    const int blocks = (int)(need < 8LL * sms ? (need > 0 ? need : 1) : 8LL * sms);
+    const int64_t need = (total + kAdjThreads - 1) / kAdjThreads, most = (int64_t)kAdjCtas * sms;
+    const int blocks = (int)(need < most ? (need > 0 ? need : 1) : most);
     launch_adjoint(L, blocks, s);
+    const int64_t nodes = (int64_t)L.map.nx * L.map.ny * L.map.nz;
+    const dim3 tiles((L.map.nx + kTileN - 1) / kTileN, (L.map.ny + kTileN - 1) / kTileN,
+                     kBwdParts * ((L.map.nz + kTileN - 1) / kTileN));
+    // by tiles where K1 is, if the replicas fit the adjoint grid and the launch grid the tiles
+    if (!L.map.interp && ff_use_tiles(L.n, L.dx, L.dy, L.dz) && tiles.y <= 65535 && tiles.z <= 65535 &&
+        7 * (int64_t)L.n <= L.map.stored_nodes) {
+        L.replicas = 32;
+        while (7 * (int64_t)L.n * L.replicas > L.map.stored_nodes) L.replicas >>= 1;
+        with_flags(L.min_image != 0, L.coul_rc > 0.f, L.Qzz != 0.f, [&](auto mi, auto cut, auto quad) {
+            ff_backward_tile_kernel<decltype(mi)::value, decltype(cut)::value, decltype(quad)::value>
+                <<<tiles, kTileThreads, 0, s>>>(L);
+            return 0;
+        });
+        finalize_tile_kernel<<<(L.n + 7) / 8, 256, 0, s>>>(L);
+        return cudaGetLastError();
+    }
     if (L.n > 0) {
-        const int64_t nodes = (int64_t)L.map.nx * L.map.ny * L.map.nz;
         const int fb = (int)((nodes + kFFBNodes - 1) / kFFBNodes);
         with_flags(L.min_image != 0, L.coul_rc > 0.f, L.Qzz != 0.f, [&](auto mi, auto cut, auto quad) {
             constexpr bool MI = decltype(mi)::value, CUT = decltype(cut)::value, QUAD = decltype(quad)::value;

@@ -53,6 +53,7 @@ struct Weights {
     float w[kTileN][kTileP];            // w[k][m]: Lagrange basis m at node k; 1 for m = kRef
     float z[kTileN / 2][kTileP][2];     // the same for node pairs: (w[2t][m], w[2t + 1][m])
     float at[kTileP];                   // the points, in nodes from the centre
+    float l[kTileN][kTileP];            // w without the differences: l[k][m] Lagrange basis m at node k
 };
 constexpr Weights make_weights() {
     Weights r{};
@@ -63,6 +64,7 @@ constexpr Weights make_weights() {
             double l = 1.0;
             for (int j = 0; j < kTileP; ++j)
                 if (j != m) l *= (u - kCheb[j]) / (kCheb[m] - kCheb[j]);
+            r.l[k][m] = (float)l;
             if (m == kRef) l = 1.0;
             r.w[k][m] = (float)l;
             r.z[k / 2][m][k & 1] = (float)l;

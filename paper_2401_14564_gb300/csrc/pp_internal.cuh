@@ -218,9 +218,10 @@ struct BwdLaunch {
     float *gx, *gy, *gz, *gq, *gR, *geps, *gtip;
     float4* gbar;   // grid adjoint dL/dF_g (force grids)
     float* gbarE;   // grid adjoint dL/dE_g (energy grids)
-    int* slab;
-    float* qsum;    // {sum_i q_i C_i, sum_i q_i Cq_i} when Qzz != 0 (force grids)
-    double* qsumd;  // the same sums on energy grids
+    int* slab;      // node layers with an adjoint: lowest, highest; blocks of the final sums that are done
+    int replicas;   // of the gradient sums, by tiles (a power of two, at most 32)
+    double* qsumd;  // {sum_i q_i C_i, sum_i q_i Cq_i} when Qzz != 0 and on energy grids
+    double* tipd;   // tip sums {kx, ky, kR}, per eV/A^2
 };
 cudaError_t launch_backward(const BwdLaunch& L, cudaStream_t s);
 // Host side of the adjoint entry points (api.cu): argument checks into a prepared launch, then the

@@ -76,7 +76,10 @@ __device__ __forceinline__ void ff_stage_atom(const FFConst& c, float x, float y
 // all nodes lie within coul_rc of every atom (kInside), or all beyond it or the atoms uncharged
 // (kBeyond), so neither is tested.
 // kRel: coordinates relative to a tile's centre, the atoms' as float pairs whose low parts sit in slots
-// that otherwise repeat a constant (ff_tile.cuh): x in s1.y, y in s3.y, -z in s3.w.
+// that otherwise repeat a constant (ff_tile.cuh): x in s1.y, y in s3.y, and along z in s3.w, -z_lo for near
+// atoms, 2 z z_lo for far ones (Smooth), whose r^2 takes it once per column: (gz - z - z_lo)^2 is (gz - z)^2 +
+// 2 z z_lo but for 2 gz z_lo, 1e-8 of r^2 at 10 half extents (near the tile's edge it is not small: 1e-6 in the
+// energies of an atom 2 A away), so near atoms pay an add per node pair.
 enum class Smooth { kNo, kInside, kBeyond };
 template <int ZP, bool kMinImage, bool kCutoff, bool kQuad, bool kSplit, bool kFloorVote = false,
           Smooth kSmooth = Smooth::kNo, bool kRel = false>
@@ -92,7 +95,7 @@ __device__ __forceinline__ void ff_accumulate_impl(const float4* s0, const float
         const float4 A0 = s0[a], A1 = s1[a], A2 = s2[a], A3 = s3[a];
         float rx = gx - A0.x;
         float ry = gy - A0.y;
-        if (kRel) {  // (an extra add per node pair in z: 3 % of the tile's time, see ff_tile.cuh)
+        if (kRel) {
             rx -= A1.y;
             ry -= A3.y;
         }
@@ -100,20 +103,20 @@ __device__ __forceinline__ void ff_accumulate_impl(const float4* s0, const float
             rx = fmaf(-c.Lx, rintf(rx * c.invLx), rx);
             ry = fmaf(-c.Ly, rintf(ry * c.invLy), ry);
         }
-        const float rxy2 = fmaf(rx, rx, ry * ry);
+        float rxy2 = fmaf(rx, rx, ry * ry);
+        if (kRel && kSmooth != Smooth::kNo) rxy2 = __fadd_rn(rxy2, A3.w);
         const float2 RX = make_float2(rx, rx), RY = make_float2(ry, ry), RXY = make_float2(rxy2, rxy2);
         const float2 NZ = make_float2(A1.x, kRel ? A1.x : A1.y), LA = make_float2(A1.z, A1.w);
         const float2 LB = make_float2(A2.x, A2.y), KQ = make_float2(A2.z, A2.w);
         const float2 EC = make_float2(A3.x, kRel ? A3.x : A3.y), ED = make_float2(A3.z, kRel ? A3.z : A3.w);
-        const float2 NZL = make_float2(A3.w, A3.w);
-        const float2 KQQ = make_float2(A0.w, A0.w);
+        const float2 KQQ = make_float2(A0.w, A0.w), NZL = make_float2(A3.w, A3.w);
         auto body = [&](auto floor_t, auto far_t) {
             constexpr bool kFloor = decltype(floor_t)::value;
             constexpr bool kFar = decltype(far_t)::value;  // every node of every lane beyond coul_rc
             auto in_rc = [&](float r2v) { return kSmooth == Smooth::kInside || (!kFar && r2v < c.rc2); };
 #pragma unroll
             for (int t = 0; t < ZP; ++t) {
-                const float2 rz = kRel ? f2add(f2add(gz[t], NZ), NZL) : f2add(gz[t], NZ);
+                const float2 rz = kRel && kSmooth == Smooth::kNo ? f2add(f2add(gz[t], NZ), NZL) : f2add(gz[t], NZ);
                 float2 r2 = f2fma(rz, rz, RXY);
                 if (kFloor) {
                     r2.x = fmaxf(r2.x, A0.z);

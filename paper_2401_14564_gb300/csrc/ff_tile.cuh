@@ -16,7 +16,7 @@
 // raised to the 8th) is 5e-7 per pair.  Coordinates are taken relative to the tile's centre (formed as a
 // float pair, the atoms' kept as float pairs), which removes the rounding of absolute node coordinates that the
 // direct kernel has; without the low parts the far sums would share an atom's rounding over a whole tile
-// (flake 8.45e-7 against 8.0e-7 below, for 3 % of the time).
+// (flake 8.45e-7 against 8.0e-7 below).
 //
 // Measured (direct sums -> tiles, Simulator.make_ff): 60-atom flake on 256x256x200 nodes, forces only, 0.408
 // -> 0.136 ms (the grid's 210 MB alone take 31 us); 40-atom molecule on 176x160x60 with the tip's quadrupole
@@ -211,11 +211,11 @@ __device__ __forceinline__ void ff_tile(const TileJob& J, const FFConst& c, int 
         }
         return t;
     };
-    auto stage = [&](const Atom& t, int slot, bool charged) {
+    auto stage = [&](const Atom& t, int slot, bool charged, bool far) {
         ff_stage_atom(c, t.x, t.y, t.z, t.R, t.eps, charged ? t.q : 0.f, r0[slot], r1[slot], r2[slot], r3[slot]);
         r1[slot].y = t.xl;
         r3[slot].y = t.yl;
-        r3[slot].w = -t.zl;
+        r3[slot].w = far ? 2.f * t.z * t.zl : -t.zl;
     };
 
     // ---- A: far atoms at the interpolation points
@@ -245,7 +245,7 @@ __device__ __forceinline__ void ff_tile(const TileJob& J, const FFConst& c, int 
             }
             if (one_chunk ? total < kFarMin : total == 0) continue;
             use_far = true;
-            if (t.far) stage(t, slot, t.charged);
+            if (t.far) stage(t, slot, t.charged, true);
             __syncthreads();
             // this group's atoms lie side by side: a quarter of each kind
             auto sum = [&](auto smooth, int from, int cnt) {
@@ -371,7 +371,7 @@ __device__ __forceinline__ void ff_tile(const TileJob& J, const FFConst& c, int 
             const bool near = t.live && !(use_far && t.far);
             int total;
             const int slot = tile_slot(near, S.count[1], &total);
-            if (near) stage(t, slot, true);
+            if (near) stage(t, slot, true, false);
             __syncthreads();
             ff_accumulate_impl<ZP, kMinImage, kCutoff, kQuad, false, true, Smooth::kNo, true>(r0, r1, r2, r3, total, c, gx, gy, gz, fx, fy,
                                                                           fz, en, fx, fy, fz, en);

@@ -3,14 +3,20 @@
 // space).  For a sample field f and a tip density g on the same periodic grid,
 //   E[n] = scale * dV * sum_h g[h]^p f[n + h]^p,   F = -grad E,
 // with the gradient taken spectrally (i k, Nyquist terms dropped so that the
-// force stays real).  Steps, all in this file:
-//   pack      z = f^p + i g^p (two real transforms in one complex one);
-//   fft3      forward 3D FFT of z: 1D passes along x, y and z;
-//   spectral  F^ = (Z_k + Z*_-k)/2, G^ = (Z_k - Z*_-k)/(2i), P = G^* F^ scale dV / N,
-//             B1 = P + i(-i kx P), B2 = (-i ky P) + i(-i kz P);
-//   fft3      inverse 3D FFTs of B1 and B2 -> (E, Fx) and (Fy, Fz) as (re, im);
-//   output    ff[n] = (Fx, Fy, Fz, E), written or added.
-// The 1D passes are Stockham auto-sort FFTs with radix-8 stages (and one
+// force stays real).  Steps, each one kernel, all in this file, with the bytes read + written per node:
+//   x forward   z = f^p + i g^p (two real transforms in one complex one), formed while loading   8 + 8
+//   y forward   in place                                                                         8 + 8
+//   z middle    a CTA holds the lines (kx, ky) and (-kx, -ky): forward along z, then
+//               F^ = (Z_k + Z*_-k)/2, G^ = (Z_k - Z*_-k)/(2i), P = G^* F^ scale dV / N, then P and
+//               -i kz P inverse along z; E is real, so only kx = 0..nx/2 is kept from here on    8 + 8
+//   y inverse   of P, -i ky P and -i kz P                                                        8 + 12
+//   x inverse   rows of (E, Fx = -i kx E) and (Fy, Fz) as (re, im) of two complex transforms,
+//               rebuilt from their halves while loading; ff[n] = (Fx, Fy, Fz, E), written or added  12 + 16
+// 96 bytes per node; separate pack, spectral and output passes around nine full-spectrum ones moved 224.
+// Measured: 512x512x128 nodes 1392 -> 870 us (3.7 TB/s of these bytes), with power 1.05 and accumulation 1582 -> 1085
+// us, 128^3 139 -> 87 us, 32^3 52 -> 29 us (5 launches for 12).  Now bound by issue (61-78 % active in the
+// first four kernels, 40 % in the last, which moves 28 of the 96 bytes).
+// The 1D transforms are Stockham auto-sort FFTs with radix-8 stages (and one
 // radix-2 or radix-4 stage) in registers, for power-of-two lengths up to 1024:
 // a CTA transforms a tile of neighbouring lines (rows along x, columns along y
 // and z, so every global access is a row of consecutive complex values); the
@@ -23,94 +29,84 @@
 namespace pp {
 namespace {
 
-constexpr int kFftThreads = 256;  // 4 CTAs per SM at 64 registers, tiles of up to 36 KB
-constexpr int kFftBlocksPerSm = 4;
+constexpr int kThreads = 256;
 constexpr int kUnits = 2;          // stage units per thread per trip
 constexpr int kLines = 16;         // lines per tile along x (at most)
 constexpr int kStridedLines = 64;  // columns per tile along y and z (at most)
 
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
-}
-
-// In-register DFT of R points (R = 2, 4, 8), natural order, w = exp(sign 2 pi i / R).
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ float2 mul_i(float2 a, float sign) { return make_float2(-sign * a.y, sign * a.x); }
-
-template <int R>
-__device__ __forceinline__ void dft(float2 (&x)[R], float sign);
-
-template <>
-__device__ __forceinline__ void dft<2>(float2 (&x)[2], float) {
-    const float2 a = x[0], b = x[1];
-    x[0] = cadd(a, b);
-    x[1] = csub(a, b);
+// a w, w = (cos, sin) of the positive angle, conjugated for SIGN = -1
+template <int SIGN>
+__device__ __forceinline__ float2 cmul(float2 w, float2 a) {
+    const float s = SIGN > 0 ? w.y : -w.y;
+    return make_float2(fmaf(w.x, a.x, -s * a.y), fmaf(w.x, a.y, s * a.x));
 }
+template <int SIGN>
+__device__ __forceinline__ float2 mul_i(float2 a) { return SIGN > 0 ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x); }
 
-template <>
-__device__ __forceinline__ void dft<4>(float2 (&x)[4], float sign) {
-    const float2 t0 = cadd(x[0], x[2]), t1 = csub(x[0], x[2]);
-    const float2 t2 = cadd(x[1], x[3]), t3 = mul_i(csub(x[1], x[3]), sign);
-    x[0] = cadd(t0, t2);
-    x[2] = csub(t0, t2);
-    x[1] = cadd(t1, t3);
-    x[3] = csub(t1, t3);
-}
+// In-register DFT of R points (R = 2, 4, 8), natural order, w = exp(SIGN 2 pi i / R).
+template <int R, int SIGN>
+struct Dft;
 
-template <>
-__device__ __forceinline__ void dft<8>(float2 (&x)[8], float sign) {
-    float2 e[4] = {x[0], x[2], x[4], x[6]}, o[4] = {x[1], x[3], x[5], x[7]};
-    dft<4>(e, sign);
-    dft<4>(o, sign);
-    const float h = 0.70710678118654752f;  // w8 = h (1 + sign i)
-    const float2 o1 = make_float2(h * (o[1].x - sign * o[1].y), h * (o[1].y + sign * o[1].x));
-    const float2 o2 = mul_i(o[2], sign);
-    const float2 o3 = make_float2(h * (-o[3].x - sign * o[3].y), h * (-o[3].y + sign * o[3].x));  // w8^3 = h(-1 + sign i)
-    x[0] = cadd(e[0], o[0]);
-    x[4] = csub(e[0], o[0]);
-    x[1] = cadd(e[1], o1);
-    x[5] = csub(e[1], o1);
-    x[2] = cadd(e[2], o2);
-    x[6] = csub(e[2], o2);
-    x[3] = cadd(e[3], o3);
-    x[7] = csub(e[3], o3);
-}
+template <int SIGN>
+struct Dft<2, SIGN> {
+    static __device__ __forceinline__ void run(float2 (&x)[2]) {
+        const float2 a = x[0], b = x[1];
+        x[0] = cadd(a, b);
+        x[1] = csub(a, b);
+    }
+};
 
-// A pass transforms tiles of nl = 2^log2nl lines of n = 2^LOG2N elements.  kContig: lines along x
-// (element p of line l at base + l lstride + p); else columns along y or z (at base + l +
-// p pstride).  In shared memory, columns are interleaved (element p of line l at p nl + l:
-// consecutive threads take consecutive lines, so a warp touches consecutive banks).  Rows lie
+template <int SIGN>
+struct Dft<4, SIGN> {
+    static __device__ __forceinline__ void run(float2 (&x)[4]) {
+        const float2 t0 = cadd(x[0], x[2]), t1 = csub(x[0], x[2]);
+        const float2 t2 = cadd(x[1], x[3]), t3 = mul_i<SIGN>(csub(x[1], x[3]));
+        x[0] = cadd(t0, t2);
+        x[2] = csub(t0, t2);
+        x[1] = cadd(t1, t3);
+        x[3] = csub(t1, t3);
+    }
+};
+
+template <int SIGN>
+struct Dft<8, SIGN> {
+    static __device__ __forceinline__ void run(float2 (&x)[8]) {
+        float2 e[4] = {x[0], x[2], x[4], x[6]}, o[4] = {x[1], x[3], x[5], x[7]};
+        Dft<4, SIGN>::run(e);
+        Dft<4, SIGN>::run(o);
+        const float h = 0.70710678118654752f, s = (float)SIGN;  // w8 = h (1 + sign i)
+        const float2 o1 = make_float2(h * (o[1].x - s * o[1].y), h * (o[1].y + s * o[1].x));
+        const float2 o2 = mul_i<SIGN>(o[2]);
+        const float2 o3 = make_float2(h * (-o[3].x - s * o[3].y), h * (-o[3].y + s * o[3].x));  // w8^3 = h(-1 + sign i)
+        x[0] = cadd(e[0], o[0]);
+        x[4] = csub(e[0], o[0]);
+        x[1] = cadd(e[1], o1);
+        x[5] = csub(e[1], o1);
+        x[2] = cadd(e[2], o2);
+        x[6] = csub(e[2], o2);
+        x[3] = cadd(e[3], o3);
+        x[7] = csub(e[3], o3);
+    }
+};
+
+// Slot of element p of line l of a tile in shared memory.  Columns (kContig = false) are interleaved,
+// p nl + l: consecutive threads take consecutive lines, so a warp touches consecutive banks.  Rows lie
 // one after the other, element e = l n + p, in a layout chosen by the stage that writes them so
 // that both its writes and the next stage's reads (runs of 16 consecutive elements) spread over
 // the 32 banks (a complex value spans two): after the first radix-8 stage (stride-8 writes) the
 // low 3 bits of e are XORed with bits 4-6; after the second (runs of 8 at stride 64) every 64
-// elements are followed by 8 pad slots; later stages write runs of 16 or more and keep e.  n is
-// a template parameter: every stage's index arithmetic folds to shifts and masks of constants.
-struct Pass {
-    int log2nl, nbi, ntiles;
-    long long outer_pitch, stride;  // stride: lstride for rows, pstride for columns
-    long long limit;                // complex values in the array (index bound)
-    float sign;
-};
-
-template <int LOG2N, bool kContig>
-struct TileAt {
-    long long base, stride, limit;
-    int log2nl;
-    __device__ __forceinline__ long long at(int l, int p) const {
-        return checked(kContig ? base + l * stride + p : base + l + p * stride, limit, kChkFft);
-    }
-    // slot of element p of line l in the layout written by the stage after radices L = 2^LOG2W
-    template <int LOG2W>
-    __device__ __forceinline__ int slot(int l, int p) const {
-        if (!kContig) return (p << log2nl) + l;
-        const int e = (l << LOG2N) + p;
-        if constexpr (LOG2W == 0) return e ^ ((e >> 4) & 7);
-        else if constexpr (LOG2W == 3) return e + 8 * (e >> 6);
-        else return e;
-    }
-};
+// elements are followed by 8 pad slots; later stages write runs of 16 or more and keep e.
+// LOG2W: log2 of the product of the radices before the writing stage.
+template <int LOG2N, bool kContig, int LOG2W>
+__device__ __forceinline__ int slot(int log2nl, int l, int p) {
+    if (!kContig) return (p << log2nl) + l;
+    const int e = (l << LOG2N) + p;
+    if constexpr (LOG2W == 0) return e ^ ((e >> 4) & 7);
+    else if constexpr (LOG2W == 3) return e + 8 * (e >> 6);
+    else return e;
+}
 
 // Slots of the largest layout (8 pad slots per 64 elements along rows).
 template <int LOG2N, bool kContig>
@@ -118,166 +114,138 @@ __host__ __device__ __forceinline__ int tile_slots(int nl) {
     return kContig ? (nl << LOG2N) + (nl << LOG2N) / 8 : nl << LOG2N;
 }
 
-// Twiddles of the stage after radices L = 2^LOG2L (all radix 8 before it), radix R = 2^LR:
-// w_{LR}^{m j} for m = 1..R-1, j = 0..L-1 at tw[(L - 1) + (m - 1) L + j], so that threads with
-// consecutive j read consecutive slots; the stages' tables together fill tw[0 .. n-2].
+// Twiddles of the stage after radices L = 2^LOG2L, radix R = 2^LR: w_{LR}^{m j} for m = 1..R-1,
+// j = 0..L-1 at tw[(L - 1) + (m - 1) L + j], so that threads with consecutive j read consecutive slots;
+// the stages' tables together fill tw[0 .. n-2].
 template <int LOG2L, int LR>
-__device__ __forceinline__ void stage_twiddles(float2* tw, float sign) {
+__device__ __forceinline__ void stage_twiddles(float2* tw) {
     constexpr int L = 1 << LOG2L, R = 1 << LR;
-    for (int e = threadIdx.x; e < (R - 1) * L; e += kFftThreads) {
+    for (int e = threadIdx.x; e < (R - 1) * L; e += blockDim.x) {
         const int m = (e >> LOG2L) + 1, j = e & (L - 1);
         float sn, cs;
         sincospif((float)(m * j) * (2.f / (float)(L * R)), &sn, &cs);
-        tw[(L - 1) + e] = make_float2(cs, sign * sn);
+        tw[(L - 1) + e] = make_float2(cs, sn);
     }
+}
+
+// The tables of all stages: radix-8 stages and, first (kRestFirst) or last, the radix-2 or radix-4 remainder.
+template <int LOG2N, bool kRestFirst>
+__device__ __forceinline__ void line_twiddles(float2* tw) {
+    constexpr int N8 = LOG2N / 3, REST = LOG2N - 3 * N8, B = kRestFirst ? REST : 0;
+    if constexpr (REST > 0) stage_twiddles<kRestFirst ? 0 : 3 * N8, REST>(tw);
+    if constexpr (N8 >= 1) stage_twiddles<B, 3>(tw);
+    if constexpr (N8 >= 2) stage_twiddles<B + 3, 3>(tw);
+    if constexpr (N8 >= 3) stage_twiddles<B + 6, 3>(tw);
 }
 
 // One Stockham stage of radix R = 2^LR after stages whose radices multiply to L = 2^LOG2L: unit
 // (line l, t), t < n/R, j = t mod L, k = t / L, reads a_m = x[t + m n/R], twiddles a_m by
-// w_{LR}^{m j}, transforms, writes y[k L R + j + m L].  kFirst reads global memory, kLast
-// writes it; the others read and write the tile in place (every read of a stage precedes its
-// writes: a stage that writes the tile runs in one trip, see lines_per_block).
-template <int LOG2N, bool kContig, int LR, int LOG2L, bool kFirst, bool kLast>
-__device__ __forceinline__ void stage(float2* data, const TileAt<LOG2N, kContig>& T, float2* x, const float2* tw,
-                                      float sign) {
+// w_{LR}^{m j}, transforms, writes y[k L R + j + m L], through `load(l, p)` and `put(l, p, v)`; `map(v)` is
+// applied to what was loaded, after all loads have been issued (powf between them ran one at a time: the
+// x pass of a 512x512x128 grid took 316 us instead of 174).
+// kSharedIn, kSharedOut: whether they exchange through the tile in shared memory; a stage that does both
+// works in place, so its reads must all come before its writes: it has at most kUnits THREADS units
+// (radix 8 and lines_per_block see to that) and a barrier between.
+template <int LOG2N, bool kContig, int LR, int LOG2L, int SIGN, int THREADS, bool kSharedIn, bool kSharedOut, class Load,
+          class Put, class Map>
+__device__ __forceinline__ void stage(int log2nl, const float2* tw, Load&& load, Put&& put, Map&& map) {
     constexpr int R = 1 << LR, LOG2NR = LOG2N - LR, NR = 1 << LOG2NR;
-    const int units = 1 << (T.log2nl + LOG2NR);
-    const int nl_mask = (1 << T.log2nl) - 1;
-    constexpr int U = kUnits;
-    for (int u0 = 0; u0 < units; u0 += kFftThreads * U) {
-        float2 a[U][R];
-        int ul[U], ut[U];
+    const int units = 1 << (log2nl + LOG2NR), nl_mask = (1 << log2nl) - 1;
+    for (int u0 = 0; u0 < units; u0 += kUnits * THREADS) {
+        float2 a[kUnits][R];
 #pragma unroll
-        for (int q = 0; q < U; ++q) {
-            const int u = u0 + q * kFftThreads + threadIdx.x;
+        for (int q = 0; q < kUnits; ++q) {
+            const int u = u0 + q * THREADS + threadIdx.x;
             // consecutive threads: consecutive t along rows, consecutive lines across columns
-            ul[q] = kContig ? u >> LOG2NR : u & nl_mask;
-            ut[q] = kContig ? u & (NR - 1) : u >> T.log2nl;
+            const int l = kContig ? u >> LOG2NR : u & nl_mask, t = kContig ? u & (NR - 1) : u >> log2nl;
             if (u < units) {
 #pragma unroll
-                for (int m = 0; m < R; ++m) {
-                    const int p = ut[q] + m * NR;
-                    if constexpr (kFirst) a[q][m] = data[T.at(ul[q], p)];
-                    else a[q][m] = x[T.template slot<LOG2L - 3>(ul[q], p)];
-                }
+                for (int m = 0; m < R; ++m) a[q][m] = load(l, t + m * NR);
             }
         }
-        if (!kFirst) __syncthreads();
+        if (kSharedIn && kSharedOut) __syncthreads();
 #pragma unroll
-        for (int q = 0; q < U; ++q) {
-            const int u = u0 + q * kFftThreads + threadIdx.x;
+        for (int q = 0; q < kUnits; ++q) {
+            const int u = u0 + q * THREADS + threadIdx.x;
+            const int l = kContig ? u >> LOG2NR : u & nl_mask, t = kContig ? u & (NR - 1) : u >> log2nl;
             if (u >= units) continue;
-            const int t = ut[q], j = t & ((1 << LOG2L) - 1), k = t >> LOG2L;
+            const int j = t & ((1 << LOG2L) - 1), k = t >> LOG2L;
 #pragma unroll
-            for (int m = 1; m < R; ++m) a[q][m] = cmul(tw[((1 << LOG2L) - 1) + ((m - 1) << LOG2L) + j], a[q][m]);
-            dft<R>(a[q], sign);
+            for (int m = 0; m < R; ++m) a[q][m] = map(a[q][m]);
+            if constexpr (LOG2L > 0) {
 #pragma unroll
-            for (int m = 0; m < R; ++m) {
-                const int p = (k << (LOG2L + LR)) + j + (m << LOG2L);
-                if constexpr (kLast) data[T.at(ul[q], p)] = a[q][m];
-                else x[T.template slot<LOG2L>(ul[q], p)] = a[q][m];
+                for (int m = 1; m < R; ++m)
+                    a[q][m] = cmul<SIGN>(tw[((1 << LOG2L) - 1) + ((m - 1) << LOG2L) + j], a[q][m]);
             }
+            Dft<R, SIGN>::run(a[q]);
+#pragma unroll
+            for (int m = 0; m < R; ++m) put(l, (k << (LOG2L + LR)) + j + (m << LOG2L), a[q][m]);
         }
-        if (!kLast) __syncthreads();
+    }
+    // the tile is complete (out), or free for the next writer (in)
+    if (kSharedIn || kSharedOut) __syncthreads();
+}
+
+struct Same {
+    __device__ __forceinline__ float2 operator()(float2 v) const { return v; }
+};
+
+// All stages of a tile's lines from `load` to `put`, through x between.  kIn, kOut: whether those ends are x
+// itself.  In place, only radix-8 stages: the remainder comes first where the input is not x, else last.
+template <int LOG2N, bool kContig, bool kRestFirst, int SIGN, int THREADS, bool kIn, bool kOut, class Load, class Put,
+          class Map = Same>
+__device__ __forceinline__ void fft_lines(int log2nl, float2* x, const float2* tw, Load&& load, Put&& put,
+                                          Map&& map = Map()) {
+    constexpr int N8 = LOG2N / 3, REST = LOG2N - 3 * N8, NS = N8 + (REST > 0 ? 1 : 0);
+    // radices of the first and the last stage
+    constexpr int LF = (kRestFirst && REST > 0) || N8 == 0 ? REST : 3, LE = (!kRestFirst && REST > 0) || N8 == 0 ? REST : 3;
+    static_assert(!(kIn && kOut) || REST == 0, "a remainder stage cannot work in place");
+    static_assert(!kContig || !kRestFirst, "the row layouts assume radix-8 stages first");
+    if constexpr (NS == 1) {
+        stage<LOG2N, kContig, LF, 0, SIGN, THREADS, kIn, kOut>(log2nl, tw, load, put, map);
+    } else {
+        auto out0 = [&](int l, int p, float2 v) { x[slot<LOG2N, kContig, 0>(log2nl, l, p)] = v; };
+        auto in0 = [&](int l, int p) { return x[slot<LOG2N, kContig, 0>(log2nl, l, p)]; };
+        auto out3 = [&](int l, int p, float2 v) { x[slot<LOG2N, kContig, 3>(log2nl, l, p)] = v; };
+        auto in3 = [&](int l, int p) { return x[slot<LOG2N, kContig, 3>(log2nl, l, p)]; };
+        auto out6 = [&](int l, int p, float2 v) { x[slot<LOG2N, kContig, 6>(log2nl, l, p)] = v; };
+        auto in6 = [&](int l, int p) { return x[slot<LOG2N, kContig, 6>(log2nl, l, p)]; };
+        stage<LOG2N, kContig, LF, 0, SIGN, THREADS, kIn, true>(log2nl, tw, load, out0, map);
+        if constexpr (NS == 2) {
+            stage<LOG2N, kContig, LE, LF, SIGN, THREADS, true, kOut>(log2nl, tw, in0, put, Same());
+        } else if constexpr (NS == 3) {
+            stage<LOG2N, kContig, 3, LF, SIGN, THREADS, true, true>(log2nl, tw, in0, out3, Same());
+            stage<LOG2N, kContig, LE, LF + 3, SIGN, THREADS, true, kOut>(log2nl, tw, in3, put, Same());
+        } else {
+            stage<LOG2N, kContig, 3, LF, SIGN, THREADS, true, true>(log2nl, tw, in0, out3, Same());
+            stage<LOG2N, kContig, 3, LF + 3, SIGN, THREADS, true, true>(log2nl, tw, in3, out6, Same());
+            stage<LOG2N, kContig, LE, LF + 6, SIGN, THREADS, true, kOut>(log2nl, tw, in6, put, Same());
+        }
     }
 }
 
-// All stages of one tile: radix-8 stages first (the first reading global memory), the radix-2
-// or radix-4 remainder last.
-template <int LOG2N, bool kContig>
-__device__ __forceinline__ void fft_tile(float2* data, const TileAt<LOG2N, kContig>& T, float2* x, const float2* tw,
-                                         float sign) {
-    constexpr int N8 = LOG2N / 3, REST = LOG2N - 3 * N8;
-    if constexpr (N8 >= 1) stage<LOG2N, kContig, 3, 0, true, N8 == 1 && REST == 0>(data, T, x, tw, sign);
-    if constexpr (N8 >= 2) stage<LOG2N, kContig, 3, 3, false, N8 == 2 && REST == 0>(data, T, x, tw, sign);
-    if constexpr (N8 >= 3) stage<LOG2N, kContig, 3, 6, false, N8 == 3 && REST == 0>(data, T, x, tw, sign);
-    if constexpr (REST == 1) stage<LOG2N, kContig, 1, 3 * N8, N8 == 0, true>(data, T, x, tw, sign);
-    if constexpr (REST == 2) stage<LOG2N, kContig, 2, 3 * N8, N8 == 0, true>(data, T, x, tw, sign);
-}
-
-// One 1D pass: CTA b takes tile b, i.e. outer index b / nbi and lines (b % nbi) nl onwards, at
-// (b / nbi) outer_pitch + line lstride + p pstride (see fft3 for the three axes of the padded
-// layout).  sign = -1 forward, +1 inverse (unnormalised).
-template <int LOG2N, bool kContig>
-__global__ void __launch_bounds__(kFftThreads, kFftBlocksPerSm) fft_pass_kernel(float2* data, const Pass P) {
-    extern __shared__ __align__(128) unsigned char smraw[];
-    constexpr int N = 1 << LOG2N;
-    float2* tw = reinterpret_cast<float2*>(smraw);  // the stages' twiddle tables, N - 1 values
-    float2* x = tw + N;
-    constexpr int N8 = LOG2N / 3, REST = LOG2N - 3 * N8;
-    if constexpr (N8 >= 1) stage_twiddles<0, 3>(tw, P.sign);
-    if constexpr (N8 >= 2) stage_twiddles<3, 3>(tw, P.sign);
-    if constexpr (N8 >= 3) stage_twiddles<6, 3>(tw, P.sign);
-    if constexpr (REST > 0) stage_twiddles<3 * N8, REST>(tw, P.sign);
-    TileAt<LOG2N, kContig> T;
-    const int b = blockIdx.x;
-    T.base = (long long)(b / P.nbi) * P.outer_pitch + ((long long)(b % P.nbi) << P.log2nl) * (kContig ? P.stride : 1);
-    T.stride = P.stride;
-    T.limit = P.limit;
-    T.log2nl = P.log2nl;
-    __syncthreads();
-    fft_tile<LOG2N, kContig>(data, T, x, tw, P.sign);
-}
+// Layouts of the scratch: the full spectrum z, node (i, j, k) at k pz + j px + i with px = nx + 16 and
+// pz = px ny + 16; the half spectra (i <= nx/2) at k hz + j hx + i.  The y and z strides are then not
+// powers of two (a power-of-two stride sends every row of a pass to the same memory channels).  Of the
+// three full arrays' room (fft_workspace_bytes), z has the first and the half arrays a = P and b = -i kz P the
+// end; once z is spent, c = E, d = Fy and e = Fz along x take its place and the gap (5 halves fit 3 wholes).
+struct Plan {
+    const float *f, *g;
+    float4* ff;
+    float2 *z, *a, *b, *c, *d, *e;
+    int nx, ny, nz;
+    int px, pz, hx, hz, zlen, hlen;  // (1040 x 1024 + 16 times 1024 complex values at most: offsets fit 32 bits)
+    float kx0, ky0, kz0;  // 2 pi / (n d) per axis
+    float norm;           // scale * dV / N
+    float power;
+    int accumulate;
+    int log2nl;           // lines of a tile (of one kind where a kernel takes several)
+};
 
 __device__ __forceinline__ float powered(float v, float p) {
     if (p == 1.f) return v;
     return v > 0.f ? powf(v, p) : 0.f;
 }
-
-// Padded complex layout of the scratch arrays: node (i, j, k) at
-// k * pz + j * px + i with px = nx + 16 and pz = px * ny + 16, so that the
-// strides of the y and z passes are not powers of two (a power-of-two stride
-// sends every row of a pass to the same memory channels) while every row stays
-// 128-byte aligned.
-struct Pad {
-    int nx, ny, nz;
-    long long px, pz;
-    __device__ __forceinline__ long long at(int i, int j, int k) const { return (long long)k * pz + (long long)j * px + i; }
-};
-
-Pad make_pad(int nx, int ny, int nz) {
-    Pad P;
-    P.nx = nx; P.ny = ny; P.nz = nz;
-    P.px = nx + 16;
-    P.pz = P.px * ny + 16;
-    return P;
-}
-
-// Elementwise kernels walk rows (j, k) of the grid: blocks take rows, threads the
-// x index, so no per-element division is needed.
-// Rows of nx >= 4 go four nodes per thread: two 16-byte loads, two 16-byte stores (row starts
-// are 16-byte aligned on both sides: nx, nx + 16 and the plane pitch are multiples of 4).
-__global__ void pack_kernel(const float* __restrict__ f, const float* __restrict__ g, float2* z, const Pad P, float p) {
-    const int rows = P.ny * P.nz;
-    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
-        const int j = r % P.ny, k = r / P.ny;
-        const long long src = (long long)r * P.nx, dst = P.at(0, j, k);
-        // the row's last complex value and last input float lie inside their arrays
-        checked(dst + P.nx - 1, (long long)P.nz * P.pz, kChkFft);
-        checked(src + P.nx - 1, (long long)P.nx * P.ny * P.nz, kChkFft);
-        if ((P.nx & 3) == 0) {
-            const float4* f4 = reinterpret_cast<const float4*>(f + src);
-            const float4* g4 = reinterpret_cast<const float4*>(g + src);
-            float4* z4 = reinterpret_cast<float4*>(z + dst);
-            for (int i = threadIdx.x; i < (P.nx >> 2); i += blockDim.x) {
-                const float4 a = __ldg(f4 + i), b = __ldg(g4 + i);
-                z4[2 * i] = make_float4(powered(a.x, p), powered(b.x, p), powered(a.y, p), powered(b.y, p));
-                z4[2 * i + 1] = make_float4(powered(a.z, p), powered(b.z, p), powered(a.w, p), powered(b.w, p));
-            }
-        } else {
-            for (int i = threadIdx.x; i < P.nx; i += blockDim.x)
-                z[dst + i] = make_float2(powered(__ldg(f + src + i), p), powered(__ldg(g + src + i), p));
-        }
-    }
-}
-
-struct SpecArgs {
-    const float2* z;
-    float2 *b1, *b2;
-    Pad P;
-    float kx0, ky0, kz0;  // 2 pi / (n d) per axis
-    float norm;           // scale * dV / N
-};
 
 // Wavenumber of index m along an axis of length n (Nyquist -> 0 for the derivative).
 __device__ __forceinline__ float wavenumber(int m, int n, float k0) {
@@ -285,51 +253,166 @@ __device__ __forceinline__ float wavenumber(int m, int n, float k0) {
     return (2 * m < n ? (float)m : (float)(m - n)) * k0;
 }
 
-__global__ void spectral_kernel(const SpecArgs A) {
-    const Pad& P = A.P;
-    const int rows = P.ny * P.nz;
-    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
-        const int j = r % P.ny, k = r / P.ny;
-        const int mj = j == 0 ? 0 : P.ny - j, mk = k == 0 ? 0 : P.nz - k;
-        const float ky = wavenumber(j, P.ny, A.ky0), kz = wavenumber(k, P.nz, A.kz0);
-        const long long row = checked(P.at(0, j, k), (long long)P.nz * P.pz - P.nx + 1, kChkFft);
-        const long long mrow = checked(P.at(0, mj, mk), (long long)P.nz * P.pz - P.nx + 1, kChkFft);
-        for (int i = threadIdx.x; i < P.nx; i += blockDim.x) {
-            const int mi = i == 0 ? 0 : P.nx - i;
-            const float2 zk = A.z[row + i];
-            const float2 zm = A.z[mrow + mi];
+// Block b: rows (b % nbi) nl onwards of plane b / nbi.
+template <int LOG2N>
+__global__ void __launch_bounds__(kThreads, 4) fft_x_forward_kernel(const Plan P) {
+    extern __shared__ __align__(128) unsigned char smraw[];
+    float2* const tw = reinterpret_cast<float2*>(smraw);
+    float2* const x = tw + (1 << LOG2N);
+    line_twiddles<LOG2N, false>(tw);
+    __syncthreads();
+    const int nbi = P.ny >> P.log2nl, k = blockIdx.x / nbi, j0 = (blockIdx.x % nbi) << P.log2nl;
+    const int nodes = (P.ny * P.nz) << LOG2N;
+    const int src = (k * P.ny + j0) << LOG2N, dst = k * P.pz + j0 * P.px;
+    fft_lines<LOG2N, true, false, -1, kThreads, false, false>(
+        P.log2nl, x, tw,
+        [&](int l, int p) {
+            const int s = checked(src + (l << LOG2N) + p, nodes, kChkFft);
+            return make_float2(__ldg(P.f + s), __ldg(P.g + s));
+        },
+        [&](int l, int p, float2 v) { P.z[checked(dst + l * P.px + p, P.zlen, kChkFft)] = v; },
+        [&](float2 v) { return make_float2(powered(v.x, P.power), powered(v.y, P.power)); });
+}
+
+// Block b: columns (b % nbi) nl onwards of plane b / nbi.
+template <int LOG2N>
+__global__ void __launch_bounds__(kThreads, 4) fft_y_forward_kernel(const Plan P) {
+    extern __shared__ __align__(128) unsigned char smraw[];
+    float2* const tw = reinterpret_cast<float2*>(smraw);
+    float2* const x = tw + (1 << LOG2N);
+    line_twiddles<LOG2N, false>(tw);
+    __syncthreads();
+    const int nbi = P.nx >> P.log2nl;
+    const int base = (int)(blockIdx.x / nbi) * P.pz + (int)((blockIdx.x % nbi) << P.log2nl);
+    auto at = [&](int l, int p) { return checked(base + l + p * P.px, P.zlen, kChkFft); };
+    fft_lines<LOG2N, false, false, -1, kThreads, false, false>(
+        P.log2nl, x, tw, [&](int l, int p) { return P.z[at(l, p)]; },
+        [&](int l, int p, float2 v) { P.z[at(l, p)] = v; });
+}
+
+// Block b: columns i = (b % nbi) nl onwards (i <= nx/2) of row j = b / nbi, and their mirrors (-i, -j) as
+// lines nl .. 2 nl - 1 of the tile.
+template <int LOG2N, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 2) fft_z_middle_kernel(const Plan P) {
+    extern __shared__ __align__(128) unsigned char smraw[];
+    constexpr int N = 1 << LOG2N;
+    float2* const tw = reinterpret_cast<float2*>(smraw);  // forward, then inverse tables
+    float2* const x = tw + 2 * N;
+    line_twiddles<LOG2N, true>(tw);
+    line_twiddles<LOG2N, false>(tw + N);
+    __syncthreads();
+    const int nl = 1 << P.log2nl, half = P.nx / 2, nbi = (half >> P.log2nl) + 1;
+    const int j = blockIdx.x / nbi, i0 = (blockIdx.x % nbi) << P.log2nl, mj = j == 0 ? 0 : P.ny - j;
+    const int log2all = P.log2nl + 1;
+    fft_lines<LOG2N, false, true, -1, THREADS, false, true>(
+        log2all, x, tw,
+        [&](int l, int p) {
+            const int i = i0 + (l & (nl - 1));
+            if (i > half) return make_float2(0.f, 0.f);
+            const int o = l < nl ? j * P.px + i : mj * P.px + (i == 0 ? 0 : P.nx - i);
+            return P.z[checked(o + p * P.pz, P.zlen, kChkFft)];
+        },
+        [&](int l, int p, float2 v) { x[(p << log2all) + l] = v; });
+    // the products at p and n - p together: each needs both lines at both
+    for (int u = threadIdx.x; u < ((N / 2 + 1) << P.log2nl); u += THREADS) {
+        const int l = u & (nl - 1), p = u >> P.log2nl, q = p == 0 ? 0 : N - p;
+        float2* const zp = x + (p << log2all) + l;
+        float2* const zq = x + (q << log2all) + l;
+        const float2 z0 = zp[0], m0 = zq[nl], z1 = zq[0], m1 = zp[nl];
+        auto product = [&](float2 zk, float2 zm, int m, float2* out) {
             // F^ = (Z_k + conj Z_-k)/2, G^ = (Z_k - conj Z_-k)/(2i)
             const float2 F = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
             const float2 G = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
-            // P = conj(G) F * norm
-            const float2 Pk = make_float2(A.norm * fmaf(G.x, F.x, G.y * F.y), A.norm * fmaf(G.x, F.y, -G.y * F.x));
-            const float kx = wavenumber(i, P.nx, A.kx0);
-            // -i k P = (k P.y, -k P.x); B1 = P + i(-i kx P), B2 = (-i ky P) + i(-i kz P); i (a + ib) = (-b, a)
-            const float2 dx = make_float2(kx * Pk.y, -kx * Pk.x);
-            const float2 dy = make_float2(ky * Pk.y, -ky * Pk.x);
-            const float2 dz = make_float2(kz * Pk.y, -kz * Pk.x);
-            A.b1[row + i] = make_float2(Pk.x - dx.y, Pk.y + dx.x);
-            A.b2[row + i] = make_float2(dy.x - dz.y, dy.y + dz.x);
-        }
+            // P = conj(G) F norm, and -i kz P
+            const float2 Pk = make_float2(P.norm * fmaf(G.x, F.x, G.y * F.y), P.norm * fmaf(G.x, F.y, -G.y * F.x));
+            const float kz = wavenumber(m, N, P.kz0);
+            out[0] = Pk;
+            out[nl] = make_float2(kz * Pk.y, -kz * Pk.x);
+        };
+        product(z0, m0, p, zp);
+        if (q != p) product(z1, m1, q, zq);
     }
+    __syncthreads();
+    fft_lines<LOG2N, false, false, 1, THREADS, true, false>(
+        log2all, x, tw + N, [&](int l, int p) { return x[(p << log2all) + l]; },
+        [&](int l, int p, float2 v) {
+            const int i = i0 + (l & (nl - 1));
+            if (i > half) return;
+            (l < nl ? P.a : P.b)[checked(j * P.hx + i + p * P.hz, P.hlen, kChkFft)] = v;
+        });
 }
 
-__global__ void output_kernel(const float2* __restrict__ b1, const float2* __restrict__ b2, float4* ff, const Pad P,
-                              int accumulate) {
-    const int rows = P.ny * P.nz;
-    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
-        const long long src = checked(P.at(0, r % P.ny, r / P.ny), (long long)P.nz * P.pz - P.nx + 1, kChkFft);
-        const long long dst = checked((long long)r * P.nx, (long long)P.nx * P.ny * P.nz - P.nx + 1, kChkFft);
-        for (int i = threadIdx.x; i < P.nx; i += blockDim.x) {
-            const float2 a = b1[src + i], b = b2[src + i];  // (E, Fx), (Fy, Fz)
-            float4 v = make_float4(a.y, b.x, b.y, a.x);     // the spectra already hold -i k P: forces
-            if (accumulate) {
-                const float4 w = ff[dst + i];
-                v = make_float4(w.x + v.x, w.y + v.y, w.z + v.z, w.w + v.w);
+// Block b: kind b % 3 (E and Fy from P, Fz from -i kz P) of columns ((b / 3) % nbi) nl onwards of plane
+// (b / 3) / nbi; the kinds that share a source run side by side.
+template <int LOG2N>
+__global__ void __launch_bounds__(kThreads, 4) fft_y_inverse_kernel(const Plan P) {
+    extern __shared__ __align__(128) unsigned char smraw[];
+    float2* const tw = reinterpret_cast<float2*>(smraw);
+    float2* const x = tw + (1 << LOG2N);
+    line_twiddles<LOG2N, false>(tw);
+    __syncthreads();
+    const int kind = blockIdx.x % 3, b = blockIdx.x / 3, half = P.nx / 2, nbi = (half >> P.log2nl) + 1;
+    const int k = b / nbi, i0 = (b % nbi) << P.log2nl;
+    const float2* const in = kind == 2 ? P.b : P.a;
+    float2* const out = kind == 0 ? P.c : kind == 1 ? P.d : P.e;
+    auto at = [&](int l, int p) { return checked(k * P.hz + p * P.hx + i0 + l, P.hlen, kChkFft); };
+    fft_lines<LOG2N, false, false, 1, kThreads, false, false>(
+        P.log2nl, x, tw,
+        [&](int l, int p) {
+            if (i0 + l > half) return make_float2(0.f, 0.f);
+            const float2 v = in[at(l, p)];
+            if (kind != 1) return v;
+            const float ky = wavenumber(p, 1 << LOG2N, P.ky0);
+            return make_float2(ky * v.y, -ky * v.x);
+        },
+        [&](int l, int p, float2 v) {
+            if (i0 + l <= half) out[at(l, p)] = v;
+        });
+}
+
+// Block b: rows (b % nbi) nl onwards of plane b / nbi.  y: the finished (E, Fx) rows.
+template <int LOG2N>
+__global__ void __launch_bounds__(kThreads, 3) fft_x_inverse_kernel(const Plan P) {
+    extern __shared__ __align__(128) unsigned char smraw[];
+    constexpr int N = 1 << LOG2N;
+    float2* const tw = reinterpret_cast<float2*>(smraw);
+    float2* const x = tw + N;
+    float2* const y = x + tile_slots<LOG2N, true>(1 << P.log2nl);
+    line_twiddles<LOG2N, false>(tw);
+    __syncthreads();
+    const int nbi = P.ny >> P.log2nl, k = blockIdx.x / nbi, j0 = (blockIdx.x % nbi) << P.log2nl;
+    const int nodes = (P.ny * P.nz) << LOG2N;
+    const int src = k * P.hz + j0 * P.hx, dst = (k * P.ny + j0) << LOG2N;
+    // element p of a real row's spectrum from its half; the ends are real
+    auto full = [&](const float2* h, int l, int p) {
+        const float2 v = h[checked(src + l * P.hx + (2 * p <= N ? p : N - p), P.hlen, kChkFft)];
+        return make_float2(v.x, p == 0 || 2 * p == N ? 0.f : 2 * p < N ? v.y : -v.y);
+    };
+    fft_lines<LOG2N, true, false, 1, kThreads, false, false>(
+        P.log2nl, x, tw,
+        [&](int l, int p) {
+            const float2 v = full(P.c, l, p);
+            const float s = 1.f + wavenumber(p, N, P.kx0);  // E^ + i (-i kx E^)
+            return make_float2(s * v.x, s * v.y);
+        },
+        [&](int l, int p, float2 v) { y[(l << LOG2N) + p] = v; });
+    __syncthreads();
+    fft_lines<LOG2N, true, false, 1, kThreads, false, false>(
+        P.log2nl, x, tw,
+        [&](int l, int p) {
+            const float2 u = full(P.d, l, p), v = full(P.e, l, p);
+            return make_float2(u.x - v.y, u.y + v.x);
+        },
+        [&](int l, int p, float2 v) {
+            const float2 u = y[(l << LOG2N) + p];
+            float4 o = make_float4(u.y, v.x, v.y, u.x);
+            float4* const to = P.ff + checked(dst + (l << LOG2N) + p, nodes, kChkFft);
+            if (P.accumulate) {
+                const float4 w = *to;
+                o = make_float4(w.x + o.x, w.y + o.y, w.z + o.z, w.w + o.w);
             }
-            ff[dst + i] = v;
-        }
-    }
+            *to = o;
+        });
 }
 
 int ilog2i(int v) {
@@ -338,105 +421,114 @@ int ilog2i(int v) {
     return l;
 }
 
-template <int LOG2N, bool kContig>
-cudaError_t launch_pass(float2* data, const Pass& P, cudaStream_t s) {
-    const size_t smem = ((size_t)(1 << LOG2N) + (size_t)tile_slots<LOG2N, kContig>(1 << P.log2nl)) * sizeof(float2);
-    auto k = fft_pass_kernel<LOG2N, kContig>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+// log2 of the lines per tile for lines of n among `avail` neighbours (powers of two): up to `want`, and at
+// most what gives `kinds` times as many lines kUnits units of a radix-8 stage per thread.
+int lines_per_block(int n, int avail, int want, int threads, int kinds) {
+    const int cap = 8 * kUnits * threads / (n * kinds);
+    const int L = avail < want ? avail : want;
+    return ilog2i(L < cap ? L : cap);
+}
+
+template <class K>
+cudaError_t launch(K kernel, long long blocks, int threads, size_t values, const Plan& P, cudaStream_t s) {
+    const int smem = (int)(values * sizeof(float2));
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    k<<<P.ntiles, kFftThreads, smem, s>>>(data, P);
+    kernel<<<(unsigned)blocks, threads, smem, s>>>(P);
     return cudaGetLastError();
 }
 
-template <bool kContig>
-cudaError_t launch_pass_n(float2* data, int log2n, const Pass& P, cudaStream_t s) {
-    switch (log2n) {
-        case 1: return launch_pass<1, kContig>(data, P, s);
-        case 2: return launch_pass<2, kContig>(data, P, s);
-        case 3: return launch_pass<3, kContig>(data, P, s);
-        case 4: return launch_pass<4, kContig>(data, P, s);
-        case 5: return launch_pass<5, kContig>(data, P, s);
-        case 6: return launch_pass<6, kContig>(data, P, s);
-        case 7: return launch_pass<7, kContig>(data, P, s);
-        case 8: return launch_pass<8, kContig>(data, P, s);
-        case 9: return launch_pass<9, kContig>(data, P, s);
-        case 10: return launch_pass<10, kContig>(data, P, s);
+// f(std::integral_constant<int, log2 n>)
+template <class F>
+cudaError_t with_log2(int n, F&& f) {
+    switch (ilog2i(n)) {
+        case 1: return f(std::integral_constant<int, 1>{});
+        case 2: return f(std::integral_constant<int, 2>{});
+        case 3: return f(std::integral_constant<int, 3>{});
+        case 4: return f(std::integral_constant<int, 4>{});
+        case 5: return f(std::integral_constant<int, 5>{});
+        case 6: return f(std::integral_constant<int, 6>{});
+        case 7: return f(std::integral_constant<int, 7>{});
+        case 8: return f(std::integral_constant<int, 8>{});
+        case 9: return f(std::integral_constant<int, 9>{});
+        case 10: return f(std::integral_constant<int, 10>{});
         default: return cudaErrorInvalidValue;
     }
 }
 
-// Tiles of nl lines of n; nbi tiles per outer index; rows along x (lines lstride apart) or columns
-// (elements pstride apart).
-cudaError_t fft_axis(float2* data, long long limit, bool rows, int n, int nl, int nbi, int nouter,
-                     long long outer_pitch, long long stride, float sign, cudaStream_t s) {
-    if (n < 2) return cudaSuccess;
-    Pass P;
-    P.log2nl = ilog2i(nl);
-    P.nbi = nbi;
-    P.ntiles = nbi * nouter;
-    P.outer_pitch = outer_pitch;
-    P.stride = stride;
-    P.limit = limit;
-    P.sign = sign;
-    return rows ? launch_pass_n<true>(data, ilog2i(n), P, s) : launch_pass_n<false>(data, ilog2i(n), P, s);
-}
-
-// Lines per tile for lines of n among `avail` neighbours: up to `want`, fewer when the axis
-// has fewer, and at most 8 U kFftThreads / n (U units per thread) so that a radix-8 stage that
-// writes shared memory (in place) has at most U kFftThreads units: all of its reads then happen
-// before its writes.
-int lines_per_block(int n, int avail, int want, int units) {
-    const int cap = 8 * units * kFftThreads / n;
-    const int L = avail < want ? avail : want;
-    return L < cap ? L : cap;
-}
-
-cudaError_t fft3(float2* data, const Pad& P, float sign, cudaStream_t s) {
-    cudaError_t e;
-    int nl = lines_per_block(P.nx, P.ny, kLines, kUnits);  // x: lines are rows j of a plane k
-    const long long lim = (long long)P.nz * P.pz;
-    if ((e = fft_axis(data, lim, true, P.nx, nl, P.ny / nl, P.nz, P.pz, P.px, sign, s)) != cudaSuccess) return e;
-    nl = lines_per_block(P.ny, P.nx, kStridedLines, kUnits);  // y: lines are columns i of a plane k
-    if ((e = fft_axis(data, lim, false, P.ny, nl, P.nx / nl, P.nz, P.pz, P.px, sign, s)) != cudaSuccess) return e;
-    nl = lines_per_block(P.nz, P.nx, kStridedLines, kUnits);  // z: lines are columns i of a row j
-    return fft_axis(data, lim, false, P.nz, nl, P.nx / nl, P.ny, P.px, P.pz, sign, s);
+void make_layout(int nx, int ny, int nz, Plan* P) {
+    P->nx = nx; P->ny = ny; P->nz = nz;
+    P->px = nx + 16;
+    P->pz = P->px * ny + 16;
+    // (below 64 nodes along x the narrower pitch keeps five halves inside three wholes)
+    P->hx = nx / 2 + (nx >= 64 ? 16 : 2);
+    P->hz = P->hx * ny + 8;
+    P->zlen = P->pz * nz;
+    P->hlen = P->hz * nz;
 }
 
 }  // namespace
 
 size_t fft_workspace_bytes(int nx, int ny, int nz) {
-    const Pad P = make_pad(nx, ny, nz);
-    return (size_t)3 * (size_t)(P.nz * P.pz) * sizeof(float2);
+    Plan P;
+    make_layout(nx, ny, nz, &P);
+    return (size_t)3 * (size_t)P.zlen * sizeof(float2);
 }
 
 cudaError_t launch_fft_correlate(const FftLaunch& L, cudaStream_t s) {
-    const Pad P = make_pad(L.nx, L.ny, L.nz);
-    const long long N = (long long)L.nx * L.ny * L.nz, NP = (long long)P.nz * P.pz;
-    float2* z = reinterpret_cast<float2*>(L.ws);
-    float2* b1 = z + NP;
-    float2* b2 = b1 + NP;
-    const int threads = 256;
-    const int rows = L.ny * L.nz;
-    const int blocks = rows < 152 * 32 ? rows : 152 * 32;
-    pack_kernel<<<blocks, threads, 0, s>>>(L.f, L.g, z, P, L.power);
-    cudaError_t e = cudaGetLastError();
+    Plan P;
+    make_layout(L.nx, L.ny, L.nz, &P);
+    P.f = L.f;
+    P.g = L.g;
+    P.ff = L.ff;
+    P.z = reinterpret_cast<float2*>(L.ws);
+    P.a = P.z + 3 * P.zlen - 2 * P.hlen;
+    P.b = P.a + P.hlen;
+    P.c = P.z;
+    P.d = P.c + P.hlen;
+    P.e = P.d + P.hlen;
+    P.kx0 = (float)(2.0 * kPi / (L.nx * (double)L.dx));
+    P.ky0 = (float)(2.0 * kPi / (L.ny * (double)L.dy));
+    P.kz0 = (float)(2.0 * kPi / (L.nz * (double)L.dz));
+    P.norm = (float)((double)L.scale * (double)L.dx * L.dy * L.dz / ((double)L.nx * L.ny * L.nz));
+    P.power = L.power;
+    P.accumulate = L.accumulate;
+    const int half = L.nx / 2;
+    cudaError_t e;
+    P.log2nl = lines_per_block(L.nx, L.ny, kLines, kThreads, 1);
+    e = with_log2(L.nx, [&](auto n) {
+        constexpr int LN = decltype(n)::value;
+        return launch(fft_x_forward_kernel<LN>, (long long)(L.ny >> P.log2nl) * L.nz, kThreads,
+                      (size_t)(1 << LN) + tile_slots<LN, true>(1 << P.log2nl), P, s);
+    });
     if (e != cudaSuccess) return e;
-    if ((e = fft3(z, P, -1.f, s)) != cudaSuccess) return e;
-    SpecArgs A;
-    A.z = z;
-    A.b1 = b1;
-    A.b2 = b2;
-    A.P = P;
-    A.kx0 = (float)(2.0 * kPi / (L.nx * (double)L.dx));
-    A.ky0 = (float)(2.0 * kPi / (L.ny * (double)L.dy));
-    A.kz0 = (float)(2.0 * kPi / (L.nz * (double)L.dz));
-    A.norm = (float)((double)L.scale * (double)L.dx * L.dy * L.dz / (double)N);
-    spectral_kernel<<<blocks, threads, 0, s>>>(A);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = fft3(b1, P, 1.f, s)) != cudaSuccess) return e;
-    if ((e = fft3(b2, P, 1.f, s)) != cudaSuccess) return e;
-    output_kernel<<<blocks, threads, 0, s>>>(b1, b2, L.ff, P, L.accumulate);
-    return cudaGetLastError();
+    P.log2nl = lines_per_block(L.ny, L.nx, kStridedLines, kThreads, 1);
+    e = with_log2(L.ny, [&](auto n) {
+        constexpr int LN = decltype(n)::value;
+        return launch(fft_y_forward_kernel<LN>, (long long)(L.nx >> P.log2nl) * L.nz, kThreads,
+                      (size_t)(1 << LN) + tile_slots<LN, false>(1 << P.log2nl), P, s);
+    });
+    if (e != cudaSuccess) return e;
+    e = with_log2(L.nz, [&](auto n) {
+        constexpr int LN = decltype(n)::value, T = LN >= 9 ? 512 : 256;
+        P.log2nl = lines_per_block(L.nz, half, kStridedLines / 2, T, 2);
+        return launch(fft_z_middle_kernel<LN, T>, (long long)((half >> P.log2nl) + 1) * L.ny, T,
+                      (size_t)(2 << LN) + tile_slots<LN, false>(2 << P.log2nl), P, s);
+    });
+    if (e != cudaSuccess) return e;
+    P.log2nl = lines_per_block(L.ny, half, kStridedLines, kThreads, 1);
+    e = with_log2(L.ny, [&](auto n) {
+        constexpr int LN = decltype(n)::value;
+        return launch(fft_y_inverse_kernel<LN>, 3LL * ((half >> P.log2nl) + 1) * L.nz, kThreads,
+                      (size_t)(1 << LN) + tile_slots<LN, false>(1 << P.log2nl), P, s);
+    });
+    if (e != cudaSuccess) return e;
+    P.log2nl = lines_per_block(L.nx, L.ny, kLines, kThreads, 1);
+    return with_log2(L.nx, [&](auto n) {
+        constexpr int LN = decltype(n)::value;
+        return launch(fft_x_inverse_kernel<LN>, (long long)(L.ny >> P.log2nl) * L.nz, kThreads,
+                      (size_t)(1 << LN) + tile_slots<LN, true>(1 << P.log2nl) + ((size_t)1 << (LN + P.log2nl)), P, s);
+    });
 }
 
 PP_CHECK_READER(check_flags_fft)

@@ -566,17 +566,14 @@ pp_status backward_prepare(const std::string& who, const pp_atoms* atoms, const 
     return PP_OK;
 }
 
-// Points the prepared launch at the workspace ws (kBwdHeader + adj_bytes bytes, 16-byte aligned),
-// clears the grid adjoint and enqueues the adjoint kernels.
-pp_status backward_launch(const std::string& who, BwdLaunch& L, void* ws, size_t adj_bytes, cudaStream_t s) {
+// Points the prepared launch at the workspace ws (kBwdHeader and the grid adjoint's bytes, 16-byte aligned) and
+// enqueues the adjoint kernels, which clear what they need of it.
+pp_status backward_launch(const std::string& who, BwdLaunch& L, void* ws, cudaStream_t s) {
     L.slab = reinterpret_cast<int*>(ws);
     L.gbar = L.map.interp ? nullptr : reinterpret_cast<float4*>(reinterpret_cast<char*>(ws) + kBwdHeader);
     L.gbarE = L.map.interp ? reinterpret_cast<float*>(reinterpret_cast<char*>(ws) + kBwdHeader) : nullptr;
     L.qsumd = reinterpret_cast<double*>(reinterpret_cast<char*>(ws) + 32);
     L.tipd = reinterpret_cast<double*>(reinterpret_cast<char*>(ws) + 64);
-    pp_status st = cuda_status(cudaMemsetAsync(reinterpret_cast<char*>(ws) + kBwdHeader, 0, adj_bytes, s),
-                               (who + " memset").c_str());
-    if (st != PP_OK) return st;
     return cuda_status(launch_backward(L, s), (who + " launch").c_str());
 }
 
@@ -601,7 +598,7 @@ pp_status pp_backward(const pp_atoms* atoms, const pp_probe* probe, const pp_gri
         set_error("pp_backward: workspace too small (need " + std::to_string(need) + " bytes)");
         return PP_ERR_CAPACITY;
     }
-    return backward_launch("pp_backward", L, ws, adj_bytes, (cudaStream_t)stream);
+    return backward_launch("pp_backward", L, ws, (cudaStream_t)stream);
 }
 
 size_t pp_batch_workspace(int nmol) { return batch_workspace_bytes(nmol); }

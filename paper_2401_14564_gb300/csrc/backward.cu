@@ -27,6 +27,10 @@ namespace pp {
 namespace {
 
 constexpr int kAdjThreads = 128;
+// Adjoint grids from this size on are cleared in the band the scan reaches alone: on the flake 8 us to find
+// it in the positions (31 MB) and 8 to clear it, against 31 for all of the 210 MB.
+constexpr int64_t kBandBytes = 64 << 20;
+
 // Resident CTAs per SM of K4, which waits on its gathers: 6 at 80 registers (flake60, whole adjoint: 5 at 93
 // registers 262 us, 6: 253, 7: 255, 8: 268; launched as one wave, where 8 CTAs per SM at 93 registers ran
 // as 1.6).
@@ -47,6 +51,8 @@ __global__ void init_kernel(const BwdLaunch P) {
         P.slab[0] = 0x7fffffff;
         P.slab[1] = -1;
         P.slab[2] = 0;
+        P.slab[4] = 0x7fffffff;
+        P.slab[5] = -1;
         P.gtip[0] = P.gtip[1] = P.gtip[2] = P.gtip[3] = P.gtip[4] = 0.f;
         P.qsumd[0] = P.qsumd[1] = 0.0;
         P.tipd[0] = P.tipd[1] = P.tipd[2] = 0.0;
@@ -740,45 +746,111 @@ __global__ void __launch_bounds__(kTileThreads, 2) ff_backward_tile_kernel(const
     }
 }
 
+// The sum of v over the warp as a float pair: FP64 adds run 2 lanes to a clock here.
+__device__ __forceinline__ float2 warp_sum_pair(float v) {
+    float hi = v, lo = 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float h = __shfl_xor_sync(0xffffffffu, hi, o), l = __shfl_xor_sync(0xffffffffu, lo, o);
+        float s, e;
+        two_sum(hi, h, s, e);
+        hi = s;
+        lo = __fadd_rn(__fadd_rn(lo, l), e);
+    }
+    return make_float2(hi, lo);
+}
+
 // Gradients from the tile kernel's replicas, a warp per atom.  dL/dq = k_e (Q C + (Qzz/2) Cq),
-// dL/dQ = k_e sum_i q_i C_i and dL/dQzz = (k_e/2) sum_i q_i Cq_i, the sums over replicas and atoms in FP64; the
-// last block writes the tip's.
+// dL/dQ = k_e sum_i q_i C_i and dL/dQzz = (k_e/2) sum_i q_i Cq_i, the sums over replicas as float pairs, the two over
+// atoms in FP64; the last block writes the tip's.  7 us; with FP64 reductions 11, and as one block for all atoms
+// 20-40 (one SM's FP64 pipe).
 __global__ void __launch_bounds__(256) finalize_tile_kernel(const BwdLaunch P) {
     __shared__ double sum[2][8];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, a = blockIdx.x * 8 + warp;
-    double v[7];
+    float w[7];
 #pragma unroll
-    for (int q = 0; q < 7; ++q) {
-        v[q] = a < P.n && lane < P.replicas ? (double)P.gbar[(7 * lane + q) * P.n + a].w : 0.0;
-        v[q] = warp_sum(v[q]);
-    }
+    for (int q = 0; q < 7; ++q) w[q] = a < P.n && lane < P.replicas ? P.gbar[(7 * lane + q) * P.n + a].w : 0.f;
+    float2 v[7];
+#pragma unroll
+    for (int q = 0; q < 7; ++q) v[q] = warp_sum_pair(w[q]);
     if (lane == 0) {
-        const double q = a < P.n ? (double)P.aq[a] : 0.0;
-        sum[0][warp] = a < P.n ? q * v[5] : 0.0;
-        sum[1][warp] = a < P.n ? q * v[6] : 0.0;
+        sum[0][warp] = sum[1][warp] = 0.0;
         if (a < P.n) {
-            const float eij = sqrtf(P.aeps[a] * P.eps_pp);
-            P.gx[a] = (float)v[0];
-            P.gy[a] = (float)v[1];
-            P.gz[a] = (float)v[2];
-            P.gR[a] = (float)v[3];
-            P.geps[a] = eij > 0.f ? (float)(v[4] * (double)P.eps_pp / (2.0 * (double)eij)) : 0.f;
-            P.gq[a] = (float)((double)P.ke * ((double)P.Q * v[5] + 0.5 * (double)P.Qzz * v[6]));
+            const float eij = sqrtf(P.aeps[a] * P.eps_pp), q = P.aq[a];
+            P.gx[a] = v[0].x;
+            P.gy[a] = v[1].x;
+            P.gz[a] = v[2].x;
+            P.gR[a] = v[3].x;
+            P.geps[a] = eij > 0.f ? v[4].x * P.eps_pp / (2.f * eij) : 0.f;
+            P.gq[a] = P.ke * fmaf(P.Q, v[5].x, 0.5f * P.Qzz * v[6].x);
+            sum[0][warp] = (double)q * ((double)v[5].x + (double)v[5].y);
+            sum[1][warp] = (double)q * ((double)v[6].x + (double)v[6].y);
         }
     }
     __syncthreads();
     if (threadIdx.x != 0) return;
     for (int t = 0; t < 2; ++t) {
         double d = 0.0;
-        for (int w = 0; w < 8; ++w) d += sum[t][w];
-        atomicAdd(P.qsumd + t, d);
+        for (int u = 0; u < 8; ++u) d += sum[t][u];
+        if (t == 0 || P.Qzz != 0.f) atomicAdd(P.qsumd + t, d);
     }
     __threadfence();
     if (atomicAdd(P.slab + 2, 1) != (int)gridDim.x - 1) return;
     __threadfence();
+    const double qC = atomicAdd(P.qsumd + 0, 0.0), qCq = atomicAdd(P.qsumd + 1, 0.0);
     for (int t = 0; t < 3; ++t) P.gtip[t] = (float)(P.tipd[t] * (double)P.nm);
-    P.gtip[3] = (float)((double)P.ke * atomicAdd(P.qsumd + 0, 0.0));
-    P.gtip[4] = P.Qzz != 0.f ? (float)(0.5 * (double)P.ke * atomicAdd(P.qsumd + 1, 0.0)) : 0.f;
+    P.gtip[3] = (float)((double)P.ke * qC);
+    P.gtip[4] = P.Qzz != 0.f ? (float)(0.5 * (double)P.ke * qCq) : 0.f;
+}
+
+// What the tile path reads of the adjoint grid must start at zero: the node layers K4 can touch and the
+// replicas' slots.  On grids far taller than the scan's band that is a fraction of the whole, so the band is
+// found from the positions first (a superset of what K4 touches; any position that is not a number: all layers).
+__global__ void __launch_bounds__(256) band_kernel(const BwdLaunch P) {
+    const int64_t total = (int64_t)P.snx * P.sny * P.snz;
+    float lo = 3.0e38f, hi = -3.0e38f;
+    bool bad = false;
+    // (eight loads in flight per thread: one at a time the flake's pass took 18 us)
+    const int64_t step = (int64_t)gridDim.x * 256;
+    for (int64_t o = (int64_t)blockIdx.x * 256 + threadIdx.x; o < total; o += 8 * step) {
+        float z[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) z[u] = __ldg(P.pos + 3 * (o + u * step < total ? o + u * step : o) + 2);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            bad |= !(fabsf(z[u]) < 3.0e38f);
+            lo = fminf(lo, z[u]);
+            hi = fmaxf(hi, z[u]);
+        }
+    }
+    // the layers of the extreme positions, by the lookup's own (monotone) arithmetic
+    int k0 = axis_cell(fmaf(lo, P.inv_dz, P.gz0s), P.map.nz, 0).i0, k1 = axis_cell(fmaf(hi, P.inv_dz, P.gz0s), P.map.nz, 0).i1;
+    if (lo > hi) k0 = P.map.nz, k1 = -1;  // a thread without points
+    if (bad) k0 = 0, k1 = P.map.nz - 1;
+    // (a block's bounds at once: two words shared by every warp's atomics took most of the pass)
+    __shared__ int b0, b1;
+    if (threadIdx.x == 0) b0 = P.map.nz, b1 = -1;
+    __syncthreads();
+    k0 = __reduce_min_sync(0xffffffffu, k0);
+    k1 = __reduce_max_sync(0xffffffffu, k1);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMin(&b0, k0);
+        atomicMax(&b1, k1);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && b1 >= b0) {
+        atomicMin(P.slab + 4, b0);
+        atomicMax(P.slab + 5, b1);
+    }
+}
+
+__global__ void __launch_bounds__(256) clear_band_kernel(const BwdLaunch P) {
+    const int64_t plane = (int64_t)P.map.nx * P.map.ny, slots = 7LL * P.n * P.replicas;
+    const int64_t first = P.slab[4] * plane, last = (P.slab[5] + 1LL) * plane;
+    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x, step = (int64_t)gridDim.x * 256;
+    for (int64_t g = t; g < slots; g += step) P.gbar[g] = z;
+    for (int64_t g = first + t; g < last; g += step) P.gbar[g] = z;
 }
 
 // s + t with the rounding error carried in c (Kahan): the f32x2 instructions are not reassociated.
@@ -1031,15 +1103,28 @@ cudaError_t launch_backward(const BwdLaunch& L0, cudaStream_t s) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t need = (total + kAdjThreads - 1) / kAdjThreads, most = (int64_t)kAdjCtas * sms;
     const int blocks = (int)(need < most ? (need > 0 ? need : 1) : most);
-    launch_adjoint(L, blocks, s);
     const int64_t nodes = (int64_t)L.map.nx * L.map.ny * L.map.nz;
     const dim3 tiles((L.map.nx + kTileN - 1) / kTileN, (L.map.ny + kTileN - 1) / kTileN,
                      kBwdParts * ((L.map.nz + kTileN - 1) / kTileN));
     // by tiles where K1 is, if the replicas fit the adjoint grid and the launch grid the tiles
-    if (!L.map.interp && ff_use_tiles(L.n, L.dx, L.dy, L.dz) && tiles.y <= 65535 && tiles.z <= 65535 &&
-        7 * (int64_t)L.n <= L.map.stored_nodes) {
+    const bool by_tiles = !L.map.interp && ff_use_tiles(L.n, L.dx, L.dy, L.dz) && tiles.y <= 65535 && tiles.z <= 65535 &&
+                          7 * (int64_t)L.n <= L.map.stored_nodes;
+    if (by_tiles) {
         L.replicas = 32;
         while (7 * (int64_t)L.n * L.replicas > L.map.stored_nodes) L.replicas >>= 1;
+    }
+    // the adjoint grid cleared: whole, or (linear grids from kBandBytes on) the band the scan reaches
+    const int64_t bytes = L.map.stored_nodes * (L.map.interp ? 4 : 16);
+    if (by_tiles && L.layout == 0 && bytes >= kBandBytes) {
+        const int64_t bb = (total + 255) / 256;
+        band_kernel<<<(int)(bb < 4LL * sms ? bb : 4LL * sms), 256, 0, s>>>(L);
+        clear_band_kernel<<<8 * sms, 256, 0, s>>>(L);
+    } else {
+        const cudaError_t e = cudaMemsetAsync(L.map.interp ? (void*)L.gbarE : (void*)L.gbar, 0, (size_t)bytes, s);
+        if (e != cudaSuccess) return e;
+    }
+    launch_adjoint(L, blocks, s);
+    if (by_tiles) {
         with_flags(L.min_image != 0, L.coul_rc > 0.f, L.Qzz != 0.f, [&](auto mi, auto cut, auto quad) {
             ff_backward_tile_kernel<decltype(mi)::value, decltype(cut)::value, decltype(quad)::value>
                 <<<tiles, kTileThreads, 0, s>>>(L);

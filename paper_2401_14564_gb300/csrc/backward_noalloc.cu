@@ -64,7 +64,7 @@ pp_status pp_backward_noalloc(const pp_atoms* atoms, const pp_probe* probe, cons
     void* ws = nullptr;
     st = scratch_address(&ws);
     if (st != PP_OK) return st;
-    return backward_launch("pp_backward_noalloc", L, ws, adj_bytes, (cudaStream_t)stream);
+    return backward_launch("pp_backward_noalloc", L, ws, (cudaStream_t)stream);
 }
 
 }  // extern "C"

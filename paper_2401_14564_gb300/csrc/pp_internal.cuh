@@ -230,7 +230,7 @@ pp_status backward_prepare(const std::string& who, const pp_atoms* atoms, const 
                            const float* ff, const pp_scan* scan, const pp_tip* tip, const pp_df* dfp,
                            const float* pos, const float* g_df, const pp_grads* grads, BwdLaunch* L,
                            size_t* adj_bytes);
-pp_status backward_launch(const std::string& who, BwdLaunch& L, void* ws, size_t adj_bytes, cudaStream_t s);
+pp_status backward_launch(const std::string& who, BwdLaunch& L, void* ws, cudaStream_t s);
 
 struct BatchArgs {
     const pp_mol_desc* descs;

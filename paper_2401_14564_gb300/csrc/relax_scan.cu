@@ -43,9 +43,11 @@ __device__ __forceinline__ int2 node_range(float a, float b, float inv_d, float 
 // x; each lane issues a bulk prefetch (a hint: it never faults and changes no
 // result) for every 32nd row.  Lateral deflections reach the neighbouring
 // tiles' rows, which those warps prefetch.
+template <bool kNarrow>
 __device__ __forceinline__ void prefetch_tile_slab(const RelaxLaunch& P, int tx, int ty, int lane) {
-    const int ia = tx << P.tile_wsh, ib = min(ia + (1 << P.tile_wsh), P.snx) - 1;
-    const int ja = ty << P.tile_hsh, jb = min(ja + (1 << P.tile_hsh), P.sny) - 1;
+    const int wsh = kNarrow ? P.tile_wsh : 3, hsh = kNarrow ? P.tile_hsh : 2;
+    const int ia = tx << wsh, ib = min(ia + (1 << wsh), P.snx) - 1;
+    const int ja = ty << hsh, jb = min(ja + (1 << hsh), P.sny) - 1;
     const int2 ri = node_range(fmaf((float)ia, P.spx, P.sx0) + P.d0x, fmaf((float)ib, P.spx, P.sx0) + P.d0x,
                                P.inv_dx, P.gx0s, P.map.nx);
     const int2 rj = node_range(fmaf((float)ja, P.spy, P.sy0) + P.d0y, fmaf((float)jb, P.spy, P.sy0) + P.d0y,
@@ -81,11 +83,13 @@ __device__ __forceinline__ void record_zspan(const RelaxLaunch& P, int2 span) {
 }
 
 // Lane l's pixel of tile (tx, ty), x fastest inside the tile; idle past its pixels.
+template <bool kNarrow>
 __device__ __forceinline__ void tile_pixel(const RelaxLaunch& P, int tx, int ty, int& i, int& j) {
-    const int lane = threadIdx.x, dj = lane >> P.tile_wsh;
-    i = (tx << P.tile_wsh) + (lane & ((1 << P.tile_wsh) - 1));
-    j = (ty << P.tile_hsh) + dj;
-    if (dj >> P.tile_hsh) i = P.snx;
+    const int wsh = kNarrow ? P.tile_wsh : 3, hsh = kNarrow ? P.tile_hsh : 2;
+    const int lane = threadIdx.x, dj = lane >> wsh;
+    i = (tx << wsh) + (lane & ((1 << wsh) - 1));
+    j = (ty << hsh) + dj;
+    if (kNarrow && (dj >> hsh)) i = P.snx;
 }
 
 // This warp's pixel (i, j); i = snx marks an idle lane.  Without a plan: lane l of the tile
@@ -93,12 +97,13 @@ __device__ __forceinline__ void tile_pixel(const RelaxLaunch& P, int tx, int ty,
 // plan_hblocks warps take the plan's listed pixels, plan_lanes lanes each (-1 or anything outside the
 // scan: idle), and warp plan_hblocks + t takes tile t less the listed pixels.  *tx < 0: no tile (no
 // slab prefetch).
+template <bool kNarrow>
 __device__ __forceinline__ void scan_pixel(const RelaxLaunch& P, int& i, int& j, int& tx, int& ty) {
     const int lane = threadIdx.x;
     if (!P.plan_list) {
         tx = blockIdx.x;
         ty = blockIdx.y;
-        tile_pixel(P, tx, ty, i, j);
+        tile_pixel<kNarrow>(P, tx, ty, i, j);
         return;
     }
     const int npix = P.snx * P.sny;
@@ -112,32 +117,33 @@ __device__ __forceinline__ void scan_pixel(const RelaxLaunch& P, int& i, int& j,
         j = ok ? p / P.snx : P.sny;
         return;
     }
-    const int ntx = (P.snx + (1 << P.tile_wsh) - 1) >> P.tile_wsh, t = b - P.plan_hblocks;
+    const int wsh = kNarrow ? P.tile_wsh : 3;
+    const int ntx = (P.snx + (1 << wsh) - 1) >> wsh, t = b - P.plan_hblocks;
     tx = t % ntx;
     ty = t / ntx;
-    tile_pixel(P, tx, ty, i, j);
+    tile_pixel<kNarrow>(P, tx, ty, i, j);
     if (i < P.snx && j < P.sny) {
         const int p = j * P.snx + i;
         if ((P.plan_mask[p >> 5] >> (p & 31)) & 1u) i = P.snx;  // run by a plan warp
     }
 }
 
-// kSpan: P.zspan is set and receives the node layers the lookups read.
-template <int LAYOUT, bool kPolish, bool kSpan>
+// kSpan: P.zspan is set and receives the node layers the lookups read.  kNarrow: tiles other than 8x4.
+template <int LAYOUT, bool kPolish, bool kSpan, bool kNarrow>
 __global__ void __launch_bounds__(kThreads) relax_scan_kernel(const RelaxLaunch P) {
     int i, j, tx, ty;
-    scan_pixel(P, i, j, tx, ty);
-    if (LAYOUT == 0 && tx >= 0) prefetch_tile_slab(P, tx, ty, threadIdx.x);
+    scan_pixel<kNarrow>(P, i, j, tx, ty);
+    if (LAYOUT == 0 && tx >= 0) prefetch_tile_slab<kNarrow>(P, tx, ty, threadIdx.x);
     const int2 span = relax_pixel<LAYOUT, false, false, false, kPolish, kSpan>(P, P, i, j);
     if constexpr (kSpan) record_zspan(P, span);
 }
 
 // Tricubic energy grid (linear layout).
-template <bool kPolish, bool kSpan>
+template <bool kPolish, bool kSpan, bool kNarrow>
 __global__ void __launch_bounds__(kThreads) relax_scan_tricubic_kernel(const RelaxLaunch P) {
     int i, j, tx, ty;
-    scan_pixel(P, i, j, tx, ty);
-    if (tx >= 0) prefetch_tile_slab(P, tx, ty, threadIdx.x);
+    scan_pixel<kNarrow>(P, i, j, tx, ty);
+    if (tx >= 0) prefetch_tile_slab<kNarrow>(P, tx, ty, threadIdx.x);
     const int2 span = relax_pixel<0, false, true, false, kPolish, kSpan>(P, P, i, j);
     if constexpr (kSpan) record_zspan(P, span);
 }
@@ -166,11 +172,17 @@ void tile_shape(RelaxLaunch& L, int sms) {
     }
 }
 
+template <bool kPolish, bool kSpan, bool kNarrow>
+void launch_relax_scan_n(const RelaxLaunch& L, dim3 grid, cudaStream_t s) {
+    if (L.map.interp == 1) relax_scan_tricubic_kernel<kPolish, kSpan, kNarrow><<<grid, kThreads, 0, s>>>(L);
+    else if (L.layout == 0) relax_scan_kernel<0, kPolish, kSpan, kNarrow><<<grid, kThreads, 0, s>>>(L);
+    else relax_scan_kernel<1, kPolish, kSpan, kNarrow><<<grid, kThreads, 0, s>>>(L);
+}
+
 template <bool kPolish, bool kSpan>
 void launch_relax_scan_t(const RelaxLaunch& L, dim3 grid, cudaStream_t s) {
-    if (L.map.interp == 1) relax_scan_tricubic_kernel<kPolish, kSpan><<<grid, kThreads, 0, s>>>(L);
-    else if (L.layout == 0) relax_scan_kernel<0, kPolish, kSpan><<<grid, kThreads, 0, s>>>(L);
-    else relax_scan_kernel<1, kPolish, kSpan><<<grid, kThreads, 0, s>>>(L);
+    if (L.tile_wsh == 3 && L.tile_hsh == 2) launch_relax_scan_n<kPolish, kSpan, false>(L, grid, s);
+    else launch_relax_scan_n<kPolish, kSpan, true>(L, grid, s);
 }
 
 }  // namespace

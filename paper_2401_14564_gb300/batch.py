@@ -1,4 +1,4 @@
-"""Many molecules in one persistent launch (pp_batch_run), optionally replayed from a CUDA graph.
+"""Many molecules in one call of persistent kernels (pp_batch_run), optionally replayed from a CUDA graph.
 
 `Batch` packs a list of workload dicts (same probe, tip, FIRE, df settings,
 scan height step and periodic flag; any grid and scan sizes) into device
@@ -23,7 +23,7 @@ class Batch:
     def __init__(self, cases, device="cuda", want_pos=False, want_iters=True, ctas=0, fire=None,
                  spin_limit=0, wait_extra=0, ff_energy=True, ff_zpt=0, ff_tile_w=0, relax_tile_w=0):
         """ff_energy=False skips the energy sums of every molecule's grid (E slots 0; the scan
-        outputs are unchanged).  ff_zpt, ff_tile_w, relax_tile_w and ctas set the work-item
+        outputs are unchanged).  ff_zpt and ff_tile_w are accepted and without effect; relax_tile_w and ctas set the work-item
         shapes and the persistent CTA count (0: defaults; tune.tune_batch picks them)."""
         if not cases:
             raise ValueError("empty batch")

@@ -1,4 +1,6 @@
-// K1: force-field grid assembly (Sec. 5.1.1 step 1).
+// K1: force-field grid assembly (Sec. 5.1.1 step 1), direct sums: for split grids, samples of fewer than 16
+// atoms and spacings above 0.35 A; everything else is assembled by tiles (ff_tile.cu, where the line lies and why
+// is said at ff_use_tiles in ff_tile.cuh).
 //
 // Every node g of the grid gets F_g = sum_i S_i(r) (r_g - r_i) and
 // E_g = sum_i E_i(r), with, for atom i and the probe particle,
@@ -169,7 +171,7 @@ cudaError_t launch_ff_assemble(const FFLaunch& L, cudaStream_t s) {
         });
         return cudaGetLastError();
     }
-    if (ff_use_tiles(L.n, L.dx, L.dy, L.dz)) return launch_ff_tiles(L, s);
+    if (ff_use_tiles(L.n, L.dx, L.dy, L.dz)) return launch_ff_tiles(L, s);  // (zpt is the direct kernel's)
     if (L.map.interp == 1) {
         constexpr int ZPT = 8;
         dim3 grid((L.map.nx + kTileX - 1) / kTileX, (L.map.ny + kTileY - 1) / kTileY, (L.kend - L.kbeg + ZPT - 1) / ZPT);

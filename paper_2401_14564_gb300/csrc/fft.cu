@@ -24,6 +24,7 @@
 // exchange through shared memory.
 #include <cuda_runtime.h>
 
+#include "fft_layout.cuh"
 #include "pp_internal.cuh"
 
 namespace pp {
@@ -224,17 +225,13 @@ __device__ __forceinline__ void fft_lines(int log2nl, float2* x, const float2* t
     }
 }
 
-// Layouts of the scratch: the full spectrum z, node (i, j, k) at k pz + j px + i with px = nx + 16 and
-// pz = px ny + 16; the half spectra (i <= nx/2) at k hz + j hx + i.  The y and z strides are then not
-// powers of two (a power-of-two stride sends every row of a pass to the same memory channels).  Of the
-// three full arrays' room (fft_workspace_bytes), z has the first and the half arrays a = P and b = -i kz P the
-// end; once z is spent, c = E, d = Fy and e = Fz along x take its place and the gap (5 halves fit 3 wholes).
+// What the kernels get; pitches and lengths as in fft_layout.cuh.
 struct Plan {
     const float *f, *g;
     float4* ff;
     float2 *z, *a, *b, *c, *d, *e;
     int nx, ny, nz;
-    int px, pz, hx, hz, zlen, hlen;  // (1040 x 1024 + 16 times 1024 complex values at most: offsets fit 32 bits)
+    int px, pz, hx, hz, zlen, hlen;
     float kx0, ky0, kz0;  // 2 pi / (n d) per axis
     float norm;           // scale * dV / N
     float power;
@@ -456,37 +453,27 @@ cudaError_t with_log2(int n, F&& f) {
     }
 }
 
-void make_layout(int nx, int ny, int nz, Plan* P) {
-    P->nx = nx; P->ny = ny; P->nz = nz;
-    P->px = nx + 16;
-    P->pz = P->px * ny + 16;
-    // (below 64 nodes along x the narrower pitch keeps five halves inside three wholes)
-    P->hx = nx / 2 + (nx >= 64 ? 16 : 2);
-    P->hz = P->hx * ny + 8;
-    P->zlen = P->pz * nz;
-    P->hlen = P->hz * nz;
-}
-
 }  // namespace
 
 size_t fft_workspace_bytes(int nx, int ny, int nz) {
-    Plan P;
-    make_layout(nx, ny, nz, &P);
-    return (size_t)3 * (size_t)P.zlen * sizeof(float2);
+    return (size_t)fft_layout(nx, ny, nz).size * sizeof(float2);
 }
 
 cudaError_t launch_fft_correlate(const FftLaunch& L, cudaStream_t s) {
     Plan P;
-    make_layout(L.nx, L.ny, L.nz, &P);
+    const FftLayout at = fft_layout(L.nx, L.ny, L.nz);
+    P.nx = L.nx; P.ny = L.ny; P.nz = L.nz;
+    P.px = at.px; P.pz = at.pz; P.hx = at.hx; P.hz = at.hz;
+    P.zlen = at.zlen; P.hlen = at.hlen;
     P.f = L.f;
     P.g = L.g;
     P.ff = L.ff;
     P.z = reinterpret_cast<float2*>(L.ws);
-    P.a = P.z + 3 * P.zlen - 2 * P.hlen;
-    P.b = P.a + P.hlen;
-    P.c = P.z;
-    P.d = P.c + P.hlen;
-    P.e = P.d + P.hlen;
+    P.a = P.z + at.a;
+    P.b = P.z + at.b;
+    P.c = P.z + at.c;
+    P.d = P.z + at.d;
+    P.e = P.z + at.e;
     P.kx0 = (float)(2.0 * kPi / (L.nx * (double)L.dx));
     P.ky0 = (float)(2.0 * kPi / (L.ny * (double)L.dy));
     P.kz0 = (float)(2.0 * kPi / (L.nz * (double)L.dz));

@@ -117,11 +117,12 @@ __device__ __forceinline__ bool tile_far(const FFConst& c, float rx, float ry, f
     const float ax = fabsf(rx), ay = fabsf(ry), az = fabsf(rz);
     const float d2 = __fmaf_rn(rx, rx, __fmaf_rn(ry, ry, __fmul_rn(rz, rz)));
     const float Rij = __fadd_rn(R, c.R_pp);
-    const float reach = fmaxf(__fmul_rn(10.f, hmax), __fmul_rn(1.75f, Rij));
+    // (the pair terms and the core floor take R_iPP squared: a sum below zero reaches as far)
+    const float reach = fmaxf(__fmul_rn(10.f, hmax), __fmul_rn(1.75f, fabsf(Rij)));
     *charged = true;
-    // (a non-finite coordinate or radius compares false: near, as the direct sum has it)
+    // (a coordinate, radius, depth or charge that is not finite: near, as the direct sum has it)
     if (!(d2 >= __fmul_rn(reach, reach)) || !(d2 < 3.0e38f)) return false;
-    if (!(fabsf(q) < 3.0e38f) || !(fabsf(eps) < 3.0e38f)) return false;
+    if (!(fabsf(Rij) < 3.0e38f) || !(fabsf(q) < 3.0e38f) || !(fabsf(eps) < 3.0e38f)) return false;
     if (kMinImage) {
         // some node of the tile sees another image of the atom
         if (!(__fadd_rn(ax, hx) < __fmul_rn(0.4999f, c.Lx)) || !(__fadd_rn(ay, hy) < __fmul_rn(0.4999f, c.Ly))) return false;
@@ -184,11 +185,11 @@ __device__ __forceinline__ void ff_tile(const TileJob& J, const FFConst& c, int 
         float xl, yl, zl;
         bool live, far, charged;
     };
-    // atom minus centre as a float pair
+    // atom minus centre as a float pair (an infinite difference has no low part: its error term is not a number)
     auto rel = [](float a, float2 ctr, float& hi, float& lo) {
         float e;
         two_sum(a, -ctr.x, hi, e);
-        lo = __fsub_rn(e, ctr.y);
+        lo = fabsf(hi) < 3.4e38f ? __fsub_rn(e, ctr.y) : 0.f;
     };
     auto load = [&](int a) {
         Atom t;

@@ -161,13 +161,15 @@ __device__ __forceinline__ int tile_slot(bool keep, int* count, int* total) {
 
 // Assembles the nodes of the tile at node (i0, j0, k0) (multiples of 16) and hands each thread's columns
 // to `store(i, j, k, fx, fy, fz, en)`: node pairs (k, k + 1) of column (i, j) as packed pairs, for the
-// layers k0 + 8 h .. k0 + 8 h + 7 of each half h with want_half(h).  Every thread of the CTA calls.
+// tile's quarters [q0, q1) of 4 layers each and maybe others of the tile.  kMost: at most that many are asked for, 2
+// or 4; kThin: one or two anywhere get no more than they ask for, otherwise the unit is a half (the kernel that can do
+// both is 3 % slower on whole grids).  Every thread of the CTA calls.
 // A thread owns a column of 16 nodes, so that an atom's lateral terms and the interpolation along y
 // are formed once for all of them (the two halves in turn, at fewer registers and three CTAs an SM: 0.142
 // against 0.135 ms on the 60-atom flake, 24.2 against 22.2 ms on the slab).
-template <bool kMinImage, bool kCutoff, bool kQuad, bool kEnergy, bool kForcesOnly, class Want, class Store>
-__device__ __forceinline__ void ff_tile(const TileJob& J, const FFConst& c, int i0, int j0, int k0, TileShared& S,
-                                        Want&& want_half, Store&& store) {
+template <bool kMinImage, bool kCutoff, bool kQuad, bool kEnergy, bool kForcesOnly, int kMost, bool kThin, class Store>
+__device__ __forceinline__ void ff_tile(const TileJob& J, const FFConst& c, int i0, int j0, int k0, int q0, int q1,
+                                        TileShared& S, Store&& store) {
     constexpr int P3 = kTileP * kTileP * kTileP;
     const int tid = threadIdx.x;
     const float2 cx = tile_centre(J.x0, i0, J.dx), cy = tile_centre(J.y0, j0, J.dy), cz = tile_centre(J.z0, k0, J.dz);
@@ -333,7 +335,7 @@ __device__ __forceinline__ void ff_tile(const TileJob& J, const FFConst& c, int 
 #pragma unroll
         for (int m = 0; m < kTileP; ++m) wy[m] = g_tile.w[j][m];
     }
-    // ZP node pairs from layer k0 + first: both halves at once, or the one half that is wanted
+    // ZP node pairs from layer k0 + first
     auto column = [&](auto zp, int first) {
         constexpr int ZP = decltype(zp)::value;
         float2 fx[ZP], fy[ZP], fz[ZP], en[ZP], gz[ZP];
@@ -380,9 +382,18 @@ __device__ __forceinline__ void ff_tile(const TileJob& J, const FFConst& c, int 
 #pragma unroll
         for (int t = 0; t < ZP; ++t) store(i0 + i, j0 + j, k0 + first + 2 * t, fx[t], fy[t], fz[t], en[t]);
     };
-    if (want_half(0) && want_half(1)) column(std::integral_constant<int, 8>{}, 0);
-    else if (want_half(0)) column(std::integral_constant<int, 4>{}, 0);
-    else if (want_half(1)) column(std::integral_constant<int, 4>{}, 8);
+    const std::integral_constant<int, 8> whole;
+    const std::integral_constant<int, 4> half_tile;
+    const std::integral_constant<int, 2> quarter;
+    if constexpr (kThin) {
+        if (kMost > 2 && q1 - q0 > 2) column(whole, 0);
+        else if (q1 - q0 == 2) column(half_tile, 4 * q0);
+        else column(quarter, 4 * q0);
+    } else {
+        if (kMost > 2 && q0 < 2 && q1 > 2) column(whole, 0);
+        else if (q0 < 2) column(half_tile, 0);
+        else column(half_tile, 8);
+    }
     __syncthreads();  // the shared buffers may be reused
 }
 

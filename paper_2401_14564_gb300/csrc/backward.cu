@@ -1106,8 +1106,8 @@ cudaError_t launch_backward(const BwdLaunch& L0, cudaStream_t s) {
     const int64_t nodes = (int64_t)L.map.nx * L.map.ny * L.map.nz;
     const dim3 tiles((L.map.nx + kTileN - 1) / kTileN, (L.map.ny + kTileN - 1) / kTileN,
                      kBwdParts * ((L.map.nz + kTileN - 1) / kTileN));
-    // by tiles where K1 is, if the replicas fit the adjoint grid and the launch grid the tiles
-    const bool by_tiles = !L.map.interp && ff_use_tiles(L.n, L.dx, L.dy, L.dz) && tiles.y <= 65535 && tiles.z <= 65535 &&
+    // by tiles where K1 can be, if the replicas fit the adjoint grid and the launch grid the tiles
+    const bool by_tiles = !L.map.interp && ff_tiles_possible(L.n, L.dx, L.dy, L.dz) && tiles.y <= 65535 && tiles.z <= 65535 &&
                           7 * (int64_t)L.n <= L.map.stored_nodes;
     if (by_tiles) {
         L.replicas = 32;

@@ -183,18 +183,25 @@ struct MolStore {
     }
 };
 
-// Direct sums (grids not assembled by tiles, see ff_use_tiles) of 8 layers from k0 of the 8x4 columns from
-// (i0, j0), by one warp: the arithmetic of ff_assemble.cu.  st: 4 x 32 records.
+// Direct sums (grids not assembled by tiles, see ff_path) of 8 layers from k0 of the 8x4 columns from
+// (i0, j0), by one warp: the arithmetic of ff_assemble.cu, with `centre` relative to the centre of the tile at
+// (it, jt, kt).  st: 4 x 32 records.
 template <bool kMinImage, bool kCutoff, bool kQuad, class Store>
 __device__ __forceinline__ void ff_direct(const BatchLaunch& B, const pp_mol_desc& D, const FFConst& cst, int i0, int j0,
-                                          int k0, float4* st, Store&& store) {
+                                          int k0, bool centre, int it, int jt, int kt, float4* st, Store&& store) {
     constexpr int ZP = 4;
+    constexpr float half = 0.5f * (kTileN - 1);
     const int lane = threadIdx.x & 31, i = i0 + (lane & 7), j = j0 + (lane >> 3);
-    const float gx = D.x0 + i * D.dx, gy = D.y0 + j * D.dy;
+    if (!kMinImage) centre = false;
+    const float gx = centre ? __fmul_rn((float)(i - it) - half, D.dx) : D.x0 + i * D.dx;
+    const float gy = centre ? __fmul_rn((float)(j - jt) - half, D.dy) : D.y0 + j * D.dy;
+    const float2 cx = tile_centre(D.x0, it, D.dx), cy = tile_centre(D.y0, jt, D.dy), cz = tile_centre(D.z0, kt, D.dz);
     float2 gz[ZP], fx[ZP], fy[ZP], fz[ZP], en[ZP];
 #pragma unroll
     for (int t = 0; t < ZP; ++t) {
-        gz[t] = make_float2(D.z0 + (k0 + 2 * t) * D.dz, D.z0 + (k0 + 2 * t + 1) * D.dz);
+        const int k = k0 + 2 * t;
+        gz[t] = centre ? make_float2(__fmul_rn((float)(k - kt) - half, D.dz), __fmul_rn((float)(k + 1 - kt) - half, D.dz))
+                       : make_float2(D.z0 + k * D.dz, D.z0 + (k + 1) * D.dz);
         fx[t] = fy[t] = fz[t] = en[t] = make_float2(0.f, 0.f);
     }
     for (int base = 0; base < D.n_atoms; base += 32) {
@@ -202,8 +209,13 @@ __device__ __forceinline__ void ff_direct(const BatchLaunch& B, const pp_mol_des
         __syncwarp();
         if (lane < cnt) {
             const int g = D.atom_offset + base + lane;
-            ff_stage_atom(cst, B.ax[g], B.ay[g], B.az[g], B.aR[g], B.aeps[g], B.aq[g], st[lane], st[32 + lane],
-                          st[64 + lane], st[96 + lane]);
+            float x = B.ax[g], y = B.ay[g], z = B.az[g];
+            if (kMinImage && centre) {
+                x = wrap_image(centred(x, cx), cst.Lx, cst.invLx);
+                y = wrap_image(centred(y, cy), cst.Ly, cst.invLy);
+                z = centred(z, cz);
+            }
+            ff_stage_atom(cst, x, y, z, B.aR[g], B.aeps[g], B.aq[g], st[lane], st[32 + lane], st[64 + lane], st[96 + lane]);
         }
         __syncwarp();
         ff_accumulate<ZP, kMinImage, kCutoff, kQuad, true>(st, st + 32, st + 64, st + 96, cnt, cst, gx, gy, gz, fx, fy, fz,
@@ -234,7 +246,8 @@ __global__ void __launch_bounds__(kTileThreads, 2) batch_ff_kernel(const BatchLa
         const FFConst cst = ff_const(B.R_pp, B.eps_pp, B.kQ, B.core_frac, D.nx * D.dx, D.ny * D.dy,
                                      kCutoff ? B.coul_rc : 0.f, kQuad ? B.kQzz : 0.f);
         const MolStore<kForcesOnly> store{B, D};
-        if (ff_use_tiles(D.n_atoms, D.dx, D.dy, D.dz)) {
+        const FFPath path = ff_path(D.n_atoms, D.nx, D.ny, D.nz, D.dx, D.dy, D.dz, kMinImage, false);
+        if (path == FFPath::kTiles) {
             const int a = D.atom_offset;
             const TileJob J = {B.ax + a, B.ay + a, B.az + a, B.aR + a, B.aeps + a, B.aq + a, D.n_atoms,
                                D.x0, D.y0, D.z0, D.dx, D.dy, D.dz, D.nx, D.ny};
@@ -245,7 +258,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) batch_ff_kernel(const BatchLa
             for (int h = 0; h < 2; ++h)
                 if (k0 + 8 * h < D.nz)
                     ff_direct<kMinImage, kCutoff, kQuad>(B, D, cst, i0 + (warp & 1) * 8, j0 + (warp >> 1) * 4, k0 + 8 * h,
-                                                         S.buf + warp * 128, store);
+                                                         path == FFPath::kCentred, i0, j0, k0, S.buf + warp * 128, store);
         }
         __threadfence();
         __syncthreads();

@@ -1,6 +1,6 @@
 // K1: force-field grid assembly (Sec. 5.1.1 step 1), direct sums: for split grids, samples of fewer than 16
-// atoms and spacings above 0.35 A; everything else is assembled by tiles (ff_tile.cu, where the line lies and why
-// is said at ff_use_tiles in ff_tile.cuh).
+// atoms, spacings above 0.35 A, and grids of whose atoms hardly any is far from a tile; everything else is assembled by
+// tiles (ff_tile.cu; where the lines lie and why is said at ff_path in ff_tile.cuh).
 //
 // Every node g of the grid gets F_g = sum_i S_i(r) (r_g - r_i) and
 // E_g = sum_i E_i(r), with, for atom i and the probe particle,
@@ -45,8 +45,10 @@ constexpr int kChunk = 256;  // atoms staged per pass
 // kForcesOnly: E slots written as 0; the energy sums are never formed (3 of
 // the 15 packed FP32 operations per pair of nodes), the force sums are
 // unchanged.
+// kCentred: coordinates relative to the centre of the 16x16x16-node tile around, on periodic cells (ff_path in
+// ff_tile.cuh); blocks of layers start at multiples of ZPT whatever range is asked for.
 template <int ZPT, bool kMinImage, bool kCutoff, bool kQuad, bool kEnergy = false, bool kSplit = false,
-          bool kForcesOnly = false>
+          bool kForcesOnly = false, bool kCentred = false>
 __global__ void __launch_bounds__(kThreads) ff_assemble_kernel(const FFLaunch P) {
     static_assert(ZPT % 2 == 0, "z-nodes come in packed pairs");
     constexpr int ZP = ZPT / 2;
@@ -56,13 +58,26 @@ __global__ void __launch_bounds__(kThreads) ff_assemble_kernel(const FFLaunch P)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i = blockIdx.x * kTileX + (warp & 1) * 8 + (lane & 7);
     const int j = blockIdx.y * kTileY + (warp >> 1) * 4 + (lane >> 3);
-    const int k0 = P.kbeg + blockIdx.z * ZPT;
+    const int k0 = kCentred ? (P.kbeg / ZPT + (int)blockIdx.z) * ZPT : P.kbeg + blockIdx.z * ZPT;
 
-    const float gx = P.x0 + i * P.dx;
-    const float gy = P.y0 + j * P.dy;
+    static_assert(!kCentred || (kMinImage && kTileX == kTileN && kTileN % kTileY == 0 && kTileN % ZPT == 0), "a block lies in one tile");
+    const int it = blockIdx.x * kTileX, jt = blockIdx.y * kTileY / kTileN * kTileN, kt = k0 / kTileN * kTileN;
+    constexpr float half = 0.5f * (kTileN - 1);
+    float2 cx, cy, cz;  // the tile's centre as float pairs
+    if (kCentred) {
+        cx = tile_centre(P.x0, it, P.dx);
+        cy = tile_centre(P.y0, jt, P.dy);
+        cz = tile_centre(P.z0, kt, P.dz);
+    }
+    const float gx = kCentred ? __fmul_rn((float)(i - it) - half, P.dx) : P.x0 + i * P.dx;
+    const float gy = kCentred ? __fmul_rn((float)(j - jt) - half, P.dy) : P.y0 + j * P.dy;
     float2 gz[ZP];
 #pragma unroll
-    for (int t = 0; t < ZP; ++t) gz[t] = make_float2(P.z0 + (k0 + 2 * t) * P.dz, P.z0 + (k0 + 2 * t + 1) * P.dz);
+    for (int t = 0; t < ZP; ++t) {
+        const int k = k0 + 2 * t;
+        if (kCentred) gz[t] = make_float2(__fmul_rn((float)(k - kt) - half, P.dz), __fmul_rn((float)(k + 1 - kt) - half, P.dz));
+        else gz[t] = make_float2(P.z0 + k * P.dz, P.z0 + (k + 1) * P.dz);
+    }
 
     float2 fx[ZP], fy[ZP], fz[ZP], en[ZP];
     float2 fxe[ZP], fye[ZP], fze[ZP], ene[ZP];  // kSplit only
@@ -76,7 +91,13 @@ __global__ void __launch_bounds__(kThreads) ff_assemble_kernel(const FFLaunch P)
         __syncthreads();
         for (int a = threadIdx.x; a < cnt; a += kThreads) {
             const int g = base + a;
-            ff_stage_atom(cst, P.x[g], P.y[g], P.z[g], P.R[g], P.eps[g], P.q[g], s0[a], s1[a], s2[a], s3[a]);
+            float x = P.x[g], y = P.y[g], z = P.z[g];
+            if (kCentred) {
+                x = wrap_image(centred(x, cx), cst.Lx, cst.invLx);
+                y = wrap_image(centred(y, cy), cst.Ly, cst.invLy);
+                z = centred(z, cz);
+            }
+            ff_stage_atom(cst, x, y, z, P.R[g], P.eps[g], P.q[g], s0[a], s1[a], s2[a], s3[a]);
         }
         __syncthreads();
         // every thread of the block runs this (out-of-grid columns return only after it): the warp vote is safe
@@ -87,12 +108,13 @@ __global__ void __launch_bounds__(kThreads) ff_assemble_kernel(const FFLaunch P)
     if (i >= P.map.nx || j >= P.map.ny) return;
     const int base_xy = axis_off(P.map.ax, i) + axis_off(P.map.ay, j);
     auto at = [&](int k) { return checked(base_xy + axis_off(P.map.az, k), P.map.stored_nodes, kChkGridWrite); };
+    auto wanted = [&](int k) { return k < P.kend && (!kCentred || k >= P.kbeg); };
     if constexpr (kEnergy) {
 #pragma unroll
         for (int t = 0; t < ZP; ++t) {
             const int k = k0 + 2 * t;
-            if (k < P.kend) P.ffE[at(k)] = en[t].x;
-            if (k + 1 < P.kend) P.ffE[at(k + 1)] = en[t].y;
+            if (wanted(k)) P.ffE[at(k)] = en[t].x;
+            if (wanted(k + 1)) P.ffE[at(k + 1)] = en[t].y;
             if constexpr (kSplit) {
                 if (k < P.kend) P.ffelE[at(k)] = ene[t].x;
                 if (k + 1 < P.kend) P.ffelE[at(k + 1)] = ene[t].y;
@@ -103,8 +125,8 @@ __global__ void __launch_bounds__(kThreads) ff_assemble_kernel(const FFLaunch P)
         for (int t = 0; t < ZP; ++t) {
             const int k = k0 + 2 * t;
             const float2 e = kForcesOnly ? make_float2(0.f, 0.f) : en[t];
-            if (k < P.kend) P.ff[at(k)] = make_float4(fx[t].x, fy[t].x, fz[t].x, e.x);
-            if (k + 1 < P.kend) P.ff[at(k + 1)] = make_float4(fx[t].y, fy[t].y, fz[t].y, e.y);
+            if (wanted(k)) P.ff[at(k)] = make_float4(fx[t].x, fy[t].x, fz[t].x, e.x);
+            if (wanted(k + 1)) P.ff[at(k + 1)] = make_float4(fx[t].y, fy[t].y, fz[t].y, e.y);
             if constexpr (kSplit) {
                 if (k < P.kend)
                     P.ffel[at(k)] = make_float4(fxe[t].x, fye[t].x, fze[t].x, ene[t].x);
@@ -144,6 +166,42 @@ cudaError_t launch_zpt(const FFLaunch& L, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+template <int ZPT>
+cudaError_t launch_centred_zpt(const FFLaunch& L, cudaStream_t s) {
+    dim3 grid((L.map.nx + kTileX - 1) / kTileX, (L.map.ny + kTileY - 1) / kTileY,
+              (L.kend + ZPT - 1) / ZPT - L.kbeg / ZPT);
+    with_flags(true, L.coul_rc > 0.f, L.kQzz != 0.f, [&](auto, auto cut, auto quad) {
+        constexpr bool CUT = decltype(cut)::value, QUAD = decltype(quad)::value;
+        if (L.map.interp == 1) ff_assemble_kernel<ZPT, true, CUT, QUAD, true, false, false, true><<<grid, kThreads, 0, s>>>(L);
+        else if (L.forces_only) ff_assemble_kernel<ZPT, true, CUT, QUAD, false, false, true, true><<<grid, kThreads, 0, s>>>(L);
+        else ff_assemble_kernel<ZPT, true, CUT, QUAD, false, false, false, true><<<grid, kThreads, 0, s>>>(L);
+        return 0;
+    });
+    return cudaGetLastError();
+}
+
+// Whether the last 4 layers or fewer of a range are worth a launch of their own beside blocks of `zpt` layers: only
+// once the blocks exceed 8 to an SM (320-atom sheet on 136x327x34 nodes 485 us in one launch, 455 in two; 21 atoms on 56x81x46
+// 10 in one, 18 in two), and not for energies (468 atoms on 111x244x41 358 and 393).
+bool tail_apart(const FFLaunch& L, int zblocks) {
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t xy = (int64_t)((L.map.nx + kTileX - 1) / kTileX) * ((L.map.ny + kTileY - 1) / kTileY);
+    return L.map.interp != 1 && xy * zblocks > 8LL * sms;
+}
+
+// Blocks of 8 layers at multiples of 8.
+cudaError_t launch_centred(const FFLaunch& L, cudaStream_t s) {
+    if ((L.kend - 1) / 4 == L.kbeg / 4) return launch_centred_zpt<4>(L, s);
+    FFLaunch bulk = L, tail = L;
+    const int r = (L.kend - 1) % 8 + 1;
+    if (r > 4 || L.kend - r <= L.kbeg || !tail_apart(L, (L.kend + 7) / 8 - L.kbeg / 8)) return launch_centred_zpt<8>(L, s);
+    bulk.kend = tail.kbeg = L.kend - r;
+    const cudaError_t e = launch_centred_zpt<8>(bulk, s);
+    return e != cudaSuccess ? e : launch_centred_zpt<4>(tail, s);
+}
+
 }  // namespace
 
 cudaError_t launch_ff_combine(const float* a, const float* b, float Q, float* out, int64_t nfloats, cudaStream_t s) {
@@ -171,7 +229,12 @@ cudaError_t launch_ff_assemble(const FFLaunch& L, cudaStream_t s) {
         });
         return cudaGetLastError();
     }
-    if (ff_use_tiles(L.n, L.dx, L.dy, L.dz)) return launch_ff_tiles(L, s);  // (zpt is the direct kernel's)
+    // (zpt is the plain direct kernel's)
+    switch (ff_path(L.n, L.map.nx, L.map.ny, L.map.nz, L.dx, L.dy, L.dz, L.min_image != 0, L.map.interp == 1)) {
+        case FFPath::kTiles: return launch_ff_tiles(L, s);
+        case FFPath::kCentred: return launch_centred(L, s);
+        case FFPath::kDirect: break;
+    }
     if (L.map.interp == 1) {
         constexpr int ZPT = 8;
         dim3 grid((L.map.nx + kTileX - 1) / kTileX, (L.map.ny + kTileY - 1) / kTileY, (L.kend - L.kbeg + ZPT - 1) / ZPT);
@@ -186,7 +249,7 @@ cudaError_t launch_ff_assemble(const FFLaunch& L, cudaStream_t s) {
     // multiple of zpt (nz = 200 at 16: 13 x 16 = 208, 4 % of the arithmetic); those r layers go to a
     // second launch of a narrower shape instead (each node's sums are the same in every shape).
     const int zpt = (L.zpt == 4 || L.zpt == 16) ? L.zpt : 8;
-    const int n = L.kend - L.kbeg, bulk = n - n % zpt, r = n - bulk;
+    const int n = L.kend - L.kbeg, r = n <= 4 || tail_apart(L, (n + zpt - 1) / zpt) ? n % zpt : 0, bulk = n - r;
     FFLaunch head = L, tail = L;
     head.kend = L.kbeg + bulk;
     tail.kbeg = L.kbeg + bulk;

@@ -9,10 +9,11 @@
 namespace pp {
 namespace {
 
-// Grids of fewer tiles than CTAs fit the GPU (two per SM) run by halves: 48 tiles of a 40-atom molecule 27 -> 18
-// us, 196 of a 120-atom periodic sheet 144 -> 115 us (direct sums: 119); with more tiles the far sums made twice cost more than
-// the better balance gives (780 tiles of an 80-atom molecule 60 -> 79 us).
-constexpr int kHalfTiles = 2;
+// Grids of fewer tiles than CTAs fit the GPU (two per SM), or of a few more, which a second wave of a few tiles ends,
+// run by halves: 48 tiles of a 40-atom molecule 27 -> 18 us, 196 of a 120-atom periodic sheet 144 -> 115 us, 308 of 67
+// atoms 53 -> 39, 324 of 492 atoms 361 -> 297; with more tiles the far sums made twice cost more than the better
+// balance gives (490 tiles of 407 atoms 109 -> 154, 780 of an 80-atom molecule 60 -> 79 us).  By quarters no grid ran faster.
+constexpr int kHalfFifths = 11;  // 2.2 tiles per SM
 
 // kEnergy: E alone, one float per node (tricubic grids).  kForcesOnly: E slots written as 0.
 // kParts: CTAs to a tile (1 or 2), which share its layers (all sum the far atoms).  A tile over a molecule has
@@ -57,7 +58,7 @@ cudaError_t launch_ff_tiles(const FFLaunch& L, cudaStream_t s) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t tiles = (int64_t)grid.x * grid.y * grid.z;
-    const int parts = tiles < (int64_t)kHalfTiles * sms ? 2 : 1;
+    const int parts = 5 * tiles < (int64_t)kHalfFifths * sms ? 2 : 1;
     grid.z *= parts;
     const bool thin = L.kbeg % 8 != 0 || (L.kend % 8 != 0 && L.kend != L.map.nz);
     with_flags(L.min_image != 0, L.coul_rc > 0.f, L.kQzz != 0.f, [&](auto mi, auto cut, auto quad) {

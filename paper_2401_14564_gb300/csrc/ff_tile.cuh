@@ -106,6 +106,21 @@ __device__ __forceinline__ float2 tile_centre(float origin, int first, float d) 
     return make_float2(s, __fadd_rn(e, pl));
 }
 
+// An atom's coordinate relative to the centre as a float pair (an infinite difference has no low part: its error term
+// is not a number).
+__device__ __forceinline__ void tile_rel(float a, float2 ctr, float& hi, float& lo) {
+    float e;
+    two_sum(a, -ctr.x, hi, e);
+    lo = fabsf(hi) < 3.4e38f ? __fsub_rn(e, ctr.y) : 0.f;
+}
+
+// The same rounded once.
+__device__ __forceinline__ float centred(float a, float2 ctr) {
+    float hi, lo;
+    tile_rel(a, ctr, hi, lo);
+    return __fadd_rn(hi, lo);
+}
+
 __device__ __forceinline__ float wrap_image(float d, float L, float invL) { return __fmaf_rn(-L, rintf(__fmul_rn(d, invL)), d); }
 
 // Whether the atom at (rx, ry, rz) from the tile's centre is summed at the interpolation points; on true,
@@ -187,12 +202,6 @@ __device__ __forceinline__ void ff_tile(const TileJob& J, const FFConst& c, int 
         float xl, yl, zl;
         bool live, far, charged;
     };
-    // atom minus centre as a float pair (an infinite difference has no low part: its error term is not a number)
-    auto rel = [](float a, float2 ctr, float& hi, float& lo) {
-        float e;
-        two_sum(a, -ctr.x, hi, e);
-        lo = fabsf(hi) < 3.4e38f ? __fsub_rn(e, ctr.y) : 0.f;
-    };
     auto load = [&](int a) {
         Atom t;
         t.live = a < J.n;
@@ -200,9 +209,9 @@ __device__ __forceinline__ void ff_tile(const TileJob& J, const FFConst& c, int 
         t.charged = true;
         t.x = t.y = t.z = t.R = t.eps = t.q = t.xl = t.yl = t.zl = 0.f;
         if (t.live) {
-            rel(__ldg(J.x + a), cx, t.x, t.xl);
-            rel(__ldg(J.y + a), cy, t.y, t.yl);
-            rel(__ldg(J.z + a), cz, t.z, t.zl);
+            tile_rel(__ldg(J.x + a), cx, t.x, t.xl);
+            tile_rel(__ldg(J.y + a), cy, t.y, t.yl);
+            tile_rel(__ldg(J.z + a), cz, t.z, t.zl);
             if (kMinImage) {
                 t.x = wrap_image(t.x, c.Lx, c.invLx);
                 t.y = wrap_image(t.y, c.Ly, c.invLy);
@@ -397,12 +406,84 @@ __device__ __forceinline__ void ff_tile(const TileJob& J, const FFConst& c, int 
     __syncthreads();  // the shared buffers may be reused
 }
 
-// Whether a grid is assembled by tiles.  Few atoms: the direct kernel's sums cost less than a tile's
-// classification and, where a tile has them, interpolation (160x160x60 nodes at 0.1 A, whole call: 16 atoms 29 us
-// directly, 23 by tiles; 24 atoms 38 and 29; 10 atoms 23 directly, where the call's own 20 us already show).  Coarse grids: beyond 0.35 A no atom nearer than
-// 26 A is far, and coordinates relative to the centre of a wide tile round worse than absolute ones.
-__host__ __device__ inline bool ff_use_tiles(int n, float dx, float dy, float dz) {
+// ---- which way a grid is assembled
+// One rounding per operation on the device and on the host, whose compiler may fuse: K1's launcher and the batch kernel
+// decide alike.
+__host__ __device__ inline float rule_mul(float a, float b) {
+#ifdef __CUDA_ARCH__
+    return __fmul_rn(a, b);
+#else
+    const volatile float r = a * b;
+    return r;
+#endif
+}
+__host__ __device__ inline float rule_add(float a, float b) {
+#ifdef __CUDA_ARCH__
+    return __fadd_rn(a, b);
+#else
+    const volatile float r = a + b;
+    return r;
+#endif
+}
+__host__ __device__ inline float rule_sqrt(float a) {
+#ifdef __CUDA_ARCH__
+    return __fsqrt_rn(a);
+#else
+    return sqrtf(a);
+#endif
+}
+
+// Estimate of the share of (node, atom) pairs at `reach` and more, for atoms spread over the cell Lx x Ly in a plane
+// 3 A below the grid (a molecule's depth and the grid's clearance): at height h those outside a disc of radius
+// sqrt(reach^2 - h^2), averaged over the grid's heights.
+__host__ __device__ inline float ff_far_share(float Lx, float Ly, float Lz, float reach) {
+    const float low = 3.f, high = rule_add(low, Lz), pi = 3.14159265f;
+    const float area = rule_mul(Lx, Ly), r2 = rule_mul(reach, reach);
+    const float in = rule_add(r2, -rule_mul(area, 1.f / pi));  // h^2 below which the disc covers the cell
+    const float h = in > 0.f ? rule_sqrt(in) : 0.f, h0 = h > low ? h : low, h1 = high < reach ? high : reach;
+    // heights out of reach of everything, times the area
+    float sum = rule_mul(area, high > reach ? rule_add(high, -(reach > low ? reach : low)) : 0.f);
+    if (h1 > h0) {
+        // integral of 1 - pi (reach^2 - h^2) / area from h0 to h1, times the area
+        const float lin = rule_mul(rule_add(area, -rule_mul(pi, r2)), rule_add(h1, -h0));
+        const float cub = rule_add(rule_mul(h1, rule_mul(h1, h1)), -rule_mul(h0, rule_mul(h0, h0)));
+        sum = rule_add(sum, rule_add(lin, rule_mul(pi / 3.f, cub)));
+    }
+    return sum / rule_mul(area, Lz);
+}
+
+// kDirect: direct sums.  Few atoms: they cost less than a tile's classification and, where a tile has them,
+// interpolation (160x160x60 nodes at 0.1 A, whole call: 16 atoms 29 us directly, 23 by tiles; 24 atoms 38 and 29;
+// 10 atoms 23 directly, where the call's own 20 us already show).  Coarse grids: beyond 0.35 A no atom nearer
+// than 26 A is far, and coordinates relative to the centre of a wide tile round worse than absolute ones.  And where a
+// tile would find little far, so that its classification, the float pairs of its coordinates and its coarser blocks
+// show: energies alone (whose direct sums are half as long) and fewer than 36 atoms, where the share of far pairs is
+// below 0.4.  Measured on either side of the line (K1 alone, us: direct sums / tiles):
+//   energies: 198 atoms on 61x111x53 nodes (0.2 A, share 0.04) 44 / 55; 86 on 177x56x79 (0.3 A, 0.33) 37 / 39; 493 on
+//   129x124x42 (0.1 A, 0.43) 193 / 94; 152 on 58x180x64 (0.1 A, 0.49) 78 / 49;
+//   32 atoms on 105x66x40 (0.1 A, 0.09) 20 / 23; 21 on 162x52x77 (0.2 A, 0.35) 18 / 21; 21 on 81x104x88 (0.15 A, 0.49)
+//   23 / 23; 30 on 64x208x98 (0.1 A, 0.71) 33 / 23; with more atoms 46 on 118x85x54 (0.1 A, 0.39) 29 / 25.
+// kCentred: direct sums with coordinates relative to the tile's centre, on periodic cells where that share is below 0.3 (energies 0.4)
+// (absolute coordinates / tiles / centred): 148 atoms on 71x215x73 (0.28 A, 0.00) 182 / 253 / 176; 184 on 106x340x85 (0.21 A,
+// 0.07) 430 / 513 / 415; 420 on 354x134x147 (0.29 A, 0.17) 2414 / 2578 / 2427; 380 on 124x386x153 (0.26 A, 0.31)
+// 1740 / 1632 / 1754; 172 on 146x193x53 (0.15 A, 0.37) 213 / 222 / 199; 228 on 281x111x196 (0.23 A, 0.44) 1090 / 897 / 1113.
+// Their coordinates round once, which keeps most of what the tiles gain in accuracy there (relative 2-norm of the error
+// against FP64, 124-atom sheet on 71x124x95: 7.7e-7 / 6.2e-7 / 6.8e-7; low parts in every pair, as the tiles have them, cost
+// 4 to 6 % of the time).  Molecules keep absolute coordinates: an atom's rounding is common to a tile's nodes, and about
+// a wide tile it exceeds theirs (99 atoms' energies at 0.25 A 7.9e-7 / 8.0e-7 / 9.3e-7).
+enum class FFPath { kDirect, kCentred, kTiles };
+__host__ __device__ inline bool ff_tiles_possible(int n, float dx, float dy, float dz) {
     return n >= 16 && dx <= 0.35f && dy <= 0.35f && dz <= 0.35f;
+}
+__host__ __device__ inline FFPath ff_path(int n, int nx, int ny, int nz, float dx, float dy, float dz, bool min_image,
+                                          bool energy) {
+    if (!ff_tiles_possible(n, dx, dy, dz)) return FFPath::kDirect;
+    if (!min_image && !energy && n >= 36) return FFPath::kTiles;
+    const float dmax = dx > dy ? (dx > dz ? dx : dz) : (dy > dz ? dy : dz);
+    const float reach = rule_mul(5.f * (kTileN - 1), dmax);  // 10 half extents
+    const float share = ff_far_share(rule_mul((float)nx, dx), rule_mul((float)ny, dy), rule_mul((float)nz, dz), reach);
+    if (share >= (min_image && !energy ? 0.3f : 0.4f)) return FFPath::kTiles;
+    return min_image ? FFPath::kCentred : FFPath::kDirect;
 }
 
 }  // namespace pp

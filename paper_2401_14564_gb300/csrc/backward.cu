@@ -45,6 +45,20 @@ __device__ __forceinline__ T warp_sum(T v) {
     return v;
 }
 
+// The sum of v over the warp as a float pair: FP64 adds run 2 lanes to a clock here.
+__device__ __forceinline__ float2 warp_sum_pair(float v) {
+    float hi = v, lo = 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float h = __shfl_xor_sync(0xffffffffu, hi, o), l = __shfl_xor_sync(0xffffffffu, lo, o);
+        float s, e;
+        two_sum(hi, h, s, e);
+        hi = s;
+        lo = __fadd_rn(__fadd_rn(lo, l), e);
+    }
+    return make_float2(hi, lo);
+}
+
 __global__ void init_kernel(const BwdLaunch P) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t == 0) {
@@ -218,8 +232,14 @@ __global__ void __launch_bounds__(kAdjThreads, kTri ? 1 : kAdjCtas) relax_adjoin
         }
     }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // (the tip sums cancel over the image: beyond a thread's own points they are summed in FP64)
-    double dkx = warp_sum((double)gkx), dky = warp_sum((double)gky), dkR = warp_sum((double)gkR);
+    // (the tip sums cancel over the image: beyond a thread's own points they are summed as float pairs, then in FP64)
+    const float2 skx = warp_sum_pair(gkx), sky = warp_sum_pair(gky), skR = warp_sum_pair(gkR);
+    double dkx = 0.0, dky = 0.0, dkR = 0.0;
+    if (lane == 0) {
+        dkx = (double)skx.x + (double)skx.y;
+        dky = (double)sky.x + (double)sky.y;
+        dkR = (double)skR.x + (double)skR.y;
+    }
     kmin = __reduce_min_sync(0xffffffffu, kmin);
     kmax = __reduce_max_sync(0xffffffffu, kmax);
     if (lane == 0) {
@@ -744,20 +764,6 @@ __global__ void __launch_bounds__(kTileThreads, 2) ff_backward_tile_kernel(const
         }
         flush();
     }
-}
-
-// The sum of v over the warp as a float pair: FP64 adds run 2 lanes to a clock here.
-__device__ __forceinline__ float2 warp_sum_pair(float v) {
-    float hi = v, lo = 0.f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float h = __shfl_xor_sync(0xffffffffu, hi, o), l = __shfl_xor_sync(0xffffffffu, lo, o);
-        float s, e;
-        two_sum(hi, h, s, e);
-        hi = s;
-        lo = __fadd_rn(__fadd_rn(lo, l), e);
-    }
-    return make_float2(hi, lo);
 }
 
 // Gradients from the tile kernel's replicas, a warp per atom.  dL/dq = k_e (Q C + (Qzz/2) Cq),

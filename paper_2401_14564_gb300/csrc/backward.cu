@@ -505,16 +505,18 @@ __global__ void __launch_bounds__(kFFBThreads) ff_backward_kernel(const BwdLaunc
 // worst relative error of a far pair 4e-7 at 10 half extents, for atoms that are the smaller part of
 // every gradient.  Atoms and node pairs share a CTA's 256 threads: atom slot tid mod 2^s, 2^s >= the list's
 // length, and the 256 / 2^s threads of a slot take the node pairs in turn, so a list of 5 near atoms and one
-// of 200 far ones both fill the warps.  A tile over a molecule has every atom near and one beside it none,
-// so a tile's near work is four CTAs' (four layers each) and its far work a fifth's.
+// of 200 far ones both fill the warps; a list a little longer than a power of two goes in parts (contract_all: 132 atoms
+// on a periodic 83x170x107 grid, whole adjoint, 144 -> 102 us; the 40-atom molecule below 103 -> 84).  A tile over
+// a molecule has every atom near and one beside it none, so a tile's near work is four CTAs' (four layers each; or
+// eight, see bwd_layers) and its far work one's.
 // The gradients cancel over the image, so their sums over the CTAs go to up to 32 replicas (in the adjoint
-// grid's unused fourth components) that finalize_tile_kernel adds in FP64: thousands of FP32 additions to one word
-// had cost 1-3e-6 relative in R and eps.
+// grid's unused fourth components) that finalize_tile_kernel adds as float pairs: thousands of FP32 additions to one
+// word had cost 1-3e-6 relative in R and eps.
 // Bound by the FP32 pipes like the direct contraction.  Measured (the whole adjoint): 60-atom flake,
-// 256x256x40 points, 417 -> 253 us; 40-atom molecule with the tip's quadrupole, 128x128x20 points, 146 -> 105 us (with
-// one CTA a tile 173: its busiest SM had 3.1 times the average's work); 300 atoms 906 -> 360 us.
+// 256x256x40 points, 400 -> 216 us; 40-atom molecule with the tip's quadrupole, 128x128x20 points, 138 -> 84 us (with
+// one CTA a tile it took twice as long: its busiest SM had 3.1 times the average's work); 300 atoms 906 -> 360 us.
 struct BwdTileShared {
-    float4 a[6 * 256];        // sums along z [component][z point][column]; then point pairs and node pairs
+    float4 a[6 * 256];        // sums along z [component][z point][column], then point pairs; or node pairs
     float b[192 * 17];        // sums along y [component][z point][y point][node along x], rows of 16 + 1 pad;
                               // then atom records, two float4 each
     int count[kTileThreads / 32];
@@ -522,12 +524,13 @@ struct BwdTileShared {
 };
 static_assert(sizeof(float) * 192 * 17 >= 2 * sizeof(float4) * kTileChunk, "atom records fit");
 
-constexpr int kBwdLayers = 4;                          // layers of a near part
-constexpr int kBwdParts = kTileN / kBwdLayers + 1;     // near parts, then the far part
-
-template <bool kMinImage, bool kCutoff, bool kQuad>
+// kBwdLayers: layers of a near part, 4, or 2 where nearly all of the work is near (bwd_layers).
+template <bool kMinImage, bool kCutoff, bool kQuad, int kBwdLayers>
 __global__ void __launch_bounds__(kTileThreads, 2) ff_backward_tile_kernel(const BwdLaunch P) {
     __shared__ BwdTileShared S;
+    constexpr int kBwdParts = kTileN / kBwdLayers + 1;           // near parts, then the far part
+    constexpr int kBwdPairs = kBwdLayers * kTileN * kTileN / 2;  // of a near part's nodes
+    static_assert(3 * kBwdPairs <= 6 * 256 && kBwdPairs % 256 == 0, "node pairs fit");
     const int klo = P.slab[0], khi = P.slab[1];
     const int i0 = blockIdx.x * kTileN, j0 = blockIdx.y * kTileN;
     const int k0 = (blockIdx.z / kBwdParts) * kTileN, part = blockIdx.z % kBwdParts;
@@ -579,8 +582,9 @@ __global__ void __launch_bounds__(kTileThreads, 2) ff_backward_tile_kernel(const
     const float hmax = fmaxf(hx, fmaxf(hy, hz));
     const FFConst fc = ff_const(P.R_pp, P.eps_pp, P.kQ, P.core_frac, P.Lx, P.Ly, kCutoff ? P.coul_rc : 0.f, 0.f);
     const BwdConst cst = bwd_const<kMinImage, kCutoff>(P);
-    float4* const pt = S.a;          // point pairs: xy, zg, gg (bwd_pair's A, B, G), 256 of each
-    float4* const nd = S.a + 768;    // node pairs, likewise
+    // point pairs (of a far part) and node pairs (of a near one): xy, zg, gg (bwd_pair's A, B, G), 256 and kBwdPairs of each
+    float4* const pt = S.a;
+    float4* const nd = S.a;
     float4* const rec = reinterpret_cast<float4*>(S.b);
 
     // the adjoints at the tile's points, as 256 pairs along x
@@ -632,10 +636,8 @@ __global__ void __launch_bounds__(kTileThreads, 2) ff_backward_tile_kernel(const
     const int first_sum = 7 * (int)((blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)) % P.replicas);
     BwdAtom at;
     int slots = 1, slot = 0, sub = 0, nsub = kTileThreads, ia = -1;
-    // takes the records first .. first + cnt - 1 as this CTA's atoms
+    // takes the records first .. first + cnt - 1 (at most `slots`) as this CTA's atoms
     auto take = [&](int first, int cnt) {
-        slots = 1;
-        while (slots < cnt) slots <<= 1;
         slot = tid & (slots - 1);
         sub = tid / slots;
         nsub = kTileThreads / slots;
@@ -658,6 +660,61 @@ __global__ void __launch_bounds__(kTileThreads, 2) ff_backward_tile_kernel(const
             atomicAdd(&P.gbar[checked((first_sum + q) * P.n + ia, P.map.stored_nodes, kChkGridWrite)].w, v[q]);
     };
 
+    // contracts the records first .. first + cnt - 1 with `pairs` pairs through contract(pair): whole rounds for every
+    // thread (the cutoff's warp votes), up to the next multiple of the threads a slot has.  A list that would leave a
+    // quarter of its slots or more idle goes in two or more, the larger power of two first.
+    auto contract_all = [&](int first, int cnt, int pairs, auto&& contract) {
+        while (cnt > 0) {
+            slots = 1;
+            while (slots < cnt) slots <<= 1;
+            int n = cnt;
+            if (slots >= 32 && 4 * cnt <= 3 * slots) n = slots = slots >> 1;
+            take(first, n);
+            const int rounds = (pairs + nsub - 1) / nsub;
+            for (int r = 0; r < rounds; ++r) contract(r * nsub + sub);
+            flush();
+            first += n;
+            cnt -= n;
+        }
+    };
+
+    int pairs = 256;  // the tile's points; of a near part, its layers' nodes with an adjoint
+    if (!far_part) {
+        float* const fxy = reinterpret_cast<float*>(nd);
+        float* const fzg = reinterpret_cast<float*>(nd + kBwdPairs);
+        float* const fgg = reinterpret_cast<float*>(nd + 2 * kBwdPairs);
+        if (tid == 0) S.nodes = 0;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kBwdLayers; ++k) {
+            const float gx = z[0][k], gy = z[1][k], gz = z[2][k];
+            const bool keep = gx != 0.f || gy != 0.f || gz != 0.f;
+            const unsigned mask = __ballot_sync(0xffffffffu, keep);
+            int first = 0;
+            if (lane == 0 && mask) first = atomicAdd(&S.nodes, __popc(mask));
+            first = __shfl_sync(0xffffffffu, first, 0);
+            if (keep) {
+                const int s = first + __popc(mask & ((1u << lane) - 1u)), w = (s >> 1) * 4, l = s & 1;
+                fxy[w + l] = __fmul_rn((float)ci - half, P.dx);
+                fxy[w + 2 + l] = __fmul_rn((float)cj - half, P.dy);
+                fzg[w + l] = __fmul_rn((float)(ka + k) - half, P.dz);
+                fzg[w + 2 + l] = gx;
+                fgg[w + l] = gy;
+                fgg[w + 2 + l] = gz;
+            }
+        }
+        __syncthreads();
+        const int cnt = S.nodes;  // (some: the part has an adjoint)
+        pairs = (cnt + 1) / 2;
+        // pad to a multiple of 256 pairs with the first node, adjoint zero
+        for (int s = cnt + tid; s < ((pairs + 255) & ~255) * 2; s += kTileThreads) {
+            const int w = (s >> 1) * 4, l = s & 1;
+            fxy[w + l] = fxy[0];
+            fxy[w + 2 + l] = fxy[2];
+            fzg[w + l] = fzg[0];
+            fzg[w + 2 + l] = fgg[w + l] = fgg[w + 2 + l] = 0.f;
+        }
+    }
     bool have_points = false;
     for (int base = 0; base < P.n; base += kTileChunk) {
         const int a = base + tid;
@@ -699,18 +756,13 @@ __global__ void __launch_bounds__(kTileThreads, 2) ff_backward_tile_kernel(const
             have_points = true;
             if (far) stage(s_far);
             __syncthreads();
-            if (n_in > 0) {
-                take(0, n_in);
-                for (int p = sub; p < 256; p += nsub)
-                    bwd_pair<false, kCutoff, kQuad, Smooth::kInside>(at, cst, pt[p], pt[256 + p], pt[512 + p], 0xffffffffu);
-                flush();
-            }
-            if (kCutoff && n_out > 0) {
-                take(n_in, n_out);
-                for (int p = sub; p < 256; p += nsub)
+            contract_all(0, n_in, pairs, [&](int p) {
+                bwd_pair<false, kCutoff, kQuad, Smooth::kInside>(at, cst, pt[p], pt[256 + p], pt[512 + p], 0xffffffffu);
+            });
+            if (kCutoff)
+                contract_all(n_in, n_out, pairs, [&](int p) {
                     bwd_pair<false, kCutoff, kQuad, Smooth::kBeyond>(at, cst, pt[p], pt[256 + p], pt[512 + p], 0xffffffffu);
-                flush();
-            }
+                });
             continue;
         }
         int n_near = 0;
@@ -718,51 +770,9 @@ __global__ void __launch_bounds__(kTileThreads, 2) ff_backward_tile_kernel(const
         if (n_near == 0) continue;
         if (live && !far) stage(s_near);
         __syncthreads();
-        take(0, n_near);
-        // the nodes with an adjoint, two layers (up to 512 nodes) at a time
-        float* const fxy = reinterpret_cast<float*>(nd);
-        float* const fzg = reinterpret_cast<float*>(nd + 256);
-        float* const fgg = reinterpret_cast<float*>(nd + 512);
-#pragma unroll
-        for (int kk = 0; kk < kBwdLayers; kk += 2) {
-            __syncthreads();
-            if (tid == 0) S.nodes = 0;
-            __syncthreads();
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const float gx = z[0][kk + u], gy = z[1][kk + u], gz = z[2][kk + u];
-                const bool keep = gx != 0.f || gy != 0.f || gz != 0.f;
-                const unsigned mask = __ballot_sync(0xffffffffu, keep);
-                int first = 0;
-                if (lane == 0 && mask) first = atomicAdd(&S.nodes, __popc(mask));
-                first = __shfl_sync(0xffffffffu, first, 0);
-                if (keep) {
-                    const int s = first + __popc(mask & ((1u << lane) - 1u)), w = (s >> 1) * 4, l = s & 1;
-                    fxy[w + l] = __fmul_rn((float)ci - half, P.dx);
-                    fxy[w + 2 + l] = __fmul_rn((float)cj - half, P.dy);
-                    fzg[w + l] = __fmul_rn((float)(ka + kk + u) - half, P.dz);
-                    fzg[w + 2 + l] = gx;
-                    fgg[w + l] = gy;
-                    fgg[w + 2 + l] = gz;
-                }
-            }
-            __syncthreads();
-            const int cnt = S.nodes;
-            if (cnt == 0) continue;
-            // whole rounds for every thread (the cutoff's warp votes): pad with the first node, adjoint zero
-            const int pairs = ((cnt + 1) / 2 + nsub - 1) / nsub * nsub;
-            for (int s = cnt + tid; s < 2 * pairs; s += kTileThreads) {
-                const int w = (s >> 1) * 4, l = s & 1;
-                fxy[w + l] = fxy[0];
-                fxy[w + 2 + l] = fxy[2];
-                fzg[w + l] = fzg[0];
-                fzg[w + 2 + l] = fgg[w + l] = fgg[w + 2 + l] = 0.f;
-            }
-            __syncthreads();
-            for (int p = sub; p < pairs; p += nsub)
-                bwd_pair<kMinImage, kCutoff, kQuad, Smooth::kNo>(at, cst, nd[p], nd[256 + p], nd[512 + p], 0xffffffffu);
-        }
-        flush();
+        contract_all(0, n_near, pairs, [&](int p) {
+            bwd_pair<kMinImage, kCutoff, kQuad, Smooth::kNo>(at, cst, nd[p], nd[kBwdPairs + p], nd[2 * kBwdPairs + p], 0xffffffffu);
+        });
     }
 }
 
@@ -1065,6 +1075,17 @@ __global__ void finalize_kernel(const BwdLaunch P) {
     }
 }
 
+// Layers of K5's near parts.  Halving them doubles the classification and the far part's share of CTAs, and evens out
+// the waves where near parts are all there is: periodic cells with less than 0.3 of the pairs far over the scan's heights
+// (ff_far_share), others with less than 0.05.  Whole adjoint, us, at 4 / 2 layers (direct sums): 192-atom sheet on 134x131
+// columns 189 / 116 (173), 560 on 117x146 345 / 210 (225), 820 on 147x280 (share 0.21) 548 / 384 (511), 51 atoms on 106x84 at
+// 0.15 A 71 / 52 (57); above the line 38 atoms on 120x103 at 0.1 A (0.26) 69 / 73, the flake (0.88) 217 / 241.
+int bwd_layers(const BwdLaunch& L) {
+    const float dmax = fmaxf(L.dx, fmaxf(L.dy, L.dz)), band = L.snz * L.sdz + 1.f, Lz = L.map.nz * L.dz;
+    const float share = ff_far_share(L.map.nx * L.dx, L.map.ny * L.dy, fminf(band, Lz), 5.f * (kTileN - 1) * dmax);
+    return share < (L.min_image ? 0.3f : 0.05f) ? 2 : 4;
+}
+
 template <int LAYOUT, int M>
 void launch_adjoint_m(const BwdLaunch& L, int blocks, cudaStream_t s) {
     if constexpr (LAYOUT == 0) {
@@ -1110,8 +1131,9 @@ cudaError_t launch_backward(const BwdLaunch& L0, cudaStream_t s) {
     const int64_t need = (total + kAdjThreads - 1) / kAdjThreads, most = (int64_t)kAdjCtas * sms;
     const int blocks = (int)(need < most ? (need > 0 ? need : 1) : most);
     const int64_t nodes = (int64_t)L.map.nx * L.map.ny * L.map.nz;
+    const int layers = bwd_layers(L);
     const dim3 tiles((L.map.nx + kTileN - 1) / kTileN, (L.map.ny + kTileN - 1) / kTileN,
-                     kBwdParts * ((L.map.nz + kTileN - 1) / kTileN));
+                     (kTileN / layers + 1) * ((L.map.nz + kTileN - 1) / kTileN));
     // by tiles where K1 can be, if the replicas fit the adjoint grid and the launch grid the tiles
     const bool by_tiles = !L.map.interp && ff_tiles_possible(L.n, L.dx, L.dy, L.dz) && tiles.y <= 65535 && tiles.z <= 65535 &&
                           7 * (int64_t)L.n <= L.map.stored_nodes;
@@ -1132,8 +1154,9 @@ cudaError_t launch_backward(const BwdLaunch& L0, cudaStream_t s) {
     launch_adjoint(L, blocks, s);
     if (by_tiles) {
         with_flags(L.min_image != 0, L.coul_rc > 0.f, L.Qzz != 0.f, [&](auto mi, auto cut, auto quad) {
-            ff_backward_tile_kernel<decltype(mi)::value, decltype(cut)::value, decltype(quad)::value>
-                <<<tiles, kTileThreads, 0, s>>>(L);
+            constexpr bool MI = decltype(mi)::value, CUT = decltype(cut)::value, QUAD = decltype(quad)::value;
+            if (layers == 2) ff_backward_tile_kernel<MI, CUT, QUAD, 2><<<tiles, kTileThreads, 0, s>>>(L);
+            else ff_backward_tile_kernel<MI, CUT, QUAD, 4><<<tiles, kTileThreads, 0, s>>>(L);
             return 0;
         });
         finalize_tile_kernel<<<(L.n + 7) / 8, 256, 0, s>>>(L);

@@ -39,7 +39,8 @@ class Simulator:
         0.025 on a force grid and 0 on a tricubic energy grid, whose scan is bound by issue slots rather
         than by its slowest tile (flake60 at 0.2 A: 1.42 ms on its own plan against 1.31 without).
         auto_plan: every scan builds the plan for the next from its own iteration counts.
-        plan_min_tiles: scans of fewer 8x4 pixel tiles get no plan (None: eight per SM)."""
+        plan_min_tiles: scans of fewer 8x4 pixel tiles get no plan (None: one per SM, and between one and eight
+        per SM auto_plan plans only where a plan pays, see _plan_next)."""
         self.case = case
         self.device = torch.device(device)
         if tuning is not None:
@@ -89,6 +90,9 @@ class Simulator:
         self._plan_k = 0       # k and lanes the held plan was built with
         self._plan_lanes = 0
         self._plan_ready = False
+        self._plan_pays = None   # whether plans pay for this simulator's scans; None: not known yet
+        self._plan_trial = None  # (pinned header, event) of the plan whose figures are on their way to the host
+        self._plan_calls = 0
         self.scan_lanes = 0    # pixels per warp of scans without a plan (0: the library's choice)
 
     def make_ff(self, atoms_dev, stream=None):
@@ -109,7 +113,7 @@ class Simulator:
         if not self.fused_df:
             pp.pp_fz_to_df(self.fz, self.scan.nz, self.scan.nx * self.scan.ny, self.scan.dz, self.dfp, out, stream)
         if self.auto_plan and self.iters is not None:
-            self.plan_from(self.iters, stream)
+            self._plan_next(stream)
 
     # ---- pixel-to-warp plan of the scan
     def plan_from(self, iters, stream=None):
@@ -118,14 +122,8 @@ class Simulator:
         costliest pixel columns run plan_lanes to a warp.  Outputs never depend on it."""
         if self.plan_frac <= 0:
             return
-        tiles = ((self.scan.nx + 7) // 8) * ((self.scan.ny + 3) // 4)
-        least = self.plan_min_tiles
-        if least is None:
-            least = 8 * torch.cuda.get_device_properties(self.device).multi_processor_count
-        if tiles < least:
-            # smaller scans run narrow warps throughout or leave issue slots free; building the plan then
-            # costs more than it saves (181x181 px, 1058 tiles: 0.236 ms with its own plan and its build
-            # against 0.215 without; 128x128: 0.201 against 0.199; 256x256, 2048 tiles: 0.549 against 0.609)
+        tiles, sms = self._scan_tiles()
+        if tiles < (sms if self.plan_min_tiles is None else self.plan_min_tiles):
             return
         npix = self.scan.nx * self.scan.ny
         k = max(1, min(npix, int(round(self.plan_frac * npix))))
@@ -138,8 +136,60 @@ class Simulator:
         self._plan_ready = True
 
     def drop_plan(self):
-        """Scans go back to 8x4 pixel tiles alone (until the next plan_from)."""
+        """Scans go back to pixel tiles alone (until the next plan_from)."""
         self._plan_ready = False
+
+    def _scan_tiles(self):
+        """8x4 pixel tiles of the scan, and the GPU's SMs."""
+        return (((self.scan.nx + 7) // 8) * ((self.scan.ny + 3) // 4),
+                torch.cuda.get_device_properties(self.device).multi_processor_count)
+
+    _PLAN_EVERY = 32  # calls between two looks at whether plans pay
+
+    @staticmethod
+    def plan_pays(gain, tiles):
+        """Whether a plan pays whose costliest column takes `gain` more FIRE updates than the costliest that stays in
+        its tile, for a scan of `tiles` pixel tiles between one and eight per SM.  Building it takes 14-17 us
+        each scan and its narrow warps issue slots that the tiles want, the more of them the more tiles there are; an update
+        of a column alone takes 0.24 us.  Measured without / with a plan, build included (us): 528 tiles, 28 heights,
+        gain 136 299 / 282, gain 279 404 / 336, gain 67 238 / 242; 666 tiles, gain 127 369 / 346; 820 tiles, gain 149
+        227 / 221, gain 141 295 / 301, gain 86 205 / 224, gain 274 402 / 331; 1058 tiles, gain 135 367 / 378, gain 262 362 / 329."""
+        return gain >= 100 + tiles / 26
+
+    def _plan_next(self, stream=None):
+        """After a scan, with auto_plan: the plan for the next one.  Scans of eight tiles per SM and more (or with
+        plan_min_tiles given) plan always.  Of smaller ones the second, and then every 32nd, builds a plan whose figures
+        come to the host while later scans run; once they are here, and until the next look, every scan plans or
+        none does.  (Nothing waits for them; under capture the last answer stands.)"""
+        tiles, sms = self._scan_tiles()
+        if self.plan_min_tiles is not None or tiles >= 8 * sms:
+            self.plan_from(self.iters, stream)
+            return
+        if self.plan_frac <= 0 or tiles < sms:
+            return
+        st = stream or torch.cuda.current_stream(self.device)
+        with torch.cuda.stream(st):
+            if torch.cuda.is_current_stream_capturing():
+                if self._plan_pays:
+                    self.plan_from(self.iters, st)
+                return
+            if self._plan_trial is not None and self._plan_trial[1].query():
+                most, rest = (int(v) for v in self._plan_trial[0][5:7])
+                self._plan_pays, self._plan_trial = self.plan_pays(most - rest, tiles), None
+                if not self._plan_pays:
+                    self.drop_plan()
+            self._plan_calls += 1
+            look = self._plan_trial is None and (self._plan_calls - 2) % self._PLAN_EVERY == 0
+            if look or self._plan_pays:
+                ready = self._plan_ready
+                self.plan_from(self.iters, st)
+                self._plan_ready = ready or bool(self._plan_pays)
+            if look:
+                header = torch.empty(8, dtype=torch.int32, pin_memory=True)
+                header.copy_(self._plan[:8], non_blocking=True)
+                event = torch.cuda.Event()
+                event.record(st)
+                self._plan_trial = (header, event)
 
     def run(self, atoms_dev, stream=None, df=None):
         """Device-resident forward pass; returns the df tensor (device)."""

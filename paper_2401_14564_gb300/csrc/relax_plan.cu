@@ -12,7 +12,8 @@
 //
 // Layout of the plan buffer (int32 words, sizes from pp_relax_plan_size):
 //   [0, 8)             header: [1] lowest bin taken, [2] columns above that bin,
-//                      [3] / [4] selection counters
+//                      [3] / [4] selection counters, [5] the costliest column's cost,
+//                      [6] that of the costliest column not listed
 //   hist   [kBins]     columns per cost bin (cost >> shift)
 //   cost   [npix]      sum over heights of the earlier scan's iters
 //   list   [hb*lanes]  the selected pixels, -1 in unused slots (hb = ceil(k/lanes))
@@ -27,9 +28,20 @@ namespace {
 constexpr int kBins = 2048;
 constexpr int kHdr = 8;
 
+// The block's largest v (>= 0), folded into *out.
+__device__ __forceinline__ void block_max(int v, int* out) {
+    __shared__ int most;
+    if (threadIdx.x == 0) most = 0;
+    __syncthreads();
+    v = __reduce_max_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0 && v > 0) atomicMax(&most, v);
+    __syncthreads();
+    if (threadIdx.x == 0 && most > 0) atomicMax(out, most);
+}
+
 // Also clears the list (-1) and the mask for plan_select_kernel, which runs after it.
 __global__ void __launch_bounds__(256) plan_cost_kernel(const int* __restrict__ iters, int nz, int npix, int shift,
-                                                        int* hist, int* cost, int* list, int nlist, unsigned* mask,
+                                                        int* hdr, int* hist, int* cost, int* list, int nlist, unsigned* mask,
                                                         int nmask) {
     __shared__ int sh[kBins];
     for (int b = threadIdx.x; b < kBins; b += blockDim.x) sh[b] = 0;
@@ -37,13 +49,16 @@ __global__ void __launch_bounds__(256) plan_cost_kernel(const int* __restrict__ 
     for (int q = gt; q < nlist; q += gs) list[q] = -1;
     for (int q = gt; q < nmask; q += gs) mask[q] = 0u;
     __syncthreads();
+    int most = 0;
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < npix; p += gridDim.x * blockDim.x) {
         long long c = 0;
         for (int k = 0; k < nz; ++k) c += max(__ldg(iters + (size_t)k * npix + p), 0);
         const int ci = (int)min(c, (long long)0x7fffffff);
         cost[p] = ci;
+        most = max(most, ci);
         atomicAdd(&sh[min(ci >> shift, kBins - 1)], 1);
     }
+    block_max(most, hdr + 5);
     __syncthreads();
     for (int b = threadIdx.x; b < kBins; b += blockDim.x)
         if (sh[b]) atomicAdd(hist + b, sh[b]);
@@ -95,16 +110,20 @@ __global__ void __launch_bounds__(1024) plan_threshold_kernel(int* hdr, const in
 __global__ void __launch_bounds__(256) plan_select_kernel(int* hdr, const int* __restrict__ cost, int npix, int shift,
                                                           int k, int* list, unsigned* mask) {
     const int t = hdr[1], above = hdr[2];
+    int most = 0;  // of the columns not listed
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < npix; p += gridDim.x * blockDim.x) {
-        const int bin = min(cost[p] >> shift, kBins - 1);
+        const int c = cost[p], bin = min(c >> shift, kBins - 1);
         int slot = k;
         if (bin > t) slot = atomicAdd(hdr + 3, 1);              // < above <= k - 1 by construction
         else if (bin == t) slot = above + atomicAdd(hdr + 4, 1);
         if (slot < k) {
             list[slot] = p;
             atomicOr(mask + (p >> 5), 1u << (p & 31));
+        } else {
+            most = max(most, c);
         }
     }
+    block_max(most, hdr + 6);
 }
 
 }  // namespace
@@ -133,7 +152,7 @@ cudaError_t launch_relax_plan(const int* iters, int nz, int npix, int max_iter, 
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int blocks = (int)std::min<long long>(((long long)npix + 255) / 256, 2LL * sms);
-    plan_cost_kernel<<<blocks, 256, 0, s>>>(iters, nz, npix, shift, hist, cost, list, (int)(hb * lanes), mask,
+    plan_cost_kernel<<<blocks, 256, 0, s>>>(iters, nz, npix, shift, hdr, hist, cost, list, (int)(hb * lanes), mask,
                                             (npix + 31) / 32);
     plan_threshold_kernel<<<1, 1024, 0, s>>>(hdr, hist, k);
     plan_select_kernel<<<blocks, 256, 0, s>>>(hdr, cost, npix, shift, k, list, mask);

@@ -355,7 +355,8 @@ typedef struct {
     long long out_capacity; /* entries in fz and iters (pos holds 3x)                         */
     long long df_capacity;  /* entries in df                                                  */
     int n_atoms_total;      /* length of the packed atom arrays                               */
-    int ctas;               /* persistent CTAs of 128 threads of the relax kernel; 0 = fill the GPU */
+    int ctas;               /* persistent CTAs of the relax kernel (128 threads) and at most of the
+                               force-field kernel (256 threads, two per SM); 0 = fill the GPU  */
     long long spin_limit;   /* polls (~128 ns apart) before a relax item stops waiting for its
                                molecule's force field; 0 = 1<<23 (about one second)           */
     int wait_extra;         /* test hook, 0 in normal use: relax items wait for this many more

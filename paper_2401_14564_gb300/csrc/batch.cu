@@ -379,10 +379,12 @@ cudaError_t launch_batch(const BatchArgs& A, cudaStream_t s) {
     int dev = 0, sms = 152, per_sm = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // (a caller's limit keeps the same SMs free of both kernels)
+    const int ff_ctas = P.ctas > 0 && P.ctas < 2 * sms ? P.ctas : 2 * sms;
     with_flags(B.min_image != 0, B.coul_rc > 0.f, B.kQzz != 0.f, [&](auto mi, auto cut, auto quad) {
         constexpr bool MI = decltype(mi)::value, CUT = decltype(cut)::value, QUAD = decltype(quad)::value;
-        if (B.forces_only) batch_ff_kernel<MI, CUT, QUAD, true><<<2 * sms, kTileThreads, 0, s>>>(B);
-        else batch_ff_kernel<MI, CUT, QUAD, false><<<2 * sms, kTileThreads, 0, s>>>(B);
+        if (B.forces_only) batch_ff_kernel<MI, CUT, QUAD, true><<<ff_ctas, kTileThreads, 0, s>>>(B);
+        else batch_ff_kernel<MI, CUT, QUAD, false><<<ff_ctas, kTileThreads, 0, s>>>(B);
         return 0;
     });
     cudaError_t e = cudaGetLastError();

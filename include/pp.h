@@ -357,10 +357,10 @@ typedef struct {
     int n_atoms_total;      /* length of the packed atom arrays                               */
     int ctas;               /* persistent CTAs of the relax kernel (128 threads) and at most of the
                                force-field kernel (256 threads, two per SM); 0 = fill the GPU  */
-    long long spin_limit;   /* polls (~128 ns apart) before a relax item stops waiting for its
-                               molecule's force field; 0 = 1<<23 (about one second)           */
-    int wait_extra;         /* test hook, 0 in normal use: relax items wait for this many more
-                               force-field tiles than exist, so every wait runs out            */
+    long long spin_limit;   /* >= 0; accepted and without effect (nothing waits: stream order puts
+                               the force fields before the scans)                              */
+    int wait_extra;         /* test hook, 0 in normal use: relax items ask for this many more
+                               force-field tiles than exist, so every check fails              */
     int ff_forces_only;     /* 1: every grid's E slots written as 0 and the energy sums skipped
                                (the forces, and so all scan outputs, are unchanged); 0 or 1    */
     /* Work-item shapes (picked by the autotuner; every choice computes the same values bit for
@@ -374,7 +374,7 @@ typedef struct {
 
 /* Status bits reported by pp_batch_status. */
 #define PP_BATCH_BAD_DESC 1 /* a descriptor was invalid or overran a buffer: that molecule was skipped */
-#define PP_BATCH_TIMEOUT 2  /* a bounded wait ran out: some relax tiles were not computed            */
+#define PP_BATCH_TIMEOUT 2  /* a force field was not complete: some relax tiles were not computed    */
 
 /* Scratch bytes of pp_batch_run for nmol molecules (0 if nmol < 1). */
 PP_API size_t pp_batch_workspace(int nmol);
@@ -383,10 +383,10 @@ PP_API size_t pp_batch_workspace(int nmol);
  * descriptor (bad ones are skipped and flagged) and lays out the work items, a
  * persistent kernel assembles the force fields by tiles of 16x16x16 nodes, and
  * another runs the relax tiles (relax_tile_w x 32/relax_tile_w pixels, all
- * heights); workers pull items from a device counter.  A relax tile waits
- * (bounded, see spin_limit) until every force-field tile of its molecule is
- * done.  Writes, per molecule, the force field, fz, df and (nullable) pos and
- * iters exactly as
+ * heights); workers pull items from a device counter.  A relax tile checks
+ * that every force-field tile of its molecule is done (stream order sees to
+ * it) and sets PP_BATCH_TIMEOUT if not.  Writes, per molecule, the force
+ * field, fz, df and (nullable) pos and iters exactly as
  * pp_make_ff + pp_relax_scan (fused df) on that molecule alone (the grid's E
  * slots 0 when params->ff_forces_only).  descs is a
  * DEVICE array of nmol descriptors; atoms are packed device arrays; ws is
@@ -401,7 +401,7 @@ PP_API pp_status pp_batch_run(const pp_mol_desc* descs, int nmol, const pp_batch
 
 /* Device-side status of the last pp_batch_run on `ws`: waits for `stream`,
  * then stores the PP_BATCH_* bits in *flags (host int).  Returns
- * PP_ERR_TIMEOUT if a wait ran out, PP_ERR_CAPACITY if a descriptor was bad,
+ * PP_ERR_TIMEOUT if a check failed, PP_ERR_CAPACITY if a descriptor was bad,
  * else PP_OK.  This call synchronises the host with the stream. */
 PP_API pp_status pp_batch_status(const void* ws, int* flags, pp_stream stream);
 

@@ -672,7 +672,7 @@ pp_status pp_batch_status(const void* ws, int* flags, pp_stream stream) {
     r = cuda_status(cudaStreamSynchronize(s), "pp_batch_status sync");
     if (r != PP_OK) return r;
     *flags = st;
-    if (st & PP_BATCH_TIMEOUT) { set_error("pp_batch_run: a bounded wait ran out"); return PP_ERR_TIMEOUT; }
+    if (st & PP_BATCH_TIMEOUT) { set_error("pp_batch_run: a force field was not complete before its scan"); return PP_ERR_TIMEOUT; }
     if (st & PP_BATCH_BAD_DESC) { set_error("pp_batch_run: invalid descriptor(s) skipped"); return PP_ERR_CAPACITY; }
     return PP_OK;
 }

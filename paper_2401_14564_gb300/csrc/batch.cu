@@ -9,8 +9,8 @@
 // 128x128 scan is only 512 warps.  The force fields are assembled by one kernel and scanned by the next:
 // with the far atoms interpolated (ff_tile.cuh) assembly is a CTA's work, and what it takes is no longer
 // enough to hide scans behind; a grid written to HBM and read back in its scan's layers costs 1 % of a
-// batch's time.  A relax tile still checks its molecule's completion counter (a bounded wait; a timeout
-// sets a status bit and the warp stops).
+// batch's time.  A relax tile checks its molecule's count of finished force-field tiles (one that is short sets a status
+// bit and the warp stops).
 #include <cstring>
 
 #include "ff_tile.cuh"
@@ -48,7 +48,6 @@ struct BatchLaunch {
     long long* seg_start;  // [2 nmol + 1]: first item of FF(m) at m, of R(m) at nmol + m, their end
     int* done_ff;          // [nmol]
     float* coef_ws;
-    long long spin_limit;
     int wait_extra;
     int forces_only;  // E slots written as 0, energy sums skipped
     int rw_sh;        // log2 of the relax tile width (4, 8 or 16 lanes along x)
@@ -145,16 +144,6 @@ __global__ void __launch_bounds__(1024) batch_plan_kernel(const BatchLaunch B) {
         __syncthreads();
     }
     if (tid == 0) B.seg_start[nseg] = carry;
-}
-
-__device__ __forceinline__ int load_acquire(const int* p) {
-    int v;
-    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ void add_release(int* p, int v) {
-    asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 // Segment holding item t among seg_start[first .. last): the last s with seg_start[s] <= t.
@@ -260,9 +249,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) batch_ff_kernel(const BatchLa
                     ff_direct<kMinImage, kCutoff, kQuad>(B, D, cst, i0 + (warp & 1) * 8, j0 + (warp >> 1) * 4, k0 + 8 * h,
                                                          path == FFPath::kCentred, i0, j0, k0, S.buf + warp * 128, store);
         }
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) add_release(B.done_ff + mol, 1);
+        if (threadIdx.x == 0) atomicAdd(B.done_ff + mol, 1);
     }
 }
 
@@ -277,25 +264,11 @@ __global__ void __launch_bounds__(kThreads, kMinCtas) batch_relax_kernel(const B
         const int seg = find_segment(B, B.nmol, 2 * B.nmol, first + t), mol = seg - B.nmol;
         const long long tile = first + t - B.seg_start[seg];
         const pp_mol_desc D = B.descs[mol];
-        // wait (bounded) for every force-field tile of this molecule
-        const int need = (int)(B.seg_start[mol + 1] - B.seg_start[mol]) + B.wait_extra;
-        int ok = 1;
-        if (lane == 0) {
-            long long polls = 0;
-            while (load_acquire(B.done_ff + mol) < need) {
-                if (++polls > B.spin_limit) {
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(128);
-            }
-        }
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        if (!ok) {
+        // every force-field tile of this molecule is done, by stream order: a check, not a wait
+        if (B.done_ff[mol] < (int)(B.seg_start[mol + 1] - B.seg_start[mol]) + B.wait_extra) {
             if (lane == 0) atomicOr(B.status, PP_BATCH_TIMEOUT);
             break;
         }
-        __syncwarp();
         MolRelax G;
         G.ff = B.ff + D.ff_offset;
         G.map.nx = D.nx; G.map.ny = D.ny; G.map.nz = D.nz;
@@ -369,7 +342,6 @@ cudaError_t launch_batch(const BatchArgs& A, cudaStream_t s) {
     B.coef = B.coef_ws;
     B.seg_start = reinterpret_cast<long long*>(w + 320);
     B.done_ff = reinterpret_cast<int*>(w + 320 + 8 * (2 * (size_t)A.nmol + 1));
-    B.spin_limit = P.spin_limit > 0 ? P.spin_limit : (1LL << 23);
     B.wait_extra = P.wait_extra;
     B.forces_only = P.ff_forces_only;
     const int rw = P.relax_tile_w > 0 ? P.relax_tile_w : 8;

@@ -2,14 +2,13 @@
 
 Choices it sweeps, each timed with CUDA events through the C ABI on the
 workload itself (inputs on the device, median of a few repetitions):
-  - pp_make_ff_tuned: z-nodes per thread (4, 8, 16);
+  - pp_make_ff_tuned: z-nodes per thread (4, 8, 16), where the grid is summed directly;
   - pp_relax_scan: force-field layout, linear or bricked (several brick shapes),
     timed on the scan alone, or on whole steps several in flight (afm.Pipeline)
     when the caller runs them that way: the two regimes can prefer different
     layouts (a lone scan is bound by its slowest columns' dependency chains,
     overlapped steps by issue slots and cache capacity);
-  - pp_batch_run: the work-item shapes (force-field tile depth and width, relax tile width) and
-    the persistent CTA count.
+  - pp_batch_run: the relax tiles' width and the persistent CTA count.
 Every candidate computes the same values (the layout and the launch shape do
 not change the arithmetic per node or per pixel), so the pick is a pure
 speed decision.  Results are cached in a JSON file keyed by GPU name and
@@ -49,8 +48,17 @@ def _time(fn, reps):
     return statistics.median(ts)
 
 
+def _zpt_matters(case):
+    """Whether ff_zpt can change how the case's grid is assembled: not for energies, nor where K1 runs by tiles or about
+    their centres (36 atoms, 16 on periodic cells, spacings up to 0.35 A)."""
+    g = case["grid"]
+    n, fine = len(case["atoms"]["x"]), max(g["dx"], g["dy"], g["dz"]) <= 0.35
+    return not g.get("interp", 0) and not (fine and n >= (16 if case["probe"]["min_image"] else 36))
+
+
 def tune_case(case, reps=3, bricks=BRICKS, zpts=ZPTS, ff_energy=True, pipeline_slots=0):
-    """Time every FF launch shape and every grid layout for the relaxation; return the fastest.
+    """Time every FF launch shape that differs (one where ff_zpt has no effect) and every grid layout for the
+    relaxation; return the fastest.
     ff_energy=False times the forces-only assembly (the one a Simulator with ff_energy=False runs).
     pipeline_slots > 0 times each layout on 4 x pipeline_slots whole steps through an
     afm.Pipeline of that many slots (the regime of Pipeline.run_many) instead of the scan alone."""
@@ -60,6 +68,8 @@ def tune_case(case, reps=3, bricks=BRICKS, zpts=ZPTS, ff_energy=True, pipeline_s
     ff_times = {}
     grid0 = pp.make_grid(case["grid"], 0)
     ff = torch.empty(pp.pp_ff_floats(grid0), dtype=torch.float32, device="cuda")
+    if not _zpt_matters(case):
+        zpts = (8,) if 8 in zpts else zpts[:1]
     for z in zpts:
         t = pp.Tuning(z, 0 if ff_energy or case["grid"].get("interp", 0) else 1)
         pp.pp_make_ff_tuned(atoms, probe, grid0, ff, t)
@@ -93,13 +103,13 @@ def tune_case(case, reps=3, bricks=BRICKS, zpts=ZPTS, ff_energy=True, pipeline_s
             else "ms per scan alone"}
 
 
-BATCH_SHAPES = (("ff_zpt", (8, 4)), ("ff_tile_w", (8, 4, 16)), ("relax_tile_w", (8, 4, 16)))
+BATCH_SHAPES = (("relax_tile_w", (8, 4, 16)),)
 
 
 def tune_batch(batch_obj, reps=2, factors=(1, 2, 3, 4, 5, 6)):
-    """Pick the batch's work-item shapes (force-field tile depth and width, relax tile width) and
-    its persistent CTA count (0 = as many as fit, else multiples of the SM count) by coordinate
-    descent from the defaults: each choice in turn is swept with the others held at their best so
+    """Pick the batch's relax tile width and its persistent CTA count (0 = as many as fit, else
+    multiples of the SM count; ff_zpt and ff_tile_w have no effect and stay 8) by coordinate descent from
+    the defaults: each choice in turn is swept with the others held at their best so
     far, timing pp_batch_run itself (CUDA events, median of reps).  Every choice computes the
     same molecules bit for bit.  Leaves the pick in batch_obj.params and returns it with the
     timings."""
@@ -127,8 +137,7 @@ def tune_batch(batch_obj, reps=2, factors=(1, 2, 3, 4, 5, 6)):
     for k, v in best.items():
         setattr(p, k, v)
     return {"choice": best, "ms": best_t, "ms_default_shapes": t_default, "tried_ms": tried,
-            "how": "coordinate descent over ff_zpt, ff_tile_w, relax_tile_w, then ctas; median of %d timed runs "
-                   "each" % reps}
+            "how": "coordinate descent over relax_tile_w, then ctas; median of %d timed runs each" % reps}
 
 
 def cached(case, path=None, **kw):

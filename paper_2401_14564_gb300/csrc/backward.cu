@@ -501,9 +501,9 @@ __global__ void __launch_bounds__(kFFBThreads) ff_backward_kernel(const BwdLaunc
 // K5 by tiles (the grids K1 assembles by tiles): the transpose of ff_tile.cuh's interpolation.  The node
 // adjoints of a 16x16x16-node tile are carried to its 8x8x8 Chebyshev points (along z, y, x), where the far
 // atoms' pair derivatives are contracted with 512 points instead of up to 4096 nodes; near atoms are
-// contracted with the nodes that hold an adjoint.  The derivatives are one order steeper than the terms:
-// worst relative error of a far pair 4e-7 at 10 half extents, for atoms that are the smaller part of
-// every gradient.  Atoms and node pairs share a CTA's 256 threads: atom slot tid mod 2^s, 2^s >= the list's
+// contracted with the nodes that hold an adjoint.  The derivatives are one order steeper than the terms: at 10 half
+// extents a far Lennard-Jones pair's is good to 7e-7 of the largest in the tile (1.7e-6 of the node's own), for atoms
+// that are the smaller part of every gradient.  Atoms and node pairs share a CTA's 256 threads: atom slot tid mod 2^s, 2^s >= the list's
 // length, and the 256 / 2^s threads of a slot take the node pairs in turn, so a list of 5 near atoms and one
 // of 200 far ones both fill the warps; a list a little longer than a power of two goes in parts (contract_all: 132 atoms
 // on a periodic 83x170x107 grid, whole adjoint, 144 -> 102 us; the 40-atom molecule below 103 -> 84).  A tile over

@@ -10,18 +10,19 @@
 //         interpolated to the nodes along x, y and z (barycentric Lagrange interpolation on the target
 //         side; published as the cluster-particle treecode, Boateng & Krasny 2013);
 //   near  everything else: summed at the nodes as before.
-// Interpolation error, worst node relative to the pair's own force, measured in FP64 at D = 10 h: 1.5e-7
-// for the r^-7 term, 1.5e-9 Coulomb; the r^-13 term's 4e-6 counts with its weight (R/D)^6 <= 0.035
-// against the r^-7 term, hence the bound on D / R.  The direct sum's own rounding (rsqrt to 2 ulp,
-// raised to the 8th) is 5e-7 per pair.  Coordinates are taken relative to the tile's centre (formed as a
+// Interpolation error, measured in FP64 at D = 10 h over directions: relative to the largest force in the tile 1.5e-9
+// (Coulomb), 1.5e-7 (the r^-7 term) and 3.9e-6 (r^-13); relative to the node's own 1.5e-9, 4.7e-7 and 3.5e-5.  The
+// last counts with its weight against the r^-7 term, (R/r)^6 <= 0.035 at the centre and 0.11 at the nearest node, hence
+// the bound on D / R: a whole Lennard-Jones pair is good to 4.7e-7 of the node's own force at any R up to it.  The
+// direct sum's own rounding (rsqrt to 2 ulp, raised to the 8th) is 5e-7 per pair, about as much.  Coordinates are taken relative to the tile's centre (formed as a
 // float pair, the atoms' kept as float pairs), which removes the rounding of absolute node coordinates that the
 // direct kernel has; without the low parts the far sums would share an atom's rounding over a whole tile
 // (flake 8.45e-7 against 8.0e-7 below).
 //
 // Measured (direct sums -> tiles, Simulator.make_ff): 60-atom flake on 256x256x200 nodes, forces only, 0.408
 // -> 0.136 ms (the grid's 210 MB alone take 31 us); 40-atom molecule on 176x160x60 with the tip's quadrupole
-// 76 -> 45 us; 97 atoms, energies only at 0.15 A, 160 -> 61 us; the 2516-atom slab on 512x512x250 109 ->
-// 23.2 ms.  FP32 pipes set the pace as before.  Error against FP64, mean over layers of the relative
+// 76 -> 45 us; 97 atoms, energies only at 0.15 A, 160 -> 60 us; the 2516-atom slab on 512x512x250 109 ->
+// 22.5 ms.  FP32 pipes set the pace as before.  Error against FP64, mean over layers of the relative
 // 2-norm: 8.1e-7 -> 8.0e-7 (flake), 3.0e-7 -> 2.9e-7 (molecule), 7.3e-7 -> 4.2e-7 (800-atom periodic sheet).
 //
 // Why 16 nodes and 8 points: 8 points keep the far sum at 1/8 of the direct one (64 columns of 8 points

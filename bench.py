@@ -40,41 +40,29 @@ SM_COUNT_NOMINAL = 152       # GB300; the bench reads the count from the device 
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from single-launch ncu
 # captures summarised in profiles/, valid only for the kernel sources they were taken on: the
 # bench reports them when the sources still hash the same, else traffic is null.
+_SCAN = ["relax_scan.cu", "relax_core.cuh", "interp.cuh"]
+_DIRECT = ["ff_assemble.cu", "ff_core.cuh", "interp.cuh"]
+_TILES = ["ff_tile.cu", "ff_tile.cuh", "ff_core.cuh", "interp.cuh"]
 TRAFFIC = {
-    "relax_scan": {"bytes": 66.21e6, "sha": "65e56d7ba4e85d47",
-                   "files": ["relax_scan.cu", "relax_core.cuh", "interp.cuh"]},
-    "relax_scan_tricubic": {"bytes": 24.60e6, "sha": "65e56d7ba4e85d47",
-                            "files": ["relax_scan.cu", "relax_core.cuh", "interp.cuh"]},
-    "ff_assemble": {"bytes": 148.45e6, "bytes_zpt16": 139.83e6, "sha": "82384c014f2b4572",
-                    "files": ["ff_assemble.cu", "ff_core.cuh", "interp.cuh"]},
-    "ff_assemble_quad": {"bytes": 148.68e6, "sha": "82384c014f2b4572",
-                         "files": ["ff_assemble.cu", "ff_core.cuh", "interp.cuh"]},
-    "ff_assemble_split": {"bytes": 357.10e6, "sha": "82384c014f2b4572",
-                          "files": ["ff_assemble.cu", "ff_core.cuh", "interp.cuh"]},
-    "ff_combine": {"bytes": 600.65e6, "sha": "82384c014f2b4572",
-                   "files": ["ff_assemble.cu", "ff_core.cuh", "interp.cuh"]},
+    "relax_scan": {"bytes": 62.63e6, "sha": "ba93cc0bc5a90b25", "files": _SCAN},
+    "relax_scan_tricubic": {"bytes": 19.52e6, "sha": "ba93cc0bc5a90b25", "files": _SCAN},
+    "ff_tile": {"bytes": 146.83e6, "sha": "7ee6a45a261d0c8e", "files": _TILES},
+    "ff_tile_quad": {"bytes": 145.24e6, "sha": "7ee6a45a261d0c8e", "files": _TILES},
+    "ff_assemble_split": {"bytes": 354.83e6, "sha": "8d62392aedade281", "files": _DIRECT},
+    "ff_combine": {"bytes": 584.55e6, "sha": "8d62392aedade281", "files": _DIRECT},
 }
 
 
-def measured_traffic(kernel, zpt=8):
+def measured_traffic(kernel):
     t = TRAFFIC[kernel]
-    if _src_hash(t["files"]) != t["sha"]:
-        return None
-    return t.get("bytes_zpt16") if int(zpt) == 16 and kernel == "ff_assemble" else t["bytes"]
+    return t["bytes"] if _src_hash(t["files"]) == t["sha"] else None
+
+
 FP32_LANES_PER_SM = 128
 
-# Figures from single-kernel ncu captures summarised in profiles/, valid for the sources they were
-# taken on (same hash rule as TRAFFIC): the FP32 operations K1 executes per node-atom pair
-# (sm__sass_thread_inst_executed_op_{fadd,fmul,ffma}_pred_on, FFMA counted twice, over the pairs of
-# the launch) and the issue-active fraction of K2 (smsp__issue_active.avg.pct_of_peak_sustained_active).
-EXECUTED = {  # per z-nodes-per-thread launch shape (16: a bulk launch of 12 x 16 layers and a tail of 8)
-    # (captures of the direct kernel; the tiles' operations per pair depend on how many atoms are far)
-    "ff_forces": {"value": None, "sha": None, "files": ["ff_tile.cu", "ff_tile.cuh", "ff_core.cuh", "interp.cuh"]},
-    "ff_energy": {"value": None, "sha": None, "files": ["ff_tile.cu", "ff_tile.cuh", "ff_core.cuh", "interp.cuh"]},
-}
-ISSUE = {
-    "relax_scan": {"value": 0.573, "sha": "65e56d7ba4e85d47", "files": ["relax_scan.cu", "relax_core.cuh", "interp.cuh"]},
-}
+# The issue-active fraction of K2 (smsp__issue_active.avg.pct_of_peak_sustained_active), from the captures summarised in
+# profiles/, valid for the sources they were taken on (same hash rule as TRAFFIC).
+ISSUE = {"relax_scan": {"value": 0.574, "sha": "ba93cc0bc5a90b25", "files": _SCAN}}
 
 
 def _src_hash(files):
@@ -85,13 +73,6 @@ def _src_hash(files):
         with open(os.path.join(ROOT, "paper_2401_14564_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
-
-
-def executed_ff_flops(energy, zpt=8):
-    t = EXECUTED["ff_energy" if energy else "ff_forces"]
-    if t["value"] is None or t["sha"] != _src_hash(t["files"]):
-        return None
-    return t["value"].get(int(zpt))
 
 
 def measured_issue(kernel):
@@ -511,8 +492,8 @@ def measure_quadrupole(case, tuning, steps, warmup, flush, alu_peak):
     return {"workload": "flake60 with tip quadrupole Qzz = -0.05 e*A^2", "ff_ms": ff_ms, "relax_ms": rx_ms,
             "ms_per_step": ff_ms + rx_ms, "pixel_z_per_s": s["nx"] * s["ny"] * s["nz"] / ((ff_ms + rx_ms) * 1e-3),
             "ff_pair_evals_per_s": pairs / (ff_ms * 1e-3), "ff_flops_per_pair": FLOPS_PER_PAIR_QUAD,
-            "ff_achieved_tflops": tflops, "ff_frac_of_alu_peak": tflops / alu_peak,
-            "ff_traffic": measured_traffic("ff_assemble_quad")}
+            "ff_direct_equivalent_tflops": tflops, "fp32_peak_tflops": alu_peak,
+            "ff_traffic": measured_traffic("ff_tile_quad")}
 
 
 def measure_tricubic(case, steps, warmup, flush, spacings=(0.1, 0.2)):
@@ -816,7 +797,7 @@ def measure_small(case, steps, warmup, flush, alu_peak, ff_energy=False, cpu=Tru
                        f"scan {s['nx']}x{s['ny']}x{s['nz']}",
            "ff_ms": ff_ms, "relax_ms": rx_ms, "ms_per_step": ff_ms + rx_ms,
            "ff_pair_evals_per_s": pairs / (ff_ms * 1e-3),
-           "ff_frac_of_alu_peak": pairs * flops_pair / (ff_ms * 1e-3) / 1e12 / alu_peak,
+           "ff_direct_equivalent_tflops": pairs * flops_pair / (ff_ms * 1e-3) / 1e12, "fp32_peak_tflops": alu_peak,
            "relax_pixel_z_per_s": units / (rx_ms * 1e-3), "pixel_z_per_s": units / ((ff_ms + rx_ms) * 1e-3),
            "fire_iters_mean": float(sim.iters.float().mean().item())}
     if cpu:
@@ -1145,18 +1126,18 @@ def main():
     alu_peak = fp32_peak_tflops(sm_max, sms)
     alu_src = f"{sms} SMs (read from the device) x 128 FP32 lanes x 2 x {sm_max:.0f} MHz ({src} max SM clock)"
     rx_gbs = it_total * BYTES_PER_FIRE_ITER / (rx_ms * 1e-3) / 1e9
-    ff_zpt = int(tuning["ff_zpt"]) if tuning is not None else 8
-    executed = executed_ff_flops(args.ff_energy, ff_zpt)
+    out_gbs = 16 * case["grid"]["nx"] * case["grid"]["ny"] * case["grid"]["nz"] / (ff_ms * 1e-3) / 1e9
     kernels = {
         "ff_assemble": {"ms": ff_ms, "share": ff_ms / (ff_ms + rx_ms), "pair_evals_per_s": pairs / (ff_ms * 1e-3),
                         "flops_per_pair": flops_pair, "energy": bool(args.ff_energy),
-                        "traffic": measured_traffic("ff_assemble", ff_zpt) if not args.ff_energy else None,
-                        "achieved_tflops": ff_tflops, "peak_tflops": alu_peak, "frac": ff_tflops / alu_peak,
-                        "executed_flops_per_pair": executed, "ff_zpt": ff_zpt,
-                        "executed_frac": (pairs * executed / (ff_ms * 1e-3) / 1e12 / alu_peak) if executed else None,
-                        "note": "frac counts the flops a direct sum over all node-atom pairs takes (the number the "
-                                ">= 50 % target is stated in); atoms far from a 16x16x16-node tile are summed at its "
-                                "8x8x8 interpolation points, so fewer are executed and frac can exceed 1"},
+                        "traffic": measured_traffic("ff_tile") if not args.ff_energy else None,
+                        "direct_equivalent_tflops": ff_tflops, "fp32_peak_tflops": alu_peak,
+                        "fp32_peak_source": alu_src, "output_gbs": out_gbs,
+                        "frac_of_hbm": out_gbs / peaks["hbm_gbs"],
+                        "note": "by tiles (ff_tile_kernel), on the FP32 pipes: atoms far from a 16x16x16-node tile are "
+                                "summed at its 8x8x8 interpolation points, so fewer operations are executed than the "
+                                "direct sum over all node-atom pairs takes; direct_equivalent_tflops counts that sum's "
+                                "and may exceed the peak (it is a throughput, no fraction of a roof)"},
         "relax_scan": {"ms": rx_ms, "share": rx_ms / (ff_ms + rx_ms), "pixel_z_per_s": units / (rx_ms * 1e-3),
                        "fire_iters_mean": it_total / units, "nonconverged_frac": nonconv,
                        "fire_iters_hist": {"bin_lower_edges": edges[:-1], "counts": it_hist},
@@ -1177,8 +1158,9 @@ def main():
     }
     dom = "ff_assemble" if ff_ms >= rx_ms else "relax_scan"
     if dom == "ff_assemble":
-        roof = {"kernel": "ff_tile", "bound": "alu", "achieved": ff_tflops, "peak": alu_peak, "unit": "TFLOP/s",
-                "frac": ff_tflops / alu_peak, "traffic": measured_traffic("ff_assemble", ff_zpt), "peak_source": alu_src}
+        roof = {"kernel": "ff_tile", "bound": "hbm", "achieved": out_gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s",
+                "frac": out_gbs / peaks["hbm_gbs"], "traffic": measured_traffic("ff_tile"), "peak_source": src,
+                "note": "the grid's bytes, written once; the FP32 pipes bound the kernel before"}
     else:
         roof = {"kernel": "relax_scan", "bound": "l2", "achieved": rx_gbs, "peak": l2["peak_gbs"], "unit": "GB/s",
                 "frac": rx_gbs / l2["peak_gbs"], "traffic": measured_traffic("relax_scan"),

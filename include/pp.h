@@ -205,8 +205,10 @@ PP_API pp_status pp_ff_combine(const float* ff, const float* ff_el, float Q, con
 
 /* Options of pp_make_ff_tuned.  ff_zpt (the launch shape, picked by the
  * autotuner) is the number of consecutive z-nodes each thread accumulates, 4,
- * 8 or 16; 0 = 8 (on grids of up to 0.35 A spacing, samples of 16 atoms and
- * more are summed by tiles of 16x16x16 nodes, whatever it says).  ff_forces_only = 1 skips the energy sums of an interp = 0
+ * 8 or 16; 0 = 8 (where the grid is summed directly: samples of fewer than
+ * 16 atoms, spacings above 0.35 A, and some samples of fewer than 36; others
+ * run by tiles of 16x16x16 nodes or, on periodic cells, in blocks of their
+ * own, whatever it says).  ff_forces_only = 1 skips the energy sums of an interp = 0
  * grid and writes 0 in every E slot: the scan reads only the forces (Sec.
  * 5.1.1 step 2), and the forces are bit for bit those of ff_forces_only = 0
  * (the default, E written). */

@@ -240,8 +240,9 @@ __global__ void __launch_bounds__(kTileThreads, 2) batch_ff_kernel(const BatchLa
             const int a = D.atom_offset;
             const TileJob J = {B.ax + a, B.ay + a, B.az + a, B.aR + a, B.aeps + a, B.aq + a, D.n_atoms,
                                D.x0, D.y0, D.z0, D.dx, D.dy, D.dz, D.nx, D.ny};
-            ff_tile<kMinImage, kCutoff, kQuad, false, kForcesOnly, 4, false>(J, cst, i0, j0, k0, 0, min(4, (D.nz - k0 + 3) >> 2), S,
-                                                                             store);
+            const int nz = D.nz;
+            ff_tile<kMinImage, kCutoff, kQuad, false, kForcesOnly, false>(J, cst, i0, j0, k0, S,
+                                                                          [&](int f, int) { return k0 + f < nz; }, store);
         } else {
             const int warp = threadIdx.x >> 5;
             for (int h = 0; h < 2; ++h)

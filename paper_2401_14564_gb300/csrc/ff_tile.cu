@@ -26,13 +26,12 @@ __global__ void __launch_bounds__(kTileThreads, 2) ff_tile_kernel(const FFLaunch
     const TileJob J = {P.x, P.y, P.z, P.R, P.eps, P.q, P.n, P.x0, P.y0, P.z0, P.dx, P.dy, P.dz, P.map.nx, P.map.ny};
     const FFConst c = ff_const(P.R_pp, P.eps_pp, P.kQ, P.core_frac, P.Lx, P.Ly, kCutoff ? P.coul_rc : 0.f,
                                kQuad ? P.kQzz : 0.f);
-    constexpr int kQuarters = 4 / kParts;
-    const int k0 = (P.kbeg / kTileN + (int)(blockIdx.z / kParts)) * kTileN, first = (int)(blockIdx.z % kParts) * kQuarters;
-    // this CTA's quarters that hold layers in [kbeg, kend)
-    const int q0 = max(first, (P.kbeg - k0) >> 2), q1 = min(first + kQuarters, (P.kend - k0 + 3) >> 2);
-    if (q0 >= q1) return;
-    ff_tile<kMinImage, kCutoff, kQuad, kEnergy, kForcesOnly, kQuarters, kThin>(
-        J, c, blockIdx.x * kTileN, blockIdx.y * kTileN, k0, q0, q1, S,
+    const int z = kParts == 2 ? blockIdx.z >> 1 : blockIdx.z, only = kParts == 2 ? blockIdx.z & 1 : -1;
+    const int k0 = (P.kbeg / kTileN + z) * kTileN;
+    if (kParts == 2 && (k0 + 8 * only >= P.kend || k0 + 8 * only + 8 <= P.kbeg)) return;
+    ff_tile<kMinImage, kCutoff, kQuad, kEnergy, kForcesOnly, kThin>(
+        J, c, blockIdx.x * kTileN, blockIdx.y * kTileN, k0, S,
+        [&](int f, int n) { return (kParts == 1 || f >> 3 == only) && k0 + f < P.kend && k0 + f + n > P.kbeg; },
         [&](int i, int j, int k, float2 fx, float2 fy, float2 fz, float2 en) {
             if (i >= P.map.nx || j >= P.map.ny) return;
             const int base_xy = axis_off(P.map.ax, i) + axis_off(P.map.ay, j);

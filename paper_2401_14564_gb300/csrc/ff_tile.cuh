@@ -176,16 +176,16 @@ __device__ __forceinline__ int tile_slot(bool keep, int* count, int* total) {
 }
 
 // Assembles the nodes of the tile at node (i0, j0, k0) (multiples of 16) and hands each thread's columns
-// to `store(i, j, k, fx, fy, fz, en)`: node pairs (k, k + 1) of column (i, j) as packed pairs, for the
-// tile's quarters [q0, q1) of 4 layers each and maybe others of the tile.  kMost: at most that many are asked for, 2
-// or 4; kThin: one or two anywhere get no more than they ask for, otherwise the unit is a half (the kernel that can do
-// both is 3 % slower on whole grids).  Every thread of the CTA calls.
+// to `store(i, j, k, fx, fy, fz, en)`: node pairs (k, k + 1) of column (i, j) as packed pairs, for the halves of the
+// tile that `want(first, count)` asks layers of (k0 + first .. k0 + first + count - 1), or with kThin, where one or two
+// quarters of four layers are asked for, for those (the kernel that can do both is 3 % slower on whole grids).  Every
+// thread of the CTA calls.
 // A thread owns a column of 16 nodes, so that an atom's lateral terms and the interpolation along y
 // are formed once for all of them (the two halves in turn, at fewer registers and three CTAs an SM: 0.142
 // against 0.135 ms on the 60-atom flake, 24.2 against 22.2 ms on the slab).
-template <bool kMinImage, bool kCutoff, bool kQuad, bool kEnergy, bool kForcesOnly, int kMost, bool kThin, class Store>
-__device__ __forceinline__ void ff_tile(const TileJob& J, const FFConst& c, int i0, int j0, int k0, int q0, int q1,
-                                        TileShared& S, Store&& store) {
+template <bool kMinImage, bool kCutoff, bool kQuad, bool kEnergy, bool kForcesOnly, bool kThin, class Want, class Store>
+__device__ __forceinline__ void ff_tile(const TileJob& J, const FFConst& c, int i0, int j0, int k0, TileShared& S,
+                                        Want&& want, Store&& store) {
     constexpr int P3 = kTileP * kTileP * kTileP;
     const int tid = threadIdx.x;
     const float2 cx = tile_centre(J.x0, i0, J.dx), cy = tile_centre(J.y0, j0, J.dy), cz = tile_centre(J.z0, k0, J.dz);
@@ -396,13 +396,16 @@ __device__ __forceinline__ void ff_tile(const TileJob& J, const FFConst& c, int 
     const std::integral_constant<int, 4> half_tile;
     const std::integral_constant<int, 2> quarter;
     if constexpr (kThin) {
-        if (kMost > 2 && q1 - q0 > 2) column(whole, 0);
+        int q0 = 0, q1 = 4;
+        while (q0 < 3 && !want(4 * q0, 4)) ++q0;
+        while (q1 > q0 + 1 && !want(4 * q1 - 4, 4)) --q1;
+        if (q1 - q0 > 2) column(whole, 0);
         else if (q1 - q0 == 2) column(half_tile, 4 * q0);
         else column(quarter, 4 * q0);
     } else {
-        if (kMost > 2 && q0 < 2 && q1 > 2) column(whole, 0);
-        else if (q0 < 2) column(half_tile, 0);
-        else column(half_tile, 8);
+        if (want(0, 8) && want(8, 8)) column(whole, 0);
+        else if (want(0, 8)) column(half_tile, 0);
+        else if (want(8, 8)) column(half_tile, 8);
     }
     __syncthreads();  // the shared buffers may be reused
 }

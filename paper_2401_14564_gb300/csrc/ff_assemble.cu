@@ -180,15 +180,15 @@ cudaError_t launch_centred_zpt(const FFLaunch& L, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// Whether the last 4 layers or fewer of a range are worth a launch of their own beside blocks of `zpt` layers: only
-// once the blocks exceed 8 to an SM (320-atom sheet on 136x327x34 nodes 485 us in one launch, 455 in two; 21 atoms on 56x81x46
-// 10 in one, 18 in two), and not for energies (468 atoms on 111x244x41 358 and 393).
-bool tail_apart(const FFLaunch& L, int zblocks) {
-    int dev = 0, sms = 152;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+// Whether the last r layers of a range, after blocks of `zpt`, are worth a narrower launch of their own.  It takes
+// a block's whole time if its blocks are too few to fill the GPU (200 take it as it is), and a launch's 5 us (1e7 node-atom
+// pairs) in any case: 320-atom sheet on 136x327x34 nodes, 369 blocks and 6e7 pairs spared, 485 us in one launch, 455 in two; 772
+// on 202x124x42 (208, 8e7) 782 and 750; 200 on 84x130x34 (102, 1e7) 110 and 119; 17 atoms on 131x159x53 21 and 27.  Not for
+// energies (468 atoms on 111x244x41 358 and 393).
+bool tail_apart(const FFLaunch& L, int zpt, int r) {
     const int64_t xy = (int64_t)((L.map.nx + kTileX - 1) / kTileX) * ((L.map.ny + kTileY - 1) / kTileY);
-    return L.map.interp != 1 && xy * zblocks > 8LL * sms;
+    const int64_t spared = r <= 4 ? zpt - 4 : r <= 8 ? zpt - 8 : 0;
+    return r > 0 && L.map.interp != 1 && xy >= 200 && xy * kThreads * spared * L.n > 10000000;
 }
 
 // Blocks of 8 layers at multiples of 8.
@@ -196,7 +196,7 @@ cudaError_t launch_centred(const FFLaunch& L, cudaStream_t s) {
     if ((L.kend - 1) / 4 == L.kbeg / 4) return launch_centred_zpt<4>(L, s);
     FFLaunch bulk = L, tail = L;
     const int r = (L.kend - 1) % 8 + 1;
-    if (r > 4 || L.kend - r <= L.kbeg || !tail_apart(L, (L.kend + 7) / 8 - L.kbeg / 8)) return launch_centred_zpt<8>(L, s);
+    if (L.kend - r <= L.kbeg || !tail_apart(L, 8, r)) return launch_centred_zpt<8>(L, s);
     bulk.kend = tail.kbeg = L.kend - r;
     const cudaError_t e = launch_centred_zpt<8>(bulk, s);
     return e != cudaSuccess ? e : launch_centred_zpt<4>(tail, s);
@@ -249,7 +249,7 @@ cudaError_t launch_ff_assemble(const FFLaunch& L, cudaStream_t s) {
     // multiple of zpt (nz = 200 at 16: 13 x 16 = 208, 4 % of the arithmetic); those r layers go to a
     // second launch of a narrower shape instead (each node's sums are the same in every shape).
     const int zpt = (L.zpt == 4 || L.zpt == 16) ? L.zpt : 8;
-    const int n = L.kend - L.kbeg, r = n <= 4 || tail_apart(L, (n + zpt - 1) / zpt) ? n % zpt : 0, bulk = n - r;
+    const int n = L.kend - L.kbeg, r = n <= 4 || tail_apart(L, zpt, n % zpt) ? n % zpt : 0, bulk = n - r;
     FFLaunch head = L, tail = L;
     head.kend = L.kbeg + bulk;
     tail.kbeg = L.kbeg + bulk;

@@ -438,22 +438,22 @@ __host__ __device__ inline float rule_sqrt(float a) {
 }
 
 // Estimate of the share of (node, atom) pairs at `reach` and more, for atoms spread over the cell Lx x Ly in a plane
-// 3 A below the grid (a molecule's depth and the grid's clearance): at height h those outside a disc of radius
-// sqrt(reach^2 - h^2), averaged over the grid's heights.
+// 3 A below the grid (a molecule's depth and the grid's clearance): at each of eight heights those outside a disc of
+// radius sqrt(reach^2 - h^2), of which a narrow cell holds a strip at most.
 __host__ __device__ inline float ff_far_share(float Lx, float Ly, float Lz, float reach) {
-    const float low = 3.f, high = rule_add(low, Lz), pi = 3.14159265f;
-    const float area = rule_mul(Lx, Ly), r2 = rule_mul(reach, reach);
-    const float in = rule_add(r2, -rule_mul(area, 1.f / pi));  // h^2 below which the disc covers the cell
-    const float h = in > 0.f ? rule_sqrt(in) : 0.f, h0 = h > low ? h : low, h1 = high < reach ? high : reach;
-    // heights out of reach of everything, times the area
-    float sum = rule_mul(area, high > reach ? rule_add(high, -(reach > low ? reach : low)) : 0.f);
-    if (h1 > h0) {
-        // integral of 1 - pi (reach^2 - h^2) / area from h0 to h1, times the area
-        const float lin = rule_mul(rule_add(area, -rule_mul(pi, r2)), rule_add(h1, -h0));
-        const float cub = rule_add(rule_mul(h1, rule_mul(h1, h1)), -rule_mul(h0, rule_mul(h0, h0)));
-        sum = rule_add(sum, rule_add(lin, rule_mul(pi / 3.f, cub)));
+    const float area = rule_mul(Lx, Ly), r2 = rule_mul(reach, reach), side = Lx < Ly ? Lx : Ly;
+    float sum = 0.f;
+    for (int i = 0; i < 8; ++i) {
+        const float h = rule_add(3.f, rule_mul((i + 0.5f) * 0.125f, Lz)), d2 = rule_add(r2, -rule_mul(h, h));
+        if (!(d2 > 0.f)) {
+            sum = rule_add(sum, 1.f);
+            continue;
+        }
+        const float disc = rule_mul(3.14159265f, d2), strip = rule_mul(2.f * rule_sqrt(d2), side);
+        const float in = disc < strip ? disc : strip;
+        if (in < area) sum = rule_add(sum, rule_add(1.f, -(in / area)));
     }
-    return sum / rule_mul(area, Lz);
+    return 0.125f * sum;
 }
 
 // kDirect: direct sums.  Few atoms: they cost less than a tile's classification and, where a tile has them,
@@ -461,12 +461,12 @@ __host__ __device__ inline float ff_far_share(float Lx, float Ly, float Lz, floa
 // 10 atoms 23 directly, where the call's own 20 us already show).  Coarse grids: beyond 0.35 A no atom nearer
 // than 26 A is far, and coordinates relative to the centre of a wide tile round worse than absolute ones.  And where a
 // tile would find little far, so that its classification, the float pairs of its coordinates and its coarser blocks
-// show: energies alone (whose direct sums are half as long) and fewer than 36 atoms, where the share of far pairs is
-// below 0.4.  Measured on either side of the line (K1 alone, us: direct sums / tiles):
-//   energies: 198 atoms on 61x111x53 nodes (0.2 A, share 0.04) 44 / 55; 86 on 177x56x79 (0.3 A, 0.33) 37 / 39; 493 on
-//   129x124x42 (0.1 A, 0.43) 193 / 94; 152 on 58x180x64 (0.1 A, 0.49) 78 / 49;
-//   32 atoms on 105x66x40 (0.1 A, 0.09) 20 / 23; 21 on 162x52x77 (0.2 A, 0.35) 18 / 21; 21 on 81x104x88 (0.15 A, 0.49)
-//   23 / 23; 30 on 64x208x98 (0.1 A, 0.71) 33 / 23; with more atoms 46 on 118x85x54 (0.1 A, 0.39) 29 / 25.
+// show: energies alone (whose direct sums are half as long) where the share of far pairs is below 0.4, and fewer than 36
+// atoms where it is below 0.6.  Measured on either side of the line (K1 alone, us: direct sums / tiles):
+//   energies: 198 atoms on 61x111x53 nodes (0.2 A, share 0.06) 44 / 55; 43 on 149x120x56 (0.2 A, 0.38) 23 / 27; 49 on
+//   86x154x46 (0.1 A, 0.43) 20 / 18; 493 on 129x124x42 (0.1 A, 0.43) 193 / 94; 84 on 61x219x60 (0.2 A, 0.51) 52 / 45;
+//   32 atoms on 105x66x40 (0.1 A, 0.10) 20 / 23; 21 on 162x52x77 (0.2 A, 0.48) 18 / 21; 31 on 132x213x46 (0.25 A, 0.53)
+//   31 / 32; 33 on 76x229x97 (0.2 A, 0.71) 47 / 35; with more atoms 46 on 118x85x54 (0.1 A) 29 / 25.
 // kCentred: direct sums with coordinates relative to the tile's centre, on periodic cells where that share is below 0.3 (energies 0.4)
 // (absolute coordinates / tiles / centred): 148 atoms on 71x215x73 (0.28 A, 0.00) 182 / 253 / 176; 184 on 106x340x85 (0.21 A,
 // 0.07) 430 / 513 / 415; 420 on 354x134x147 (0.29 A, 0.17) 2414 / 2578 / 2427; 380 on 124x386x153 (0.26 A, 0.31)
@@ -486,8 +486,8 @@ __host__ __device__ inline FFPath ff_path(int n, int nx, int ny, int nz, float d
     const float dmax = dx > dy ? (dx > dz ? dx : dz) : (dy > dz ? dy : dz);
     const float reach = rule_mul(5.f * (kTileN - 1), dmax);  // 10 half extents
     const float share = ff_far_share(rule_mul((float)nx, dx), rule_mul((float)ny, dy), rule_mul((float)nz, dz), reach);
-    if (share >= (min_image && !energy ? 0.3f : 0.4f)) return FFPath::kTiles;
-    return min_image ? FFPath::kCentred : FFPath::kDirect;
+    if (min_image) return share < (energy ? 0.4f : 0.3f) ? FFPath::kCentred : FFPath::kTiles;
+    return share < (energy ? 0.4f : 0.6f) ? FFPath::kDirect : FFPath::kTiles;
 }
 
 }  // namespace pp

@@ -28,22 +28,18 @@ namespace {
 constexpr int kBins = 2048;
 constexpr int kHdr = 8;
 
-// The block's largest v (>= 0), folded into *out.
-__device__ __forceinline__ void block_max(int v, int* out) {
-    __shared__ int most;
-    if (threadIdx.x == 0) most = 0;
-    __syncthreads();
+// The warp's largest v (>= 0), folded into *most (shared).
+__device__ __forceinline__ void warp_most(int v, int* most) {
     v = __reduce_max_sync(0xffffffffu, v);
-    if ((threadIdx.x & 31) == 0 && v > 0) atomicMax(&most, v);
-    __syncthreads();
-    if (threadIdx.x == 0 && most > 0) atomicMax(out, most);
+    if ((threadIdx.x & 31) == 0 && v > 0) atomicMax(most, v);
 }
 
 // Also clears the list (-1) and the mask for plan_select_kernel, which runs after it.
 __global__ void __launch_bounds__(256) plan_cost_kernel(const int* __restrict__ iters, int nz, int npix, int shift,
                                                         int* hdr, int* hist, int* cost, int* list, int nlist, unsigned* mask,
                                                         int nmask) {
-    __shared__ int sh[kBins];
+    __shared__ int sh[kBins], costliest;
+    if (threadIdx.x == 0) costliest = 0;
     for (int b = threadIdx.x; b < kBins; b += blockDim.x) sh[b] = 0;
     const int gt = blockIdx.x * blockDim.x + threadIdx.x, gs = gridDim.x * blockDim.x;
     for (int q = gt; q < nlist; q += gs) list[q] = -1;
@@ -58,8 +54,9 @@ __global__ void __launch_bounds__(256) plan_cost_kernel(const int* __restrict__ 
         most = max(most, ci);
         atomicAdd(&sh[min(ci >> shift, kBins - 1)], 1);
     }
-    block_max(most, hdr + 5);
+    warp_most(most, &costliest);
     __syncthreads();
+    if (threadIdx.x == 0 && costliest > 0) atomicMax(hdr + 5, costliest);
     for (int b = threadIdx.x; b < kBins; b += blockDim.x)
         if (sh[b]) atomicAdd(hist + b, sh[b]);
 }
@@ -109,8 +106,11 @@ __global__ void __launch_bounds__(1024) plan_threshold_kernel(int* hdr, const in
 
 __global__ void __launch_bounds__(256) plan_select_kernel(int* hdr, const int* __restrict__ cost, int npix, int shift,
                                                           int k, int* list, unsigned* mask) {
+    __shared__ int rest;  // the costliest column not listed
+    if (threadIdx.x == 0) rest = 0;
+    __syncthreads();
     const int t = hdr[1], above = hdr[2];
-    int most = 0;  // of the columns not listed
+    int most = 0;
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < npix; p += gridDim.x * blockDim.x) {
         const int c = cost[p], bin = min(c >> shift, kBins - 1);
         int slot = k;
@@ -123,7 +123,9 @@ __global__ void __launch_bounds__(256) plan_select_kernel(int* hdr, const int* _
             most = max(most, c);
         }
     }
-    block_max(most, hdr + 6);
+    warp_most(most, &rest);
+    __syncthreads();
+    if (threadIdx.x == 0 && rest > 0) atomicMax(hdr + 6, rest);
 }
 
 }  // namespace

@@ -39,7 +39,7 @@ def molecule(n, shape, d, interp=0):
 CASES = {"sheet_near": sheet((7, 5), (71, 93, 28)), "sheet_near_quad": sheet((7, 5), (71, 93, 23), Qzz=-0.05),
          "sheet_far": sheet((9, 6), (190, 201, 20)), "sheet_tail": sheet((14, 8), (142, 142, 60)),
          "energies_near": molecule(40, (55, 66, 60), 0.2, 1),
-         "energies_far": molecule(40, (180, 151, 37), 0.1, 1), "atoms_35": molecule(35, (71, 66, 43), 0.1), "atoms_35_far": molecule(35, (150, 141, 43), 0.1),
+         "energies_far": molecule(40, (180, 151, 37), 0.1, 1), "atoms_35": molecule(35, (71, 66, 43), 0.1), "atoms_35_far": molecule(35, (190, 171, 43), 0.1),
         
          "atoms_36": molecule(36, (71, 66, 43), 0.1), "atoms_15": molecule(15, (71, 66, 43), 0.1)}
 CASES = {k: case32(c) for k, c in CASES.items()}

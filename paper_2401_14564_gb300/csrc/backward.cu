@@ -660,10 +660,22 @@ __global__ void __launch_bounds__(kTileThreads, 2) ff_backward_tile_kernel(const
             atomicAdd(&P.gbar[checked((first_sum + q) * P.n + ia, P.map.stored_nodes, kChkGridWrite)].w, v[q]);
     };
 
-    // contracts the records first .. first + cnt - 1 with `pairs` pairs through contract(pair): whole rounds for every
-    // thread (the cutoff's warp votes), up to the next multiple of the threads a slot has.  A list that would leave a
+    int pairs = 256;   // the tile's points; of a near part, its layers' nodes with an adjoint
+    int padded = 256;  // pairs that may be read: from `pairs` on the first node with adjoint zero
+    float* const fxy = reinterpret_cast<float*>(nd);
+    float* const fzg = reinterpret_cast<float*>(nd + kBwdPairs);
+    float* const fgg = reinterpret_cast<float*>(nd + 2 * kBwdPairs);
+    auto pad_node = [&](int s) {
+        const int w = (s >> 1) * 4, l = s & 1;
+        fxy[w + l] = fxy[0];
+        fxy[w + 2 + l] = fxy[2];
+        fzg[w + l] = fzg[0];
+        fzg[w + 2 + l] = fgg[w + l] = fgg[w + 2 + l] = 0.f;
+    };
+    // contracts the records first .. first + cnt - 1 with all pairs through contract(pair): whole rounds for every
+    // thread (the cutoff's warp votes), padded to a multiple of the threads a slot has.  A list that would leave a
     // quarter of its slots or more idle goes in two or more, the larger power of two first.
-    auto contract_all = [&](int first, int cnt, int pairs, auto&& contract) {
+    auto contract_all = [&](int first, int cnt, auto&& contract) {
         while (cnt > 0) {
             slots = 1;
             while (slots < cnt) slots <<= 1;
@@ -671,6 +683,11 @@ __global__ void __launch_bounds__(kTileThreads, 2) ff_backward_tile_kernel(const
             if (slots >= 32 && 4 * cnt <= 3 * slots) n = slots = slots >> 1;
             take(first, n);
             const int rounds = (pairs + nsub - 1) / nsub;
+            if (rounds * nsub > padded) {  // (a near part; nobody reads these yet)
+                for (int s = 2 * padded + tid; s < 2 * rounds * nsub; s += kTileThreads) pad_node(s);
+                padded = rounds * nsub;
+                __syncthreads();
+            }
             for (int r = 0; r < rounds; ++r) contract(r * nsub + sub);
             flush();
             first += n;
@@ -678,11 +695,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) ff_backward_tile_kernel(const
         }
     };
 
-    int pairs = 256;  // the tile's points; of a near part, its layers' nodes with an adjoint
     if (!far_part) {
-        float* const fxy = reinterpret_cast<float*>(nd);
-        float* const fzg = reinterpret_cast<float*>(nd + kBwdPairs);
-        float* const fgg = reinterpret_cast<float*>(nd + 2 * kBwdPairs);
         if (tid == 0) S.nodes = 0;
         __syncthreads();
 #pragma unroll
@@ -705,15 +718,8 @@ __global__ void __launch_bounds__(kTileThreads, 2) ff_backward_tile_kernel(const
         }
         __syncthreads();
         const int cnt = S.nodes;  // (some: the part has an adjoint)
-        pairs = (cnt + 1) / 2;
-        // pad to a multiple of 256 pairs with the first node, adjoint zero
-        for (int s = cnt + tid; s < ((pairs + 255) & ~255) * 2; s += kTileThreads) {
-            const int w = (s >> 1) * 4, l = s & 1;
-            fxy[w + l] = fxy[0];
-            fxy[w + 2 + l] = fxy[2];
-            fzg[w + l] = fzg[0];
-            fzg[w + 2 + l] = fgg[w + l] = fgg[w + 2 + l] = 0.f;
-        }
+        padded = pairs = (cnt + 1) / 2;
+        if ((cnt & 1) && tid == 0) pad_node(cnt);
     }
     bool have_points = false;
     for (int base = 0; base < P.n; base += kTileChunk) {
@@ -756,11 +762,11 @@ __global__ void __launch_bounds__(kTileThreads, 2) ff_backward_tile_kernel(const
             have_points = true;
             if (far) stage(s_far);
             __syncthreads();
-            contract_all(0, n_in, pairs, [&](int p) {
+            contract_all(0, n_in, [&](int p) {
                 bwd_pair<false, kCutoff, kQuad, Smooth::kInside>(at, cst, pt[p], pt[256 + p], pt[512 + p], 0xffffffffu);
             });
             if (kCutoff)
-                contract_all(n_in, n_out, pairs, [&](int p) {
+                contract_all(n_in, n_out, [&](int p) {
                     bwd_pair<false, kCutoff, kQuad, Smooth::kBeyond>(at, cst, pt[p], pt[256 + p], pt[512 + p], 0xffffffffu);
                 });
             continue;
@@ -770,7 +776,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) ff_backward_tile_kernel(const
         if (n_near == 0) continue;
         if (live && !far) stage(s_near);
         __syncthreads();
-        contract_all(0, n_near, pairs, [&](int p) {
+        contract_all(0, n_near, [&](int p) {
             bwd_pair<kMinImage, kCutoff, kQuad, Smooth::kNo>(at, cst, nd[p], nd[kBwdPairs + p], nd[2 * kBwdPairs + p], 0xffffffffu);
         });
     }

@@ -462,13 +462,14 @@ __host__ __device__ inline float ff_far_share(float Lx, float Ly, float Lz, floa
 // than 26 A is far, and coordinates relative to the centre of a wide tile round worse than absolute ones.  And where a
 // tile would find little far, so that its classification, the float pairs of its coordinates and its coarser blocks
 // show: energies alone (whose direct sums are half as long) where the share of far pairs is below 0.4, and fewer than 36
-// atoms where it is below 0.6.  Measured on either side of the line (K1 alone, us: direct sums / tiles):
+// atoms where it is below 0.3.  Measured on either side of the line (K1 alone, us: direct sums / tiles):
 //   energies: 198 atoms on 61x111x53 nodes (0.2 A, share 0.06) 44 / 55; 43 on 149x120x56 (0.2 A, 0.38) 23 / 27; 49 on
 //   86x154x46 (0.1 A, 0.43) 20 / 18; 493 on 129x124x42 (0.1 A, 0.43) 193 / 94; 84 on 61x219x60 (0.2 A, 0.51) 52 / 45;
-//   32 atoms on 105x66x40 (0.1 A, 0.10) 20 / 23; 21 on 162x52x77 (0.2 A, 0.48) 18 / 21; 31 on 132x213x46 (0.25 A, 0.53)
-//   31 / 32; 33 on 76x229x97 (0.2 A, 0.71) 47 / 35; with more atoms 46 on 118x85x54 (0.1 A) 29 / 25.
-// kCentred: direct sums with coordinates relative to the tile's centre, on periodic cells where that share is below 0.3 (energies 0.4)
-// (absolute coordinates / tiles / centred): 148 atoms on 71x215x73 (0.28 A, 0.00) 182 / 253 / 176; 184 on 106x340x85 (0.21 A,
+//   32 atoms on 105x66x40 (0.1 A, 0.10) 20 / 23; 28 on 105x65x69 (0.2 A, 0.24) 16 / 20; 33 on 76x229x97 (0.2 A, 0.71) 47 / 35;
+//   with more atoms 46 on 118x85x54 (0.1 A) 29 / 25.  (Between 0.3 and 0.6 few atoms' direct sums are up to 15 % faster alone,
+//   but the batch, which must write the same bits by 16-node tiles, loses 2 to 5 %: 4 molecules at 84 px 756 -> 798.)
+// kCentred: direct sums with coordinates relative to the tile's centre, on periodic cells where that share is below 0.3
+// (energies 0.4; absolute coordinates / tiles / centred): 148 atoms on 71x215x73 (0.28 A, 0.00) 182 / 253 / 176; 184 on 106x340x85 (0.21 A,
 // 0.07) 430 / 513 / 415; 420 on 354x134x147 (0.29 A, 0.17) 2414 / 2578 / 2427; 380 on 124x386x153 (0.26 A, 0.31)
 // 1740 / 1632 / 1754; 172 on 146x193x53 (0.15 A, 0.37) 213 / 222 / 199; 228 on 281x111x196 (0.23 A, 0.44) 1090 / 897 / 1113.
 // Their coordinates round once, which keeps most of what the tiles gain in accuracy there (relative 2-norm of the error
@@ -486,8 +487,8 @@ __host__ __device__ inline FFPath ff_path(int n, int nx, int ny, int nz, float d
     const float dmax = dx > dy ? (dx > dz ? dx : dz) : (dy > dz ? dy : dz);
     const float reach = rule_mul(5.f * (kTileN - 1), dmax);  // 10 half extents
     const float share = ff_far_share(rule_mul((float)nx, dx), rule_mul((float)ny, dy), rule_mul((float)nz, dz), reach);
-    if (min_image) return share < (energy ? 0.4f : 0.3f) ? FFPath::kCentred : FFPath::kTiles;
-    return share < (energy ? 0.4f : 0.6f) ? FFPath::kDirect : FFPath::kTiles;
+    if (share >= (energy ? 0.4f : 0.3f)) return FFPath::kTiles;
+    return min_image ? FFPath::kCentred : FFPath::kDirect;
 }
 
 }  // namespace pp

@@ -44,12 +44,12 @@ _SCAN = ["relax_scan.cu", "relax_core.cuh", "interp.cuh"]
 _DIRECT = ["ff_assemble.cu", "ff_core.cuh", "interp.cuh"]
 _TILES = ["ff_tile.cu", "ff_tile.cuh", "ff_core.cuh", "interp.cuh"]
 TRAFFIC = {
-    "relax_scan": {"bytes": 62.63e6, "sha": "ba93cc0bc5a90b25", "files": _SCAN},
-    "relax_scan_tricubic": {"bytes": 19.52e6, "sha": "ba93cc0bc5a90b25", "files": _SCAN},
-    "ff_tile": {"bytes": 146.99e6, "sha": "50c912b0f6642464", "files": _TILES},
-    "ff_tile_quad": {"bytes": 145.57e6, "sha": "50c912b0f6642464", "files": _TILES},
-    "ff_assemble_split": {"bytes": 354.83e6, "sha": "8d62392aedade281", "files": _DIRECT},
-    "ff_combine": {"bytes": 584.55e6, "sha": "8d62392aedade281", "files": _DIRECT},
+    "relax_scan": {"bytes": 62.71e6, "sha": "ba93cc0bc5a90b25", "files": _SCAN},
+    "relax_scan_tricubic": {"bytes": 19.69e6, "sha": "ba93cc0bc5a90b25", "files": _SCAN},
+    "ff_tile": {"bytes": 146.67e6, "sha": "b180fb8e04f175ce", "files": _TILES},
+    "ff_tile_quad": {"bytes": 145.31e6, "sha": "b180fb8e04f175ce", "files": _TILES},
+    "ff_assemble_split": {"bytes": 354.93e6, "sha": "ab682838d104c9e6", "files": _DIRECT},
+    "ff_combine": {"bytes": 584.62e6, "sha": "ab682838d104c9e6", "files": _DIRECT},
 }
 
 
